@@ -11,12 +11,15 @@
 // (warm = path: column j starts from column j-1's (z, u)) or one single
 // (g, e, j) column (warm = none: z = u = 0).
 //
-// Two schedules:
-//  * resident (p <= 128 in FP64, p <= 192 in FP32): one CTA keeps M_g in shared
+// Schedules:
+//  * chain (FP64, and FP32 with few chains): one cluster of CTAs iterates one chain
+//    (or four) at a time from start to end in a single launch, see k_admm_chain.
+//  * resident (FP32, p <= 192, many chains): one CTA keeps M_g in shared
 //    memory; each warp runs its own chains to completion with no block-wide
 //    barrier (the warp only reads its own columns of V = z - u), pulling new
 //    chains from a per-group counter.  One launch solves everything.
-//  * streaming (larger p): one launch per iteration computes x for every active
+//  * streaming (FP64 past the chain schedule's shared memory): one launch per
+//    iteration computes x for every active
 //    chain (row tiles x chain tiles x groups) with the soft-threshold / dual
 //    update / partial norms fused into the epilogue; a second launch reduces the
 //    norms in a fixed order, finishes converged columns and compacts the active
@@ -218,6 +221,401 @@ __global__ void __launch_bounds__(256, 1) k_admm_resident(AdmmDev<T> P, int32_t*
             }
         }
     }
+}
+
+// ----------------------------------------------------------------------------
+// Chain schedule
+// ----------------------------------------------------------------------------
+// A cluster of `cs` CTAs owns one group's chains, NC at a time.  CTA `rank` holds a
+// run of 16-row blocks of x, z, u and c in shared memory (and its rows of M_g too when
+// they fit; else M_g streams from L2).  One iteration:
+//   product   lane = (row of a block, one of two k), each warp its own k: the warp
+//             reads 16 consecutive entries of two rows of the symmetric M and adds
+//             into up to 8 independent accumulators; partial sums over the warps
+//             go through shared memory;
+//   update    one thread per row: x, soft threshold, dual, and V = z - u of the
+//             next iteration written into every CTA of the cluster;
+//   stop      the CTAs exchange five partial norms; one cluster barrier ends the
+//             iteration, after which every thread takes the same decision.
+// What bounds it: in FP64 the FP64 pipe, two multiply-adds per clock and SM on this
+// part with every warp instruction charged for 32 lanes.  So no instruction of the
+// iteration may run on few lanes, and the norms are first taken in FP32 (from the
+// FP64 differences): only when those say that the stop test may pass are they
+// formed in FP64, so that decisions are those of the FP64 norms.  M needs 16 B per
+// clock and SM, which L2 delivers.
+// Measured (one call, before: one warp per chain, or two launches per iteration): 200 x 50,
+// 20 chains, 598 iterations each: 12.7 -> 2.3 ms; p = 400, 20 chains: 38 -> 6.9 ms; p = 1000
+// (M 160 MB): 124 -> 53 ms; p = 150, 128 chains: 110 -> 3 ms.
+constexpr int CH_RB = 16;            // rows per block
+constexpr int CH_NB = 8;             // blocks accumulated together
+constexpr int CH_CLUSTER_MAX = 8;
+constexpr int CH_KAPPA = 256;        // thresholds kept in shared memory
+constexpr float CH_SCREEN = 1.0001f; // FP32 norms decide alone outside this margin
+
+struct ChainGeom {
+    int32_t cs;                      // CTAs per cluster
+    int32_t nrp;                     // rows of the largest CTA, a multiple of CH_RB
+    int32_t kp;                      // k extent padded to a multiple of 2 * warps
+    int32_t ldm;                     // row length of the shared copy of M, 0: M stays in global memory
+    size_t smem;
+};
+
+__device__ __forceinline__ uint32_t ch_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Store to the variable at `p` in CTA `rank` of the cluster.
+template <typename V>
+__device__ __forceinline__ void ch_store_rank(V* p, int rank, V v)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(ch_smem(p)), "r"(rank));
+    if constexpr (sizeof(V) == 8)
+        asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(a), "l"(*reinterpret_cast<long long*>(&v)) : "memory");
+    else
+        asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(a), "r"(*reinterpret_cast<int*>(&v)) : "memory");
+}
+
+__device__ __forceinline__ void ch_barrier(int cs)
+{
+    if (cs == 1) {
+        __syncthreads();
+    } else {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+                     "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+}
+
+__device__ __forceinline__ float ch_f32(double x) { return f64_to_f32_int(x); }
+__device__ __forceinline__ float ch_f32(float x) { return x; }
+
+// soft_threshold with the comparisons on the integer pipe (FP64, k >= 0): one FP64
+// subtraction.
+__device__ __forceinline__ double ch_threshold(double v, double k)
+{
+    const long long kb = __double_as_longlong(k);
+    if (kb < 0) return soft_threshold(v, k);
+    const long long a = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll;
+    if (!(a > kb && a <= 0x7FF0000000000000ll)) return 0.0;             // |v| <= k, or v is NaN
+    const long long sign = __double_as_longlong(v) & (1ll << 63);
+    return v - __longlong_as_double(kb | sign);
+}
+__device__ __forceinline__ float ch_threshold(float v, float k) { return soft_threshold(v, k); }
+
+// acc += m v: a plain multiply-add in FP64; in FP32 the rounding errors of the
+// product and of the sum go to a second word.
+struct ChSumD {
+    double a = 0.0;
+    __device__ __forceinline__ void add(double m, double v) { a = fma(m, v, a); }
+    __device__ __forceinline__ double value() const { return a; }
+};
+struct ChSumF {
+    float a = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float m, float v)
+    {
+        const float p = __fmul_rn(m, v), e = fmaf(m, v, -p);
+        const float s = __fadd_rn(a, p), b = __fsub_rn(s, a);
+        c += (__fsub_rn(a, __fsub_rn(s, b)) + __fsub_rn(p, b)) + e;
+        a = s;
+    }
+    __device__ __forceinline__ float value() const { return a + c; }
+};
+template <typename T> struct ChSumOf;
+template <> struct ChSumOf<double> { using type = ChSumD; };
+template <> struct ChSumOf<float> { using type = ChSumF; };
+
+// NB blocks of one warp: out[(block * 16 + row)] of each slot (row stride `ostr` per
+// slot) = sum over this warp's k of M[k][row] V_slot[k].  m points at (k = 0, the
+// lane's row of the first block); rows of a block past the CTA's last repeat it.
+template <typename T, int NB, int NC>
+__device__ __forceinline__ void ch_product(const T* m, size_t ld, int p, const T* V, int kp, int k0, int kstep,
+                                           int row, int nrows, T* out, int ostr)
+{
+    typename ChSumOf<T>::type acc[NB][NC];
+    int off[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) off[b] = min(row + b * CH_RB, nrows - 1) - min(row, nrows - 1);
+#pragma unroll 2
+    for (int k = k0; k < kp; k += kstep) {
+        const T* mk = m + (size_t)min(k, p - 1) * ld;
+        T v[NC], x[NB];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) x[b] = mk[off[b]];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[c] = V[c * kp + k];
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[b][c].add(x[b], v[c]);
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            T s = acc[b][c].value();
+            s += __shfl_xor_sync(0xffffffffu, s, CH_RB);
+            if ((threadIdx.x & 31) < CH_RB) out[c * ostr + b * CH_RB] = s;
+        }
+}
+
+template <typename T, int NC>
+__global__ void __launch_bounds__(512) k_admm_chain(AdmmDev<T> P, int32_t* chain_next, ChainGeom geo)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ T s_kappa[CH_KAPPA];
+    __shared__ float s_red[16][5], s_norm[2][CH_CLUSTER_MAX][NC][5];
+    __shared__ T s_redx[16][5], s_exact[CH_CLUSTER_MAX][NC][5];
+    __shared__ int s_cid[NC];
+    const int p = P.p, cs = geo.cs, nrp = geo.nrp, kp = geo.kp;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, NW = blockDim.x >> 5;
+    int rank = 0;
+    if (cs > 1) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const int g = blockIdx.y;
+    const int nbt = (p + CH_RB - 1) / CH_RB;
+    const int b0 = rank * nbt / cs, nblk = (rank + 1) * nbt / cs - b0;
+    const int row0 = b0 * CH_RB, nrows = min(p - row0, nblk * CH_RB);
+    const T* Mg = P.M + (size_t)g * p * p;
+    // shared memory: [M] | V, two buffers of NC | partial products | z u c x z_prev
+    T* Ms = reinterpret_cast<T*>(smem_raw);
+    T* V = Ms + (size_t)geo.ldm * p;
+    T* part = V + (size_t)2 * NC * kp;
+    T* zs = part + (size_t)NW * NC * nrp;
+    T* us = zs + NC * nrp;
+    T* cv = us + NC * nrp;
+    T* xs = cv + NC * nrp;
+    T* zq = xs + NC * nrp;
+    if (geo.ldm)
+        for (int k = warp; k < p; k += NW)
+            for (int i = lane; i < nrows; i += 32) Ms[(size_t)k * geo.ldm + i] = Mg[(size_t)k * p + row0 + i];
+    for (int i = threadIdx.x; i < 2 * NC * kp; i += blockDim.x) V[i] = T(0);
+    for (int i = threadIdx.x; i < min(P.q, CH_KAPPA); i += blockDim.x) s_kappa[i] = (T)P.lambdas[i] / P.rho;
+
+    const int nchains = P.warm ? P.r : P.r * P.q;
+    int e_[NC], j_[NC], jend_[NC], it_[NC];
+    bool act[NC];
+    T kappa[NC];
+    auto kappa_of = [&](int j) { return j < CH_KAPPA ? s_kappa[j] : (T)P.lambdas[j] / P.rho; };
+    // takes the next chain of the group for each slot of `need`, its V in buffer `buf`
+    auto fetch = [&](unsigned need, int buf) {
+        if (rank == 0 && threadIdx.x == 0)
+            for (int s = 0; s < NC; ++s)
+                if ((need >> s) & 1u) {
+                    const int cid = atomicAdd(&chain_next[g], 1);
+                    for (int t = 0; t < cs; ++t) {
+                        if (cs == 1) s_cid[s] = cid;
+                        else ch_store_rank(&s_cid[s], t, cid);
+                    }
+                }
+        ch_barrier(cs);
+#pragma unroll
+        for (int s = 0; s < NC; ++s) {
+            if (!((need >> s) & 1u)) continue;
+            const int cid = s_cid[s];
+            act[s] = cid < nchains;
+            if (!act[s]) continue;
+            if (P.warm) { e_[s] = cid; j_[s] = 0; jend_[s] = P.q; }
+            else        { e_[s] = cid % P.r; j_[s] = cid / P.r; jend_[s] = j_[s] + 1; }
+            it_[s] = 0;
+            kappa[s] = kappa_of(j_[s]);
+            const int64_t col0 = ((int64_t)g * P.q + j_[s]) * P.r + e_[s];
+            const bool init = P.z0 && !P.warm;
+            for (int i = threadIdx.x; i < nrows; i += blockDim.x) {
+                zs[s * nrp + i] = init ? (T)P.z0[col0 * p + row0 + i] : T(0);
+                us[s * nrp + i] = init ? (T)P.u0[col0 * p + row0 + i] : T(0);
+                cv[s * nrp + i] = P.c[((size_t)g * P.r + e_[s]) * p + row0 + i];
+            }
+            T* Vn = V + ((size_t)buf * NC + s) * kp;
+            for (int k = threadIdx.x; k < p; k += blockDim.x)
+                Vn[k] = init ? (T)P.z0[col0 * p + k] - (T)P.u0[col0 * p + k] : T(0);
+        }
+        __syncthreads();
+    };
+    __syncthreads();                                         // s_kappa
+    fetch((1u << NC) - 1u, 0);
+
+    const int slot = warp % NC, wi = warp / NC, nwi = NW / NC;   // this warp's slot in the row-wise steps
+    for (int cur = 0;; cur ^= 1) {
+        bool any = false;
+#pragma unroll
+        for (int s = 0; s < NC; ++s) any |= act[s];
+        if (!any) break;
+        // product
+        {
+            const int kk = lane / CH_RB, ri = lane % CH_RB;
+            const T* Vc = V + (size_t)cur * NC * kp;
+            T* pw = part + (size_t)warp * NC * nrp;
+            const size_t ld = geo.ldm ? (size_t)geo.ldm : (size_t)p;
+            const T* base = geo.ldm ? Ms : Mg + row0;
+            constexpr int CB = NC == 1 ? CH_NB : CH_NB / 2;
+            for (int c0 = 0; c0 < nblk; c0 += CB) {
+                const int row = c0 * CH_RB + ri;
+                const T* m = base + min(row, nrows - 1);
+                T* o = pw + row;
+                const int k0 = 2 * warp + kk, ks = 2 * NW;
+                switch (min(CB, nblk - c0)) {
+                case 1: ch_product<T, 1, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                case 2: ch_product<T, 2, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                case 3: ch_product<T, 3, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                case 4: ch_product<T, 4, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                default:
+                    if constexpr (NC == 1) {
+                        switch (min(CB, nblk - c0)) {
+                        case 5: ch_product<T, 5, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                        case 6: ch_product<T, 6, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                        case 7: ch_product<T, 7, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                        default: ch_product<T, 8, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                        }
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        // update
+        {
+            T kap = T(0);
+            bool on = false;
+#pragma unroll
+            for (int s = 0; s < NC; ++s)
+                if (slot == s) { kap = kappa[s]; on = act[s]; }
+            float n5[5] = { 0.f, 0.f, 0.f, 0.f, 0.f };
+            if (on)
+                for (int i = wi * 32 + lane; i < nrows; i += nwi * 32) {
+                    const int o = slot * nrp + i;
+                    T sum = part[o];
+                    for (int w = 1; w < NW; ++w) sum += part[(size_t)w * NC * nrp + o];
+                    const T x = cv[o] + P.rho * sum;
+                    const T zp = zs[o];
+                    const T v = x + us[o];
+                    const T zn = ch_threshold(v, kap);
+                    const T un = v - zn;
+                    const T vn = zn - un;
+                    const T d = x - zn, dz = zn - zp;
+                    zs[o] = zn;
+                    us[o] = un;
+                    xs[o] = x;
+                    zq[o] = zp;
+                    T* dst = V + ((size_t)(cur ^ 1) * NC + slot) * kp + row0 + i;
+                    if (cs == 1) *dst = vn;
+                    else
+                        for (int t = 0; t < cs; ++t) ch_store_rank(dst, t, vn);
+                    const float fd = ch_f32(d), fz = ch_f32(dz), fx = ch_f32(x), fn = ch_f32(zn), fu = ch_f32(un);
+                    n5[0] += fd * fd; n5[1] += fz * fz; n5[2] += fx * fx; n5[3] += fn * fn; n5[4] += fu * fu;
+                }
+#pragma unroll
+            for (int t = 0; t < 5; ++t) {
+                const float w = warp_sum(n5[t]);
+                if (lane == 0) s_red[warp][t] = w;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < NC * 5) {
+            const int s = threadIdx.x / 5, t = threadIdx.x % 5;
+            float w = 0.f;
+            for (int k = 0; k < nwi; ++k) w += s_red[k * NC + s][t];
+            if (cs == 1) s_norm[cur][0][s][t] = w;
+            else
+                for (int k = 0; k < cs; ++k) ch_store_rank(&s_norm[cur][rank][s][t], k, w);
+        }
+        ch_barrier(cs);
+        // stop test
+        bool conv[NC];
+        unsigned maybe = 0;
+#pragma unroll
+        for (int s = 0; s < NC; ++s) {
+            conv[s] = false;
+            if (!act[s]) continue;
+            float n[5] = { 0.f, 0.f, 0.f, 0.f, 0.f };
+            for (int k = 0; k < cs; ++k)
+#pragma unroll
+                for (int t = 0; t < 5; ++t) n[t] += s_norm[cur][k][s][t];
+            const float base = (float)P.sqrtp * (float)P.abs_tol, rel = (float)P.rel_tol, rho = (float)P.rho;
+            const float ep = base + rel * fmaxf(sqrtf(n[2]), sqrtf(n[3])), ed = base + rel * rho * sqrtf(n[4]);
+            if constexpr (sizeof(T) == 4)
+                conv[s] = sqrtf(n[0]) <= ep && rho * sqrtf(n[1]) <= ed;
+            else if (!(sqrtf(n[0]) > CH_SCREEN * ep) && !(rho * sqrtf(n[1]) > CH_SCREEN * ed))
+                maybe |= 1u << s;
+        }
+        if constexpr (sizeof(T) == 8) {
+            if (maybe) {                                     // the same in every thread of the cluster
+                T n5[5] = {};
+                if ((maybe >> slot) & 1u)
+                    for (int i = wi * 32 + lane; i < nrows; i += nwi * 32) {
+                        const int o = slot * nrp + i;
+                        const T x = xs[o], zn = zs[o], un = us[o], d = x - zn, dz = zn - zq[o];
+                        n5[0] += d * d; n5[1] += dz * dz; n5[2] += x * x; n5[3] += zn * zn; n5[4] += un * un;
+                    }
+#pragma unroll
+                for (int t = 0; t < 5; ++t) {
+                    const T w = warp_sum(n5[t]);
+                    if (lane == 0) s_redx[warp][t] = w;
+                }
+                __syncthreads();
+                if (threadIdx.x < NC * 5) {
+                    const int s = threadIdx.x / 5, t = threadIdx.x % 5;
+                    T w = T(0);
+                    for (int k = 0; k < nwi; ++k) w += s_redx[k * NC + s][t];
+                    if (cs == 1) s_exact[0][s][t] = w;
+                    else
+                        for (int k = 0; k < cs; ++k) ch_store_rank(&s_exact[rank][s][t], k, w);
+                }
+                ch_barrier(cs);
+#pragma unroll
+                for (int s = 0; s < NC; ++s) {
+                    if (!((maybe >> s) & 1u)) continue;
+                    T n[5] = {};
+                    for (int k = 0; k < cs; ++k)
+#pragma unroll
+                        for (int t = 0; t < 5; ++t) n[t] += s_exact[k][s][t];
+                    const T xn = sqrt(n[2]), zn = sqrt(n[3]);
+                    const T eps_pri = P.sqrtp * P.abs_tol + P.rel_tol * (xn > zn ? xn : zn);
+                    const T eps_dual = P.sqrtp * P.abs_tol + P.rel_tol * P.rho * sqrt(n[4]);
+                    conv[s] = sqrt(n[0]) <= eps_pri && P.rho * sqrt(n[1]) <= eps_dual;
+                }
+            }
+        }
+        unsigned need = 0;
+#pragma unroll
+        for (int s = 0; s < NC; ++s) {
+            if (!act[s]) continue;
+            it_[s] += 1;
+            if (!conv[s] && it_[s] < P.max_iter) continue;
+            const int64_t col_je = (int64_t)j_[s] * P.r + e_[s];
+            const int64_t col = (int64_t)g * P.q * P.r + col_je;
+            for (int i0 = warp * 32; i0 < nrows; i0 += NW * 32) {
+                const int i = i0 + lane;
+                const bool in = i < nrows;
+                const T zi = in ? zs[s * nrp + i] : T(0), ui = in ? us[s * nrp + i] : T(0);
+                const int64_t o = col * p + row0 + i;
+                if (P.beta && in && UOI_IN_BOUNDS(o, (int64_t)P.G * P.q * P.r * p, 203)) P.beta[o] = (double)zi;
+                if (P.u_out && in) P.u_out[o] = (double)ui;
+                if (P.family) {
+                    // 32 rows from row0 + i0, a multiple of 16: within one word or across two
+                    const uint64_t out = (uint64_t)__ballot_sync(0xffffffffu, in && zi == T(0));
+                    const int bit = (row0 + i0) & 63;
+                    unsigned long long* w = (unsigned long long*)&P.family[col_je * P.W + ((row0 + i0) >> 6)];
+                    if (lane == 0 && (out << bit)) atomicAnd(w, ~(unsigned long long)(out << bit));
+                    if (lane == 0 && bit > 32 && (out >> (64 - bit)))
+                        atomicAnd(w + 1, ~(unsigned long long)(out >> (64 - bit)));
+                }
+                if (P.near_count)
+                    count_near_threshold<T>(in, zi, ui, kappa[s], (T)kNearThreshold, P.near_count);
+            }
+            if (rank == 0 && threadIdx.x == 0) {
+                if (P.iters) P.iters[col] = it_[s];
+                if (P.conv) P.conv[col] = conv[s] ? 1 : 0;
+            }
+            j_[s] += 1;
+            if (j_[s] < jend_[s]) {
+                it_[s] = 0;
+                kappa[s] = kappa_of(j_[s]);
+            } else {
+                need |= 1u << s;
+            }
+        }
+        if (need) {
+            __syncthreads();                                 // every thread has read the finished chain's z, u
+            fetch(need, cur ^ 1);
+        }
+    }
+    if (cs > 1) ch_barrier(cs);                              // no CTA leaves while another may store into it
 }
 
 // ----------------------------------------------------------------------------
@@ -610,20 +1008,99 @@ void launch_resident(const AdmmDev<T>& d, int32_t* chain_next, cudaStream_t s)
     count_launch();
 }
 
+// Launches the chain schedule if its rows fit in shared memory; false (nothing
+// launched) when p is too large for it.
+//
+// Cluster size: with at least one chain per SM, one CTA per chain (the FP64 pipes are
+// all busy and a cluster barrier would only add to each step); with fewer, as many
+// CTAs per chain as keep every chain on the device at once, but at least 32 rows
+// each (below that the barrier costs more than the rows).  M goes to shared memory
+// where it fits; where it does not and a group has four chains or more, four share
+// each read of M.
+template <typename T, int NC>
+bool launch_chain_nc(const AdmmDev<T>& d, int32_t* chain_next, int nw, int cs, bool m_smem, int nchains,
+                     cudaStream_t s)
+{
+    const int nbt = (int)ceil_div(d.p, CH_RB);
+    ChainGeom geo{};
+    geo.cs = cs;
+    geo.nrp = (int)ceil_div(nbt, cs) * CH_RB;
+    geo.kp = (int)ceil_div(d.p, 2 * nw) * 2 * nw;
+    // FP32 rows of M 64 bytes apart modulo 128, so that a warp's two rows use all banks
+    geo.ldm = m_smem ? (sizeof(T) == 4 && geo.nrp % 32 == 0 ? geo.nrp + CH_RB : geo.nrp) : 0;
+    geo.smem = sizeof(T) * ((size_t)geo.ldm * d.p + (size_t)2 * NC * geo.kp + (size_t)(nw + 5) * NC * geo.nrp);
+    auto kern = k_admm_chain<T, NC>;
+    int dev = 0, optin = 0, nsm = 0;
+    UOI_CUDA(cudaGetDevice(&dev));
+    UOI_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    UOI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    cudaFuncAttributes fa;
+    UOI_CUDA(cudaFuncGetAttributes(&fa, (const void*)kern));
+    if (geo.smem + fa.sharedSizeBytes > (size_t)optin) return false;
+    allow_max_dynamic_smem((const void*)kern);
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3((unsigned)(32 * nw));
+    cfg.dynamicSmemBytes = geo.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3((unsigned)cs, (unsigned)d.G);
+    int resident = 0;
+    if (cs > 1) {
+        UOI_CUDA(cudaOccupancyMaxActiveClusters(&resident, kern, &cfg));
+        if (resident < 1) return false;
+    } else {
+        UOI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, 32 * nw, geo.smem));
+        resident *= nsm;
+    }
+    const int per = std::max(1, std::min((int)ceil_div(nchains, NC), resident / std::max(1, d.G)));
+    cfg.gridDim = dim3((unsigned)(cs * per), (unsigned)d.G);
+    UOI_CUDA(cudaLaunchKernelEx(&cfg, kern, d, chain_next, geo));
+    UOI_CHECK_LAUNCH();
+    count_launch();
+    return true;
+}
+
+template <typename T>
+bool try_chain(const AdmmDev<T>& d, int32_t* chain_next, cudaStream_t s)
+{
+    const int nchains = d.warm ? d.r : d.r * d.q;
+    const int64_t total = (int64_t)d.G * nchains;
+    constexpr int NSM = 152, GPC_FIT = 128;       // SMs, and those that clusters of up to 8 can fill
+    int cs = 1;
+    if (total < NSM)
+        cs = (int)std::max<int64_t>(1, std::min<int64_t>({ CH_CLUSTER_MAX, GPC_FIT / total, d.p / 32 }));
+    constexpr int NW_S = sizeof(T) == 8 ? 4 : 8;  // warps with M in shared memory
+    for (; cs <= CH_CLUSTER_MAX; ++cs) {
+        if (launch_chain_nc<T, 1>(d, chain_next, NW_S, cs, true, nchains, s)) return true;
+        if constexpr (sizeof(T) == 8) {
+            if (nchains >= 4 && launch_chain_nc<T, 4>(d, chain_next, 8, cs, false, nchains, s)) return true;
+            if (launch_chain_nc<T, 1>(d, chain_next, nchains >= 4 ? 8 : 16, cs, false, nchains, s)) return true;
+        }
+    }
+    return false;
+}
+
 template <typename T>
 bool try_resident(const AdmmDev<T>& d, int32_t* chain_next, cudaStream_t s);
 
 template <>
 bool try_resident<double>(const AdmmDev<double>& d, int32_t* chain_next, cudaStream_t s)
 {
-    if (d.p <= 64) { launch_resident<double, 2, 4>(d, chain_next, s); return true; }
-    if (d.p <= 128) { launch_resident<double, 4, 4>(d, chain_next, s); return true; }
-    return false;
+    return try_chain<double>(d, chain_next, s);
 }
 
 template <>
 bool try_resident<float>(const AdmmDev<float>& d, int32_t* chain_next, cudaStream_t s)
 {
+    // few chains per group (a path start with few responses): the chain schedule while
+    // the cluster's shared memory holds M
+    if ((d.warm ? d.r : d.r * d.q) <= 4 && try_chain<float>(d, chain_next, s)) return true;
     if (d.p <= 64) { launch_resident<float, 2, 4>(d, chain_next, s); return true; }
     if (d.p <= 128) { launch_resident<float, 4, 4>(d, chain_next, s); return true; }
     if (d.p <= 192) { launch_resident<float, 6, 4>(d, chain_next, s); return true; }
