@@ -304,7 +304,7 @@ void moments(int precision, const double* X, int64_t ldx, const double* Y, int64
     if (precision == UOI_PREC_MIXED && gram_tc_available())
         moments_tc(X, ldx, Y, ldy, m, p, r, w, mask, B, G, Bm, s, X32, lower_only);
     else
-        moments_fp64(X, ldx, Y, ldy, m, p, r, w, mask, B, G, Bm, 0, s);
+        moments_f64(X, ldx, Y, ldy, m, p, r, w, mask, B, G, Bm, 0, s);
 }
 
 template <typename T>
@@ -560,7 +560,7 @@ int fit_core(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t
         if (r <= 4)
             xty_small(Xd, ldx, Yd, ldy, m, p, r, xty.as<double>(), s);
         else
-            moments_fp64(Xd, ldx, Yd, ldy, m, p, r, nullptr, nullptr, 1, nullptr, xty.as<double>(), 1, s);
+            moments_f64(Xd, ldx, Yd, ldy, m, p, r, nullptr, nullptr, 1, nullptr, xty.as<double>(), 1, s);
         lambda_grid(xty.as<double>(), p * r, m, q, prm->lambda_min_ratio, lam.as<double>(), s);
     }
 
@@ -1151,7 +1151,7 @@ int uoi_ws_dataset(const double* X, const double* Y, int64_t n, int64_t p, int64
         const int64_t rows = (int64_t)B * q * r * p;
         DevBuf G(sizeof(double) * (size_t)(B * p * p), s), Bm(sizeof(double) * (size_t)(B * p * r), s);
         DevBuf nk(sizeof(double) * B, s), A(sizeof(double) * (size_t)(B * p * p), s);
-        moments_fp64(Xd, p, Yd, r, n, p, r, wd, nullptr, B, G.as<double>(), Bm.as<double>(), 0, s);
+        moments_f64(Xd, p, Yd, r, n, p, r, wd, nullptr, B, G.as<double>(), Bm.as<double>(), 0, s);
         weight_sums(wd, nullptr, n, B, nk.as<double>(), s);
         DevBuf st(sizeof(DevStatus), s);
         UOI_CUDA(cudaMemsetAsync(st.ptr, 0, st.bytes, s));

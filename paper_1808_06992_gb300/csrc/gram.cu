@@ -3,7 +3,8 @@
 // For bootstrap k the LASSO of Eq. 2 on T^k only needs G_k = X^T W_k X and
 // B_k = X^T W_k Y (W_k = diag of the bootstrap multiplicities): the ADMM
 // x-update of Eq. 5 then never touches the n rows again.  This is the plain
-// FP64 form; the tensor-core form lives in gram_tc.cu.
+// FP64 form on the CUDA cores, for callers that cannot allocate and inputs that the
+// tensor-core form (gram_f64tc.cu) does not take; the mixed form lives in gram_tc.cu.
 #include <algorithm>
 
 #include "kernels.h"
@@ -317,7 +318,7 @@ void moments_fp64_cols(const double* X, int64_t ldx, const double* Y, int64_t ld
         X, ldx, m, cols, nu, Xu.as<double>());
     UOI_CHECK_LAUNCH();
     DevBuf Gu(sizeof(double) * (size_t)(B * nu * nu), s), Bu(sizeof(double) * (size_t)(B * nu * r), s);
-    moments_fp64(Xu.as<double>(), nu, Y, ldy, m, nu, r, w, mask, B, Gu.as<double>(), Bu.as<double>(), 0, s);
+    moments_f64(Xu.as<double>(), nu, Y, ldy, m, nu, r, w, mask, B, Gu.as<double>(), Bu.as<double>(), 0, s);
     const int64_t total = (nu * nu + nu * r) * B;
     k_scatter_moments<<<(unsigned)std::min<int64_t>(ceil_div(total, 256), 152 * 32), 256, 0, s>>>(
         Gu.as<double>(), Bu.as<double>(), nu, r, B, cols, p_out, G, Bm);

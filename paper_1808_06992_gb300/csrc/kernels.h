@@ -97,7 +97,12 @@ void weight_sums(const uint32_t* w, const uint8_t* mask, int64_t m, int32_t B, d
 void moments_fp64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t m,
                   int64_t p, int64_t r, const uint32_t* w, const uint8_t* mask, int32_t B,
                   double* G, double* Bm, int b_only, cudaStream_t s);
-// moments_fp64 restricted to the nu X columns listed in cols, written into the
+// The same moments in FP64 accuracy on the tensor cores (gram_f64tc.cu), where they can
+// be used: else moments_fp64.  Allocates from the pool and waits for the stream.
+void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t m, int64_t p, int64_t r,
+                 const uint32_t* w, const uint8_t* mask, int32_t B, double* G, double* Bm, int b_only,
+                 cudaStream_t s);
+// moments_f64 restricted to the nu X columns listed in cols, written into the
 // p_out x p_out / p_out x r outputs at the original feature indices (other
 // entries untouched).
 void moments_fp64_cols(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t m, int64_t p_out,
