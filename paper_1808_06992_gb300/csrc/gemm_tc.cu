@@ -114,7 +114,7 @@ k_gemm3_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0 && elect_one()) {
         // ---------------- TMA producer ----------------
         const int blkA = ((g * a.MT + mt) * a.kst) * GT_PIECES;
         const int blkB = ((g * a.NT + nt) * a.kst) * GT_PIECES;
@@ -133,7 +133,7 @@ k_gemm3_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUte
         if (abort_flag)
             for (int s_ = max(0, a.kst - GT_STAGES); s_ < a.kst; ++s_)
                 mbar_wait(&full_bar[s_ % GT_STAGES], (s_ / GT_STAGES) & 1, &abort_flag, a.wait_ns);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         // ---------------- MMA issuer: all three products into accumulator b ----------------
         const uint32_t idesc = idesc_f16(GT_TM, GT_TN);
         int s_ = 0;

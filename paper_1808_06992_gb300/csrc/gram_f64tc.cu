@@ -26,8 +26,8 @@
 // instruction); 28 bf16 products replace one FP64 product at 4096 per clock.  Tiles are
 // 128 x 64 because the 7 accumulators of a tile (448 of 512 TMEM columns) cap N.
 // Measured against the CUDA-core form (k_moments_fp64, selection moments of 20
-// bootstraps): 20000 x 1000 414 -> 19.4 ms, 5000 x 400 26.0 -> 1.7 ms, 200 x 50 0.23 ->
-// 0.14 ms; X^T Y of 192 responses x 5000 rows (the lambda grid of a VAR) 5.9 -> 0.3 ms.
+// bootstraps): 20000 x 1000 414 -> 10.9 ms, 5000 x 400 26.0 -> 1.05 ms, 200 x 50 0.23 ->
+// 0.13 ms; X^T Y of 192 responses x 5000 rows (the lambda grid of a VAR) 5.9 -> 0.3 ms.
 // No size was found where the CUDA-core form is the faster one.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -136,7 +136,7 @@ k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0 && elect_one()) {
         for (int g = 0; g < nst; ++g) {
             const int s = g % OZ_STAGES;
             if (g >= OZ_STAGES && !mbar_wait(&empty_bar[s], ((g / OZ_STAGES) - 1) & 1, &abort_flag, a.wait_ns)) {
@@ -153,7 +153,7 @@ k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         if (abort_flag)
             for (int g = max(0, nst - OZ_STAGES); g < nst; ++g)
                 mbar_wait(&full_bar[g % OZ_STAGES], (g / OZ_STAGES) & 1, &abort_flag, a.wait_ns);
-    } else if (warp == 1 && lane == 0 && nc > 0) {
+    } else if (warp == 1 && nc > 0 && elect_one()) {
         constexpr uint32_t idesc = idesc_bf16(OZ_TM, OZ_TN);
         int g = 0;
         for (int c = 0; c < nc && !abort_flag; ++c) {

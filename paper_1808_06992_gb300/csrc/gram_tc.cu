@@ -118,7 +118,7 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmA, GramTcArgs a)
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0 && kstages > 0) {
+    if (warp == 0 && kstages > 0 && elect_one()) {
         // ---------------- TMA producer (both CTAs) ----------------
         const int zA = item * 2;
         const int jb = tj * TN + rank * (TN / 2);    // this CTA's half of the column tile
@@ -143,7 +143,7 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmA, GramTcArgs a)
             for (int g = max(0, kstages - STAGES); g < kstages; ++g)
                 mbar_wait(&full_bar[g % STAGES], (g / STAGES) & 1, &abort_flag, a.wait_ns);
         }
-    } else if (warp == 1 && lane == 0 && kstages > 0 && rank == 0) {
+    } else if (warp == 1 && kstages > 0 && rank == 0 && elect_one()) {
         // ---------------- MMA issuer (first CTA, for the pair) ----------------
         constexpr uint32_t idesc = idesc_bf16(2 * TM, TN);
         int g = 0;
@@ -186,7 +186,7 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmA, GramTcArgs a)
         mma_commit_pair(&done_bar);                 // every MMA issued above has completed
         int dummy = 0;
         mbar_wait(&done_bar, 0, &dummy, a.wait_ns);
-    } else if (warp == 1 && lane == 0 && kstages > 0) {
+    } else if (warp == 1 && kstages > 0 && rank != 0 && elect_one()) {
         // second CTA: its TMEM is written by the first CTA's MMAs until this arrives
         int dummy = 0;
         mbar_wait(&done_bar, 0, &dummy, a.wait_ns);

@@ -97,7 +97,7 @@ k_mlp_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0 && nst > 0) {
+    if (warp == 0 && nst > 0 && elect_one()) {
         // ---------------- TMA producer ----------------
         for (int i = 0; i < nst; ++i) {
             const int s = i % MT_STAGES;
@@ -117,7 +117,7 @@ k_mlp_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             for (int i = max(0, nst - MT_STAGES); i < nst; ++i)
                 mbar_wait(&full_bar[i % MT_STAGES], (i / MT_STAGES) & 1, &abort_flag, a.wait_ns);
         }
-    } else if (warp == 1 && lane == 0 && nst > 0) {
+    } else if (warp == 1 && nst > 0 && elect_one()) {
         // ---------------- MMA issuer ----------------
         constexpr uint32_t idesc = idesc_bf16(MT_TM, MT_TN);
         for (int i = 0; i < nst; ++i) {

@@ -163,7 +163,7 @@ __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUten
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0 && elect_one()) {
         // ---------------- TMA producer ----------------
         const int blkA = ((g * a.RT + rt) * a.kst) * XT_PIECES;   // first 8 KB block of this row tile
         const int rowB = g * a.nchains + n0;
@@ -184,7 +184,7 @@ __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUten
         if (abort_flag)
             for (int s_ = max(0, a.kst - nst); s_ < a.kst; ++s_)
                 mbar_wait(&full_bar[s_ % nst], (s_ / nst) & 1, &abort_flag, a.wait_ns);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         // ---------------- MMA issuer ----------------
         const uint32_t idesc = idesc_f16(XT_TM, a.NT);
         const uint32_t d2 = tmem + 128u;
