@@ -1115,6 +1115,8 @@ void admm_solve(const AdmmProblem<T>& P, cudaStream_t s)
     if (P.G <= 0 || P.p <= 0 || P.r <= 0 || P.q <= 0) return;
     AdmmDev<T> d = to_dev(P);
     const int32_t nchains = P.warm ? (int32_t)P.r : (int32_t)(P.r * P.q);
+    if constexpr (sizeof(T) == 4)
+        if (nchains > 4 && admm_solve_wide(P, s)) return;
     {
         DevBuf next(sizeof(int32_t) * P.G, s);
         UOI_CUDA(cudaMemsetAsync(next.ptr, 0, next.bytes, s));

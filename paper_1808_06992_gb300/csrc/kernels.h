@@ -217,6 +217,9 @@ void admm_solve(const AdmmProblem<T>& P, cudaStream_t s);
 // Streaming schedule with the tensor-core x-update (FP32 state, p > resident limit).
 bool admm_tc_available();
 void admm_solve_tc(const AdmmProblem<float>& P, cudaStream_t s);
+// The whole solve in one launch for many chains and p <= 512 (admm_wide.cu); false
+// (nothing launched) where it does not apply.
+bool admm_solve_wide(const AdmmProblem<float>& P, cudaStream_t s);
 // Grouped solve of a batch of problems.  Each batch worker thread enters the batch
 // before a fit and leaves it after; the fit's first tensor-core ADMM solve
 // (admm_solve<float> past the resident schedule) joins the batch instead of
