@@ -60,15 +60,136 @@ __global__ void k_sum_slices(const float* part, int slices, int64_t count, float
     }
 }
 
-// column sums of an N x C matrix in a fixed order: dst[c] = sum_n A[n*C + c]
-template <typename TA>
-__global__ void k_col_sums(const TA* A, int64_t N, int C, float* dst)
+// Sums over the rows of a batch, one FP32 chain per output in row order (row n + 1 is added
+// to the sum of the rows before it): for the K columns of the row vectors w (N x K)
+//   dst[c * sc + k * sk] = sum_n A[n][c] w[n][k],  and  sums[c] = sum_n A[n][c] (nullable),
+// from A's transpose At (512 x ldt BF16, rows past N zero).  A block takes 32 columns and one
+// k (blockIdx.y; K = the plain sums), 128 rows at a time: warps 1-3 copy 256-byte runs of
+// the columns to shared memory, three steps ahead of warp 0, which only adds (lane =
+// column; copying and adding in one warp took 13-17 clocks per row).
+// What bounds it: the chain of dependent additions (the order of the sums is part of the
+// result: any other moves it by 7e-5 at 65536 rows).  10 clocks per row now, 0.33-0.36 ms at
+// 65536 rows; one thread per column reading row by row waited for memory at every row
+// (22 ms for K = 8).  A whole gradient of 65536 rows went from 46 to 2.3 ms.
+constexpr int SUM_ROWS = 128;
+constexpr int SUM_LD = SUM_ROWS / 8 + 1;            // 16-byte vectors per column, one of padding
+constexpr int SUM_STAGES = 4;
+
+__device__ __forceinline__ void sum_copy16(void* dst, const void* src, bool in)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(in ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void sum_copy4(void* dst, const void* src, bool in)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(in ? 4 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void sum_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void sum_wait()          // the oldest step in flight has landed
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(SUM_STAGES - 2) : "memory");
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(128)
+k_row_sums(const __nv_bfloat16* __restrict__ At, int64_t ldt, const float* __restrict__ w, int K, int64_t N,
+           float* dst, int sc, int sk, float* sums)
+{
+    __shared__ __align__(16) uint4 tile[SUM_STAGES][32 * SUM_LD];
+    __shared__ __align__(16) float sw[SUM_STAGES][SUM_ROWS];
+    const int lane = threadIdx.x & 31, k = blockIdx.y, c0 = blockIdx.x * 32;
+    const bool plain = k == K, adds = threadIdx.x < 32;
+    const int ht = threadIdx.x - 32;                 // 96 copying threads: vector ht % 16 of columns ht / 16 + 6 i
+    const int v = ht & 15, cl = ht >> 4;
+    auto load = [&](int st, int64_t n0) {
+        if (!adds) {
+            const bool in = n0 + 8 * v < ldt;
+            const __nv_bfloat16* src = At + (int64_t)(c0 + cl) * ldt + n0 + 8 * v;
+#pragma unroll
+            for (int i = 0; i < 6; ++i)
+                if (cl + 6 * i < 32) sum_copy16(&tile[st][(cl + 6 * i) * SUM_LD + v], in ? src + 6 * i * ldt : At, in);
+            if (!plain)
+                for (int t = ht; t < SUM_ROWS; t += 96)
+                    sum_copy4(&sw[st][t], n0 + t < N ? w + (n0 + t) * K + k : w, n0 + t < N);
+        }
+        sum_commit();
+    };
     float s = 0.f;
-    for (int64_t n = 0; n < N; ++n) s += (float)A[n * C + c];
-    dst[c] = s;
+    for (int st = 0; st < SUM_STAGES - 1; ++st) load(st, (int64_t)st * SUM_ROWS);
+    int st = 0;
+    for (int64_t n0 = 0; n0 < N; n0 += SUM_ROWS) {
+        sum_wait();
+        load(st == 0 ? SUM_STAGES - 1 : st - 1, n0 + (SUM_STAGES - 1) * SUM_ROWS);   // the slot added last
+        if (adds) {
+            // every vector of the step is read before the chain goes on, and w one vector ahead:
+            // nothing but the additions waits for the one before
+            uint4 x[SUM_ROWS / 8];
+#pragma unroll
+            for (int i = 0; i < SUM_ROWS / 8; ++i) x[i] = tile[st][lane * SUM_LD + i];
+            const float4* wp = reinterpret_cast<const float4*>(sw[st]);
+            float4 wn[2] = { wp[0], wp[1] };
+#pragma unroll
+            for (int i = 0; i < SUM_ROWS / 8; ++i) {
+                const uint32_t p[4] = { x[i].x, x[i].y, x[i].z, x[i].w };
+                float d[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) d[t] = __uint_as_float(t & 1 ? p[t / 2] & 0xFFFF0000u : p[t / 2] << 16);
+                if (plain) {
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) s += d[t];
+                } else {
+                    const float wr[8] = { wn[0].x, wn[0].y, wn[0].z, wn[0].w, wn[1].x, wn[1].y, wn[1].z, wn[1].w };
+                    if (i + 1 < SUM_ROWS / 8) {
+                        wn[0] = wp[2 * i + 2];
+                        wn[1] = wp[2 * i + 3];
+                    }
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) s = fmaf(d[t], wr[t], s);
+                }
+            }
+        }
+        st = st == SUM_STAGES - 1 ? 0 : st + 1;
+    }
+    if (!adds) return;
+    const int c = c0 + lane;
+    if (plain) sums[c] = s;
+    else dst[(int64_t)c * sc + (int64_t)k * sk] = s;
+}
+
+// g[j] = sum_n dout[n][j] in row order, one warp per output (every lane keeps the sum).
+__global__ void __launch_bounds__(32) k_head_bias(const float* __restrict__ dout, int64_t N, float* g)
+{
+    constexpr int ROWS = 512;
+    __shared__ __align__(16) float sv[SUM_STAGES][ROWS];
+    const int j = blockIdx.x, lane = threadIdx.x;
+    auto load = [&](int st, int64_t n0) {
+#pragma unroll
+        for (int u = 0; u < ROWS / 32; ++u) {
+            const int64_t n = n0 + 32 * u + lane;
+            sum_copy4(&sv[st][32 * u + lane], n < N ? dout + n * WS_OUT + j : dout, n < N);
+        }
+        sum_commit();
+    };
+    float s = 0.f;
+    for (int st = 0; st < SUM_STAGES - 1; ++st) load(st, (int64_t)st * ROWS);
+    int st = 0;
+    for (int64_t n0 = 0; n0 < N; n0 += ROWS) {
+        sum_wait();
+        load(st == 0 ? SUM_STAGES - 1 : st - 1, n0 + (SUM_STAGES - 1) * ROWS);
+#pragma unroll 8
+        for (int i = 0; i < ROWS / 4; ++i) {
+            const float4 x = *reinterpret_cast<const float4*>(&sv[st][4 * i]);
+            s += x.x;
+            s += x.y;
+            s += x.z;
+            s += x.w;
+        }
+        st = st == SUM_STAGES - 1 ? 0 : st + 1;
+    }
+    if (lane == 0) g[j] = s;
 }
 
 // layer 1 (K = 8): a1 = X W1^T + b1, h1 = gelu(a1) stored in BF16 (and transposed,
@@ -99,6 +220,7 @@ k_layer_in(const float* X, int64_t N, const __nv_bfloat16* w, const float* maste
 #pragma unroll 2
         for (int v = 0; v < LIN_GROUP; v += 8) {
             uint32_t packed[4];
+            float pr[8];
 #pragma unroll
             for (int u = 0; u < 8; u += 2) {
                 float r2[2];
@@ -108,12 +230,17 @@ k_layer_in(const float* X, int64_t N, const __nv_bfloat16* w, const float* maste
                     float acc = sb[o];
 #pragma unroll
                     for (int k = 0; k < WS_IN; ++k) acc = fmaf(xv[k], sw[o * WS_IN + k], acc);
-                    if (pre) pre[n * WS_H + o] = acc;
+                    pr[u + h2] = acc;
                     r2[h2] = gelu_f(acc);
                     if (ht) ht[(int64_t)o * ldt + n] = __float2bfloat16_rn(r2[h2]);
                 }
                 const __nv_bfloat162 hb = __floats2bfloat162_rn(r2[0], r2[1]);
                 packed[u / 2] = *reinterpret_cast<const uint32_t*>(&hb);
+            }
+            if (pre) {                                   // a lane's 8 outputs: one whole sector
+                float4* pd = reinterpret_cast<float4*>(pre + n * WS_H + o0 + v);
+                pd[0] = make_float4(pr[0], pr[1], pr[2], pr[3]);
+                pd[1] = make_float4(pr[4], pr[5], pr[6], pr[7]);
             }
             *reinterpret_cast<uint4*>(h + n * WS_H + o0 + v) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
         }
@@ -182,53 +309,53 @@ __global__ void k_loss_grad(const float* out, const float* T, int64_t N, float* 
     if (threadIdx.x == 0) loss_part[blockIdx.x] = red[0];
 }
 
-// da3 = (dOut W4) * gelu'(a3), stored in BF16 and transposed (da3t[k * ldt + n])
-__global__ void k_head_back(const float* dout, int64_t N, const __nv_bfloat16* w, const float* pre3,
-                            __nv_bfloat16* da3, __nv_bfloat16* da3t, int64_t ldt)
+// da3 = (dOut W4) * gelu'(a3), stored in BF16 and transposed (da3t[k * ldt + n]): tiles of
+// 64 rows x 64 features, the transpose turned over in shared memory so that both are
+// written in 128-byte runs.  256 threads.
+__global__ void __launch_bounds__(256)
+k_head_back(const float* dout, int64_t N, const __nv_bfloat16* w, const float* pre3, __nv_bfloat16* da3,
+            __nv_bfloat16* da3t, int64_t ldt)
 {
-    const int64_t total = N * WS_H;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t n = t / WS_H;
-        const int k = (int)(t % WS_H);
-        float s = 0.f;
+    __shared__ __nv_bfloat16 tile[64][66];
+    const int64_t n0 = (int64_t)blockIdx.x * 64;
+    const int k0 = blockIdx.y * 64, c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+    const int k = k0 + 2 * c;
+    float w4[WS_OUT][2];
 #pragma unroll
-        for (int j = 0; j < WS_OUT; ++j)
-            s = fmaf(dout[n * 3 + j], __bfloat162float(w[OFF_W4 + j * WS_H + k]), s);
-        const __nv_bfloat16 d = __float2bfloat16_rn(s * gelu_grad_f(pre3[t]));
-        da3[t] = d;
-        da3t[(int64_t)k * ldt + n] = d;
+    for (int j = 0; j < WS_OUT; ++j)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) w4[j][u] = __bfloat162float(w[OFF_W4 + j * WS_H + k + u]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = r0 + 8 * i;
+        const int64_t n = n0 + r;
+        __nv_bfloat162 d = __floats2bfloat162_rn(0.f, 0.f);
+        if (n < N) {
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int j = 0; j < WS_OUT; ++j) {
+                const float g = __ldg(dout + n * 3 + j);
+                s0 = fmaf(g, w4[j][0], s0);
+                s1 = fmaf(g, w4[j][1], s1);
+            }
+            const float2 p = *reinterpret_cast<const float2*>(pre3 + n * WS_H + k);
+            d = __floats2bfloat162_rn(s0 * gelu_grad_f(p.x), s1 * gelu_grad_f(p.y));
+            *reinterpret_cast<__nv_bfloat162*>(da3 + n * WS_H + k) = d;
+        }
+        tile[r][2 * c] = d.x;
+        tile[r][2 * c + 1] = d.y;
     }
-}
-
-// gradient of W1 (K over rows, 8 inputs): g[o][k] = sum_n da1[n][o] X[n][k]
-__global__ void k_grad_w1(const __nv_bfloat16* da1, const float* X, int64_t N, float* g)
-{
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= WS_H) return;
-    float s[WS_IN] = {};
-    for (int64_t n = 0; n < N; ++n) {
-        const float d = __bfloat162float(da1[n * WS_H + o]);
+    __syncthreads();
+    // feature rows of the transpose: a warp writes 64 sample rows of one feature at a time
 #pragma unroll
-        for (int k = 0; k < WS_IN; ++k) s[k] = fmaf(d, X[n * WS_IN + k], s[k]);
+    for (int i = 0; i < 8; ++i) {
+        const int f = r0 + 8 * i;
+        __nv_bfloat16* o = da3t + (int64_t)(k0 + f) * ldt + n0 + 2 * c;
+        if (n0 + 2 * c + 1 < N)
+            *reinterpret_cast<__nv_bfloat162*>(o) = __halves2bfloat162(tile[2 * c][f], tile[2 * c + 1][f]);
+        else if (n0 + 2 * c < N)
+            *o = tile[2 * c][f];
     }
-#pragma unroll
-    for (int k = 0; k < WS_IN; ++k) g[OFF_W1 + o * WS_IN + k] = s[k];
-}
-
-// gradient of W4: g[j][k] = sum_n dout[n][j] h3[n][k]
-__global__ void k_grad_w4(const float* dout, const __nv_bfloat16* h3, int64_t N, float* g)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= WS_H) return;
-    float s[WS_OUT] = {};
-    for (int64_t n = 0; n < N; ++n) {
-        const float hv = __bfloat162float(h3[n * WS_H + k]);
-#pragma unroll
-        for (int j = 0; j < WS_OUT; ++j) s[j] = fmaf(dout[n * 3 + j], hv, s[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < WS_OUT; ++j) g[OFF_W4 + j * WS_H + k] = s[j];
 }
 
 __global__ void k_transpose_bf16(const __nv_bfloat16* src, __nv_bfloat16* dst, int rows, int cols)
@@ -319,7 +446,7 @@ unsigned blocks_for(int64_t work) { return (unsigned)std::min<int64_t>(ceil_div(
 struct Acts {
     DevBuf a1, a2, a3;        // FP32 pre-activations (training)
     DevBuf h1, h2, h3;        // BF16 hidden activations, N x 512
-    DevBuf h1t, h2t;          // BF16 512 x ldt transposes (training: the weight gradients' B)
+    DevBuf h1t, h2t, h3t;     // BF16 512 x ldt transposes (training: the weight gradients' operands)
     DevBuf head;              // inference: the head's partial sums, HEAD_SLOTS x N x 3
     DevBuf out;
     int64_t ldt = 0;
@@ -346,9 +473,10 @@ void forward(WsModel* M, const float* X, int64_t N, Acts& A, bool train, int32_t
     if (train) {
         A.a1.alloc(hsz, s); A.a2.alloc(hsz, s); A.a3.alloc(hsz, s);
         const size_t tb = sizeof(__nv_bfloat16) * (size_t)WS_H * A.ldt;
-        A.h1t.alloc(tb, s); A.h2t.alloc(tb, s);
+        A.h1t.alloc(tb, s); A.h2t.alloc(tb, s); A.h3t.alloc(tb, s);
         UOI_CUDA(cudaMemsetAsync(A.h1t.ptr, 0, tb, s));      // padding rows of the K extent
         UOI_CUDA(cudaMemsetAsync(A.h2t.ptr, 0, tb, s));
+        UOI_CUDA(cudaMemsetAsync(A.h3t.ptr, 0, tb, s));
     }
     A.h1.alloc(hb, s); A.h2.alloc(hb, s);
     if (train) A.h3.alloc(hb, s);
@@ -371,7 +499,7 @@ void forward(WsModel* M, const float* X, int64_t N, Acts& A, bool train, int32_t
         return;
     }
     mlp_forward_tc(A.h2.as<__nv_bfloat16>(), N, M->w + OFF_W3, WS_H, M->master + OFF_B3,
-                   train ? A.a3.as<float>() : nullptr, A.h3.as<__nv_bfloat16>(), nullptr, 0, err, s);
+                   A.a3.as<float>(), A.h3.as<__nv_bfloat16>(), A.h3t.as<__nv_bfloat16>(), A.ldt, err, s);
     k_head<<<(unsigned)ceil_div(N * 32, 256), 256, 0, s>>>(A.h3.as<__nv_bfloat16>(), N, M->w, M->master,
                                                            A.out.as<float>());
     UOI_CHECK_LAUNCH();
@@ -393,6 +521,38 @@ void grad_square(const __nv_bfloat16* dAt, const __nv_bfloat16* Ht, int64_t ldt,
     count_launch();
 }
 
+// Work on the calling thread's second stream beside s: after() gives that stream, ordered
+// after everything s has queued so far; join() makes s wait for it (the destructor does
+// so too, before buffers of s that the work reads are given back).
+struct SideWork {
+    cudaStream_t s, q;
+    cudaEvent_t ev = nullptr;
+    bool open = false;
+    explicit SideWork(cudaStream_t st) : s(st), q(side_stream())
+    {
+        UOI_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    }
+    cudaStream_t after()
+    {
+        UOI_CUDA(cudaEventRecord(ev, s));
+        UOI_CUDA(cudaStreamWaitEvent(q, ev, 0));
+        open = true;
+        return q;
+    }
+    void join()
+    {
+        if (!open) return;
+        open = false;
+        UOI_CUDA(cudaEventRecord(ev, q));
+        UOI_CUDA(cudaStreamWaitEvent(s, ev, 0));
+    }
+    ~SideWork()
+    {
+        if (open && cudaEventRecord(ev, q) == cudaSuccess) cudaStreamWaitEvent(s, ev, 0);
+        if (ev) cudaEventDestroy(ev);
+    }
+};
+
 // Full gradient into g (N_PARAMS floats); returns the mean loss.
 double loss_grad(WsModel* M, const float* X, const float* T, int64_t N, float* g, cudaStream_t s)
 {
@@ -407,34 +567,41 @@ double loss_grad(WsModel* M, const float* X, const float* T, int64_t N, float* g
     UOI_CHECK_LAUNCH();
     const size_t hb = sizeof(__nv_bfloat16) * (size_t)N * WS_H;
     const size_t tb = sizeof(__nv_bfloat16) * (size_t)WS_H * A.ldt;
-    DevBuf da3(hb, s), da2(hb, s), da3t(tb, s), da2t(tb, s);
+    DevBuf da3(hb, s), da2(hb, s), da3t(tb, s), da2t(tb, s), da1t(tb, s);
+    UOI_CUDA(cudaMemsetAsync(da1t.ptr, 0, tb, s));
     UOI_CUDA(cudaMemsetAsync(da3t.ptr, 0, tb, s));
     UOI_CUDA(cudaMemsetAsync(da2t.ptr, 0, tb, s));
-    k_grad_w4<<<WS_H / 128, 128, 0, s>>>(dout.as<float>(), A.h3.as<__nv_bfloat16>(), N, g);
+    // The row sums occupy a few SMs for the length of their chains: they run on the
+    // thread's second stream beside the products, each after what it reads is complete,
+    // and s waits for them at the end.
+    SideWork side(s);
+    auto row_sums = [&](int K, const DevBuf& at, const float* w, float* dst, int sc, int sk, float* sums) {
+        cudaStream_t q = side.after();
+        k_row_sums<<<dim3(WS_H / 32, (unsigned)(K + (sums ? 1 : 0))), 128, 0, q>>>(at.as<__nv_bfloat16>(), A.ldt, w, K, N,
+                                                                                dst, sc, sk, sums);
+        UOI_CHECK_LAUNCH();
+        count_launch();
+    };
+    row_sums(WS_OUT, A.h3t, dout.as<float>(), g + OFF_W4, 1, WS_H, nullptr);
+    k_head_bias<<<WS_OUT, 32, 0, side.after()>>>(dout.as<float>(), N, g + OFF_B4);
     UOI_CHECK_LAUNCH();
-    k_col_sums<float><<<1, 32, 0, s>>>(dout.as<float>(), N, WS_OUT, g + OFF_B4);
-    UOI_CHECK_LAUNCH();
-    k_head_back<<<blocks_for(N * WS_H), 256, 0, s>>>(dout.as<float>(), N, M->w, A.a3.as<float>(),
-                                                     da3.as<__nv_bfloat16>(), da3t.as<__nv_bfloat16>(), A.ldt);
+    k_head_back<<<dim3((unsigned)ceil_div(N, 64), WS_H / 64), 256, 0, s>>>(
+        dout.as<float>(), N, M->w, A.a3.as<float>(), da3.as<__nv_bfloat16>(), da3t.as<__nv_bfloat16>(), A.ldt);
     UOI_CHECK_LAUNCH();
     // layer 3
     grad_square(da3t.as<__nv_bfloat16>(), A.h2t.as<__nv_bfloat16>(), A.ldt, N, g + OFF_W3, err.as<int32_t>(), s);
-    k_col_sums<__nv_bfloat16><<<WS_H / 128, 128, 0, s>>>(da3.as<__nv_bfloat16>(), N, WS_H, g + OFF_B3);
-    UOI_CHECK_LAUNCH();
+    row_sums(0, da3t, nullptr, nullptr, 0, 0, g + OFF_B3);
     mlp_backward_tc(da3.as<__nv_bfloat16>(), N, M->w3t, WS_H, A.a2.as<float>(), da2.as<__nv_bfloat16>(),
                     da2t.as<__nv_bfloat16>(), A.ldt, err.as<int32_t>(), s);                  // da2
     // layer 2
     grad_square(da2t.as<__nv_bfloat16>(), A.h1t.as<__nv_bfloat16>(), A.ldt, N, g + OFF_W2, err.as<int32_t>(), s);
-    k_col_sums<__nv_bfloat16><<<WS_H / 128, 128, 0, s>>>(da2.as<__nv_bfloat16>(), N, WS_H, g + OFF_B2);
-    UOI_CHECK_LAUNCH();
+    row_sums(0, da2t, nullptr, nullptr, 0, 0, g + OFF_B2);
     mlp_backward_tc(da2.as<__nv_bfloat16>(), N, M->w2t, WS_H, A.a1.as<float>(), da3.as<__nv_bfloat16>(),
-                    nullptr, 0, err.as<int32_t>(), s);                                       // da1 (in da3)
+                    da1t.as<__nv_bfloat16>(), A.ldt, err.as<int32_t>(), s);                  // da1 (in da3)
     // layer 1
-    k_grad_w1<<<WS_H / 128, 128, 0, s>>>(da3.as<__nv_bfloat16>(), X, N, g);
-    UOI_CHECK_LAUNCH();
-    k_col_sums<__nv_bfloat16><<<WS_H / 128, 128, 0, s>>>(da3.as<__nv_bfloat16>(), N, WS_H, g + OFF_B1);
-    UOI_CHECK_LAUNCH();
-    count_launch(8);
+    row_sums(WS_IN, da1t, X, g + OFF_W1, WS_IN, 1, g + OFF_B1);
+    side.join();
+    count_launch(3);
     check_err(err, s);
     std::vector<double> h(lb);
     UOI_CUDA(cudaMemcpyAsync(h.data(), lp.ptr, sizeof(double) * lb, cudaMemcpyDeviceToHost, s));
