@@ -25,6 +25,7 @@
 //    norms in a fixed order, finishes converged columns and compacts the active
 //    list.  The host checks the active count every few iterations.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "kernels.h"
@@ -237,15 +238,23 @@ __global__ void __launch_bounds__(256, 1) k_admm_resident(AdmmDev<T> P, int32_t*
 //             next iteration written into every CTA of the cluster;
 //   stop      the CTAs exchange five partial norms; one cluster barrier ends the
 //             iteration, after which every thread takes the same decision.
-// What bounds it: in FP64 the FP64 pipe, two multiply-adds per clock and SM on this
-// part with every warp instruction charged for 32 lanes.  So no instruction of the
-// iteration may run on few lanes, and the norms are first taken in FP32 (from the
-// FP64 differences): only when those say that the stop test may pass are they
-// formed in FP64, so that decisions are those of the FP64 norms.  M needs 16 B per
-// clock and SM, which L2 delivers.
-// Measured (one call, before: one warp per chain, or two launches per iteration): 200 x 50,
-// 20 chains, 598 iterations each: 12.7 -> 2.3 ms; p = 400, 20 chains: 38 -> 6.9 ms; p = 1000
-// (M 160 MB): 124 -> 53 ms; p = 150, 128 chains: 110 -> 3 ms.
+// FP64 products run on the integer pipe.  M and V are taken to integers Q, P of up to 57 bits
+// with sign (a power of two above the group's largest entry of M, on its diagonal, and above
+// V's largest value at this step), split into balanced digits of 28 bits, and
+//   x - c = rho 2^(..) sum_k hi hi' 2^56 + (hi lo' + lo hi') 2^28      (+ lo lo', below 2^-58)
+// is summed exactly in 64 bits by three 32 x 32 + 64 -> 64 multiply-adds per entry.  This
+// part's FP64 pipe charges 19 clocks and SM per warp instruction, the integer pipe 1 per
+// multiply-add.  The error is that of rounding M and V, 2^-57 of their largest values, where
+// an FP64 dot product rounds every partial sum at 2^-53.  The rest of an iteration is FP64:
+// no instruction of it may run on few lanes, and the norms are first taken in FP32 (from the
+// FP64 differences): only when those say that the stop test may pass are they formed in
+// FP64, so that decisions are those of the FP64 norms.
+// What bounds it: for small p the length of one iteration (about 10 dependent FP64 operations
+// at 64 clocks, two block barriers, the exchange); past L2 the stream of M.
+// Measured (one call; one warp per chain or two launches per iteration, then this schedule
+// with FP64 products, then as it is): 200 x 50, 20 chains, 598 iterations each: 12.7, 2.3,
+// 1.65 ms; p = 400, 20 chains: 38, 6.9, 3.8 ms; p = 1000 (M 160 MB): 124, 52, 26 ms;
+// p = 150, 128 chains: 110, 5.1, 3.0 ms.
 constexpr int CH_RB = 16;            // rows per block
 constexpr int CH_NB = 8;             // blocks accumulated together
 constexpr int CH_CLUSTER_MAX = 8;
@@ -257,6 +266,8 @@ struct ChainGeom {
     int32_t nrp;                     // rows of the largest CTA, a multiple of CH_RB
     int32_t kp;                      // k extent padded to a multiple of 2 * warps
     int32_t ldm;                     // row length of the shared copy of M, 0: M stays in global memory
+    int32_t bits;                    // FP64: ch_bits of the products one thread sums
+    int32_t fits;                    // FP64: the sum of all p products fits 63 bits
     size_t smem;
 };
 
@@ -284,8 +295,21 @@ __device__ __forceinline__ void ch_barrier(int cs)
     }
 }
 
-__device__ __forceinline__ float ch_f32(double x) { return f64_to_f32_int(x); }
-__device__ __forceinline__ float ch_f32(float x) { return x; }
+// |x| truncated to FP32 by integer operations (0 below 2^-126, Inf past FP32).
+__device__ __forceinline__ float ch_abs32(double x)
+{
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+    const uint32_t f = __funnelshift_l((uint32_t)__double2loint(x), h, 3) + 0x40000000u;   // exponent bias 1023 -> 127
+    return __uint_as_float(h < 0x38100000u ? 0u : h >= 0x47F00000u ? (h > 0x7FF00000u ? 0x7FC00000u : 0x7F800000u) : f);
+}
+__device__ __forceinline__ float ch_abs32(float x) { return x; }
+
+__device__ __forceinline__ float ch_sqrt(float x)            // to 2^-22
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 
 // soft_threshold with the comparisons on the integer pipe (FP64, k >= 0): one FP64
 // subtraction.
@@ -300,14 +324,63 @@ __device__ __forceinline__ double ch_threshold(double v, double k)
 }
 __device__ __forceinline__ float ch_threshold(float v, float k) { return soft_threshold(v, k); }
 
-// acc += m v: a plain multiply-add in FP64; in FP32 the rounding errors of the
-// product and of the sum go to a second word.
+// An entry of M or V as the kernel multiplies it: FP32 itself, or (FP64) an integer of up to
+// 57 bits as two balanced 28-bit digits, hi 2^28 + lo.
+template <typename T> struct ChNumOf;
+template <> struct ChNumOf<float> { using type = float; };
+template <> struct ChNumOf<double> { using type = int2; };
+
+// Bits of Q and P below the sign, at most 56: `terms` products of their upper digits fit
+// 61 bits.
+inline int ch_bits(int terms)
+{
+    int lg = 0;
+    while ((1 << lg) < terms) ++lg;
+    return 28 + (61 - (lg < 5 ? 5 : lg)) / 2;
+}
+
+// rint(x 2^(bits - e)) for |x| < 2^e as two digits.
+__device__ __forceinline__ int2 ch_fixed(double x, int e, int bits)
+{
+    const long long b = __double_as_longlong(x);
+    const int ex = (int)((b >> 52) & 0x7FF);
+    long long q = b & 0xFFFFFFFFFFFFFll;
+    if (ex) q |= 1ll << 52;
+    const int sh = max(ex, 1) - 1075 + bits - e;          // at most bits - 53
+    if (sh >= 0) q <<= sh;
+    else if (sh < -54) q = 0;
+    else q = (q + (1ll << (-sh - 1))) >> -sh;
+    if (b < 0) q = -q;
+    const long long hi = (q + (1ll << 27)) >> 28;
+    return make_int2((int)hi, (int)(q - (hi << 28)));
+}
+
+// e with |x| < 2^e for values whose high word (without sign) is at most h.
+__device__ __forceinline__ int ch_exponent(uint32_t h) { return max((int)(h >> 20), 1) - 1022; }
+
+// High word of |x|, 1 for a subnormal that lies in the low word alone.
+__device__ __forceinline__ uint32_t ch_high(double x)
+{
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+    return h == 0 && __double2loint(x) != 0 ? 1u : h;
+}
+
+// acc += m v.  FP64: exact 64-bit sums of the digits' products; value() is the sum in units
+// of 2^56, rounded.  FP32: the rounding errors of the product and of the sum go to a second
+// word.
 struct ChSumD {
-    double a = 0.0;
-    __device__ __forceinline__ void add(double m, double v) { a = fma(m, v, a); }
-    __device__ __forceinline__ double value() const { return a; }
+    using Out = long long;
+    long long hh = 0, mid = 0;
+    __device__ __forceinline__ void add(int2 m, int2 v)
+    {
+        hh += (long long)m.x * v.x;
+        mid += (long long)m.x * v.y;
+        mid += (long long)m.y * v.x;
+    }
+    __device__ __forceinline__ long long value() const { return hh + ((mid + (1ll << 27)) >> 28); }
 };
 struct ChSumF {
+    using Out = float;
     float a = 0.f, c = 0.f;
     __device__ __forceinline__ void add(float m, float v)
     {
@@ -325,20 +398,26 @@ template <> struct ChSumOf<float> { using type = ChSumF; };
 // NB blocks of one warp: out[(block * 16 + row)] of each slot (row stride `ostr` per
 // slot) = sum over this warp's k of M[k][row] V_slot[k].  m points at (k = 0, the
 // lane's row of the first block); rows of a block past the CTA's last repeat it.
-template <typename T, int NB, int NC>
-__device__ __forceinline__ void ch_product(const T* m, size_t ld, int p, const T* V, int kp, int k0, int kstep,
-                                           int row, int nrows, T* out, int ostr)
+template <typename T, int NB, int NC, bool SHARED>
+__device__ __forceinline__ void ch_product(const typename ChNumOf<T>::type* m, size_t ld, int p,
+                                           const typename ChNumOf<T>::type* V, int kp, int k0, int kstep, int row,
+                                           int nrows, typename ChSumOf<T>::type::Out* out, int ostr)
 {
+    using Num = typename ChNumOf<T>::type;
     typename ChSumOf<T>::type acc[NB][NC];
     int off[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b) off[b] = min(row + b * CH_RB, nrows - 1) - min(row, nrows - 1);
-#pragma unroll 2
-    for (int k = k0; k < kp; k += kstep) {
-        const T* mk = m + (size_t)min(k, p - 1) * ld;
-        T v[NC], x[NB];
+    // rows of the shared copy reach to kp (its padding meets zeros of V); streamed rows past
+    // p - 1 repeat the last
+    const size_t step = (size_t)kstep * ld;
+    const Num* mk = m + (size_t)min(k0, p - 1) * ld;
+#pragma unroll(NB > 4 || !SHARED ? 2 : 4)
+    for (int k = k0; k < kp; k += kstep, mk += step) {
+        const Num* mr = SHARED ? mk : m + (size_t)min(k, p - 1) * ld;
+        Num v[NC], x[NB];
 #pragma unroll
-        for (int b = 0; b < NB; ++b) x[b] = mk[off[b]];
+        for (int b = 0; b < NB; ++b) x[b] = mr[off[b]];
 #pragma unroll
         for (int c = 0; c < NC; ++c) v[c] = V[c * kp + k];
 #pragma unroll
@@ -350,20 +429,26 @@ __device__ __forceinline__ void ch_product(const T* m, size_t ld, int p, const T
     for (int b = 0; b < NB; ++b)
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            T s = acc[b][c].value();
+            typename ChSumOf<T>::type::Out s = acc[b][c].value();
             s += __shfl_xor_sync(0xffffffffu, s, CH_RB);
             if ((threadIdx.x & 31) < CH_RB) out[c * ostr + b * CH_RB] = s;
         }
 }
 
 template <typename T, int NC>
-__global__ void __launch_bounds__(512) k_admm_chain(AdmmDev<T> P, int32_t* chain_next, ChainGeom geo)
+__global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P, int32_t* chain_next, ChainGeom geo,
+                                                   const int32_t* m_exp)
 {
+    using Num = typename ChNumOf<T>::type;
+    using Sum = typename ChSumOf<T>::type::Out;
+    constexpr bool F64 = sizeof(T) == 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ T s_kappa[CH_KAPPA];
-    __shared__ float s_red[16][5], s_norm[2][CH_CLUSTER_MAX][NC][5];
+    __shared__ __align__(16) float s_red[5][16];
+    __shared__ float s_norm[2][CH_CLUSTER_MAX][NC][5];
     __shared__ T s_redx[16][5], s_exact[CH_CLUSTER_MAX][NC][5];
     __shared__ int s_cid[NC];
+    __shared__ uint32_t s_max[2][CH_CLUSTER_MAX][NC], s_redm[16];   // largest high word of |V'|
     const int p = P.p, cs = geo.cs, nrp = geo.nrp, kp = geo.kp;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, NW = blockDim.x >> 5;
     int rank = 0;
@@ -373,18 +458,57 @@ __global__ void __launch_bounds__(512) k_admm_chain(AdmmDev<T> P, int32_t* chain
     const int b0 = rank * nbt / cs, nblk = (rank + 1) * nbt / cs - b0;
     const int row0 = b0 * CH_RB, nrows = min(p - row0, nblk * CH_RB);
     const T* Mg = P.M + (size_t)g * p * p;
-    // shared memory: [M] | V, two buffers of NC | partial products | z u c x z_prev
-    T* Ms = reinterpret_cast<T*>(smem_raw);
-    T* V = Ms + (size_t)geo.ldm * p;
-    T* part = V + (size_t)2 * NC * kp;
-    T* zs = part + (size_t)NW * NC * nrp;
+    // shared memory: [M] | V, two buffers of NC | [FP64: V's digits] | partial products | z u c x z_prev
+    Num* Ms = reinterpret_cast<Num*>(smem_raw);
+    T* V = reinterpret_cast<T*>(Ms + (size_t)geo.ldm * kp);
+    Num* Vi = reinterpret_cast<Num*>(V + (size_t)2 * NC * kp);
+    Sum* part = reinterpret_cast<Sum*>(Vi + (F64 ? (size_t)NC * kp : 0));
+    T* zs = reinterpret_cast<T*>(part + (size_t)NW * NC * nrp);
     T* us = zs + NC * nrp;
     T* cv = us + NC * nrp;
     T* xs = cv + NC * nrp;
     T* zq = xs + NC * nrp;
-    if (geo.ldm)
-        for (int k = warp; k < p; k += NW)
-            for (int i = lane; i < nrows; i += 32) Ms[(size_t)k * geo.ldm + i] = Mg[(size_t)k * p + row0 + i];
+    const Num* Mi = reinterpret_cast<const Num*>(Mg);        // streamed M: digits already
+    int em = 0;                                              // |M| < 2^em
+    if constexpr (F64) {
+        if (geo.ldm) {
+            uint32_t h = 0;
+            for (int i = threadIdx.x; i < p; i += blockDim.x) h = max(h, ch_high(Mg[(size_t)i * p + i]));
+            h = __reduce_max_sync(0xffffffffu, h);
+            if (lane == 0) s_redm[warp] = h;
+            __syncthreads();
+            for (int w = 0; w < NW; ++w) h = max(h, s_redm[w]);
+            em = ch_exponent(h);
+            for (int k = warp; k < p; k += NW)
+                for (int i = lane; i < nrows; i += 32)
+                    Ms[(size_t)k * geo.ldm + i] = ch_fixed(Mg[(size_t)k * p + row0 + i], em, geo.bits);
+        } else {
+            em = m_exp[g];
+        }
+    } else if (geo.ldm) {
+        for (int k = warp; k < kp; k += NW)
+            for (int i = lane; i < nrows; i += 32)
+                Ms[(size_t)k * geo.ldm + i] = k < p ? Mg[(size_t)k * p + row0 + i] : T(0);
+    }
+    // digits of V_slot from buffer `buf`, their scale in rs[slot]: x = c + rs (sum of digits)
+    T rs[NC];
+    int rho_e = 0;                                           // exponent field of rho (0: subnormal, scaled by scalbn)
+    if constexpr (F64) {
+        rho_e = (__double2hiint(P.rho) >> 20) & 0x7FF;
+        if (rho_e == 0) rho_e = -100000;
+    }
+    auto digits = [&](int buf, int s, uint32_t h) {
+        if constexpr (F64) {
+            const int ev = h == 0 ? 0 : ch_exponent(h);
+            const T* src = V + ((size_t)buf * NC + s) * kp;
+            for (int k = threadIdx.x; k < kp; k += blockDim.x) Vi[s * kp + k] = ch_fixed(src[k], ev, geo.bits);
+            // M = Q 2^(em - bits), V = P 2^(ev - bits), sums in units of 2^56; NaN if V holds Inf or NaN
+            const int x = em + ev - 2 * geo.bits + 56;
+            if (h >= 0x7FF00000u) rs[s] = __longlong_as_double(0x7FF8000000000000ll);
+            else if (x + rho_e > 0 && x + rho_e < 2046) rs[s] = __longlong_as_double(__double_as_longlong(P.rho) + ((long long)x << 52));
+            else rs[s] = scalbn(P.rho, x);
+        }
+    };
     for (int i = threadIdx.x; i < 2 * NC * kp; i += blockDim.x) V[i] = T(0);
     for (int i = threadIdx.x; i < min(P.q, CH_KAPPA); i += blockDim.x) s_kappa[i] = (T)P.lambdas[i] / P.rho;
 
@@ -423,8 +547,22 @@ __global__ void __launch_bounds__(512) k_admm_chain(AdmmDev<T> P, int32_t* chain
                 cv[s * nrp + i] = P.c[((size_t)g * P.r + e_[s]) * p + row0 + i];
             }
             T* Vn = V + ((size_t)buf * NC + s) * kp;
-            for (int k = threadIdx.x; k < p; k += blockDim.x)
-                Vn[k] = init ? (T)P.z0[col0 * p + k] - (T)P.u0[col0 * p + k] : T(0);
+            uint32_t h = 0;
+            for (int k = threadIdx.x; k < p; k += blockDim.x) {
+                const T v0 = init ? (T)P.z0[col0 * p + k] - (T)P.u0[col0 * p + k] : T(0);
+                Vn[k] = v0;
+                if constexpr (F64) h = max(h, ch_high(v0));
+            }
+            if constexpr (F64) {
+                if (init) {                              // the largest value of the start, over the block
+                    h = __reduce_max_sync(0xffffffffu, h);
+                    __syncthreads();
+                    if (lane == 0) s_redm[warp] = h;
+                    __syncthreads();
+                    for (int w = 0; w < NW; ++w) h = max(h, s_redm[w]);
+                }
+                digits(buf, s, h);                       // a zero start needs no barrier: every digit is zero
+            }
         }
         __syncthreads();
     };
@@ -440,28 +578,35 @@ __global__ void __launch_bounds__(512) k_admm_chain(AdmmDev<T> P, int32_t* chain
         // product
         {
             const int kk = lane / CH_RB, ri = lane % CH_RB;
-            const T* Vc = V + (size_t)cur * NC * kp;
-            T* pw = part + (size_t)warp * NC * nrp;
+            const Num* Vc;
+            if constexpr (F64) Vc = Vi;
+            else Vc = V + (size_t)cur * NC * kp;
+            Sum* pw = part + (size_t)warp * NC * nrp;
             const size_t ld = geo.ldm ? (size_t)geo.ldm : (size_t)p;
-            const T* base = geo.ldm ? Ms : Mg + row0;
+            const Num* base = geo.ldm ? Ms : Mi + row0;
             constexpr int CB = NC == 1 ? CH_NB : CH_NB / 2;
             for (int c0 = 0; c0 < nblk; c0 += CB) {
                 const int row = c0 * CH_RB + ri;
-                const T* m = base + min(row, nrows - 1);
-                T* o = pw + row;
+                const Num* m = base + min(row, nrows - 1);
+                Sum* o = pw + row;
                 const int k0 = 2 * warp + kk, ks = 2 * NW;
+                auto run = [&](auto nb) {
+                    constexpr int NB = decltype(nb)::value;
+                    if (geo.ldm) ch_product<T, NB, NC, true>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp);
+                    else if constexpr (F64) ch_product<T, NB, NC, false>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp);
+                };
                 switch (min(CB, nblk - c0)) {
-                case 1: ch_product<T, 1, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
-                case 2: ch_product<T, 2, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
-                case 3: ch_product<T, 3, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
-                case 4: ch_product<T, 4, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                case 1: run(std::integral_constant<int, 1>{}); break;
+                case 2: run(std::integral_constant<int, 2>{}); break;
+                case 3: run(std::integral_constant<int, 3>{}); break;
+                case 4: run(std::integral_constant<int, 4>{}); break;
                 default:
                     if constexpr (NC == 1) {
                         switch (min(CB, nblk - c0)) {
-                        case 5: ch_product<T, 5, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
-                        case 6: ch_product<T, 6, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
-                        case 7: ch_product<T, 7, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
-                        default: ch_product<T, 8, NC>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp); break;
+                        case 5: run(std::integral_constant<int, 5>{}); break;
+                        case 6: run(std::integral_constant<int, 6>{}); break;
+                        case 7: run(std::integral_constant<int, 7>{}); break;
+                        default: run(std::integral_constant<int, 8>{}); break;
                         }
                     }
                 }
@@ -470,23 +615,41 @@ __global__ void __launch_bounds__(512) k_admm_chain(AdmmDev<T> P, int32_t* chain
         __syncthreads();
         // update
         {
-            T kap = T(0);
+            T kap = T(0), scale = T(0);
             bool on = false;
+            uint32_t big = 0;                                // largest high word of |V'|
 #pragma unroll
             for (int s = 0; s < NC; ++s)
-                if (slot == s) { kap = kappa[s]; on = act[s]; }
+                if (slot == s) { kap = kappa[s]; on = act[s]; scale = rs[s]; }
             float n5[5] = { 0.f, 0.f, 0.f, 0.f, 0.f };
             if (on)
                 for (int i = wi * 32 + lane; i < nrows; i += nwi * 32) {
                     const int o = slot * nrp + i;
-                    T sum = part[o];
-                    for (int w = 1; w < NW; ++w) sum += part[(size_t)w * NC * nrp + o];
-                    const T x = cv[o] + P.rho * sum;
+                    T x;
+                    if constexpr (F64) {
+                        // partial sums below 2^62 each: their halves add up in 64 bits
+                        long long up = 0, dn = 0;
+                        if (geo.fits) {                      // and all of them below 2^63
+                            for (int w = 0; w < NW; ++w) dn += part[(size_t)w * NC * nrp + o];
+                        } else {
+                            for (int w = 0; w < NW; ++w) {
+                                const long long q = part[(size_t)w * NC * nrp + o];
+                                up += q >> 32;
+                                dn += (long long)(uint32_t)q;
+                            }
+                        }
+                        x = cv[o] + scale * fma((double)up, 4294967296.0, (double)dn);
+                    } else {
+                        T sum = part[o];
+                        for (int w = 1; w < NW; ++w) sum += part[(size_t)w * NC * nrp + o];
+                        x = cv[o] + P.rho * sum;
+                    }
                     const T zp = zs[o];
                     const T v = x + us[o];
                     const T zn = ch_threshold(v, kap);
                     const T un = v - zn;
                     const T vn = zn - un;
+                    if constexpr (F64) big = max(big, ch_high(vn));
                     const T d = x - zn, dz = zn - zp;
                     zs[o] = zn;
                     us[o] = un;
@@ -496,25 +659,50 @@ __global__ void __launch_bounds__(512) k_admm_chain(AdmmDev<T> P, int32_t* chain
                     if (cs == 1) *dst = vn;
                     else
                         for (int t = 0; t < cs; ++t) ch_store_rank(dst, t, vn);
-                    const float fd = ch_f32(d), fz = ch_f32(dz), fx = ch_f32(x), fn = ch_f32(zn), fu = ch_f32(un);
+                    const float fd = ch_abs32(d), fz = ch_abs32(dz), fx = ch_abs32(x), fn = ch_abs32(zn), fu = ch_abs32(un);
                     n5[0] += fd * fd; n5[1] += fz * fz; n5[2] += fx * fx; n5[3] += fn * fn; n5[4] += fu * fu;
                 }
 #pragma unroll
             for (int t = 0; t < 5; ++t) {
                 const float w = warp_sum(n5[t]);
-                if (lane == 0) s_red[warp][t] = w;
+                if (lane == 0) s_red[t][warp] = w;
+            }
+            if constexpr (F64) {
+                big = __reduce_max_sync(0xffffffffu, big);
+                if (lane == 0) s_redm[warp] = big;
             }
         }
         __syncthreads();
-        if (threadIdx.x < NC * 5) {
-            const int s = threadIdx.x / 5, t = threadIdx.x % 5;
-            float w = 0.f;
-            for (int k = 0; k < nwi; ++k) w += s_red[k * NC + s][t];
-            if (cs == 1) s_norm[cur][0][s][t] = w;
-            else
-                for (int k = 0; k < cs; ++k) ch_store_rank(&s_norm[cur][rank][s][t], k, w);
+        // the CTA's norms and largest V' to every CTA of the cluster, one thread per value and CTA;
+        // a CTA alone reads its warps' values as they are
+        if (cs > 1) {
+            constexpr int per = NC * 6;
+            for (int i = threadIdx.x; i < per * cs; i += blockDim.x) {
+                const int k = i / per, s = (i % per) / 6, t = i % 6;
+                if (t < 5) {
+                    float w = 0.f;
+                    for (int q = 0; q < nwi; ++q) w += s_red[t][q * NC + s];
+                    ch_store_rank(&s_norm[cur][rank][s][t], k, w);
+                } else if (F64) {
+                    uint32_t h = 0;
+                    for (int q = 0; q < nwi; ++q) h = max(h, s_redm[q * NC + s]);
+                    ch_store_rank(&s_max[cur][rank][s], k, h);
+                }
+            }
+            ch_barrier(cs);
         }
-        ch_barrier(cs);
+        if constexpr (F64) {
+#pragma unroll
+            for (int s = 0; s < NC; ++s) {
+                if (!act[s]) continue;
+                uint32_t h = 0;
+                if (cs == 1)
+                    for (int q = 0; q < nwi; ++q) h = max(h, s_redm[q * NC + s]);
+                else
+                    for (int k = 0; k < cs; ++k) h = max(h, s_max[cur][k][s]);
+                digits(cur ^ 1, s, h);                       // of the next product
+            }
+        }
         // stop test
         bool conv[NC];
         unsigned maybe = 0;
@@ -523,15 +711,24 @@ __global__ void __launch_bounds__(512) k_admm_chain(AdmmDev<T> P, int32_t* chain
             conv[s] = false;
             if (!act[s]) continue;
             float n[5] = { 0.f, 0.f, 0.f, 0.f, 0.f };
-            for (int k = 0; k < cs; ++k)
+            if (cs > 1) {
+                for (int k = 0; k < cs; ++k)
 #pragma unroll
-                for (int t = 0; t < 5; ++t) n[t] += s_norm[cur][k][s][t];
+                    for (int t = 0; t < 5; ++t) n[t] += s_norm[cur][k][s][t];
+            } else {
+                for (int q = 0; q < nwi; ++q)
+#pragma unroll
+                    for (int t = 0; t < 5; ++t) n[t] += s_red[t][q * NC + s];
+            }
             const float base = (float)P.sqrtp * (float)P.abs_tol, rel = (float)P.rel_tol, rho = (float)P.rho;
-            const float ep = base + rel * fmaxf(sqrtf(n[2]), sqrtf(n[3])), ed = base + rel * rho * sqrtf(n[4]);
-            if constexpr (sizeof(T) == 4)
+            if constexpr (!F64) {
+                const float ep = base + rel * fmaxf(sqrtf(n[2]), sqrtf(n[3])), ed = base + rel * rho * sqrtf(n[4]);
                 conv[s] = sqrtf(n[0]) <= ep && rho * sqrtf(n[1]) <= ed;
-            else if (!(sqrtf(n[0]) > CH_SCREEN * ep) && !(rho * sqrtf(n[1]) > CH_SCREEN * ed))
-                maybe |= 1u << s;
+            } else {
+                const float ep = CH_SCREEN * (base + rel * ch_sqrt(fmaxf(n[2], n[3])));
+                const float ed = CH_SCREEN * (base + rel * rho * ch_sqrt(n[4]));
+                if (!(ch_sqrt(n[0]) > ep) && !(rho * ch_sqrt(n[1]) > ed)) maybe |= 1u << s;
+            }
         }
         if constexpr (sizeof(T) == 8) {
             if (maybe) {                                     // the same in every thread of the cluster
@@ -613,9 +810,37 @@ __global__ void __launch_bounds__(512) k_admm_chain(AdmmDev<T> P, int32_t* chain
         if (need) {
             __syncthreads();                                 // every thread has read the finished chain's z, u
             fetch(need, cur ^ 1);
+        } else if (F64) {
+            __syncthreads();                                 // V's digits
         }
     }
     if (cs > 1) ch_barrier(cs);                              // no CTA leaves while another may store into it
+}
+
+// Streamed M of the FP64 chain schedule: exponent of each group, then digits in place.
+__global__ void k_chain_exponent(const double* M, int p, int32_t* em)
+{
+    __shared__ uint32_t red[8];
+    const double* m = M + (size_t)blockIdx.x * p * p;
+    uint32_t h = 0;
+    for (int i = threadIdx.x; i < p; i += blockDim.x) h = max(h, ch_high(m[(size_t)i * p + i]));
+    h = __reduce_max_sync(0xffffffffu, h);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = h;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) h = max(h, red[w]);
+        em[blockIdx.x] = ch_exponent(h);
+    }
+}
+
+__global__ void k_chain_digits(double* M, int64_t pp, const int32_t* em, int bits)
+{
+    double* m = M + (size_t)blockIdx.y * pp;
+    const int e = em[blockIdx.y];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < pp; i += (int64_t)gridDim.x * blockDim.x) {
+        const int2 d = ch_fixed(m[i], e, bits);
+        m[i] = __hiloint2double(d.y, d.x);                   // the pair's first member in the low word
+    }
 }
 
 // ----------------------------------------------------------------------------
@@ -1028,7 +1253,10 @@ bool launch_chain_nc(const AdmmDev<T>& d, int32_t* chain_next, int nw, int cs, b
     geo.kp = (int)ceil_div(d.p, 2 * nw) * 2 * nw;
     // FP32 rows of M 64 bytes apart modulo 128, so that a warp's two rows use all banks
     geo.ldm = m_smem ? (sizeof(T) == 4 && geo.nrp % 32 == 0 ? geo.nrp + CH_RB : geo.nrp) : 0;
-    geo.smem = sizeof(T) * ((size_t)geo.ldm * d.p + (size_t)2 * NC * geo.kp + (size_t)(nw + 5) * NC * geo.nrp);
+    geo.smem = sizeof(T) * ((size_t)geo.ldm * geo.kp + (size_t)(sizeof(T) == 8 ? 3 : 2) * NC * geo.kp +
+                            (size_t)(nw + 5) * NC * geo.nrp);
+    geo.bits = ch_bits(geo.kp / (2 * nw));
+    geo.fits = 2 * (geo.bits - 28) + (geo.kp <= 64 ? 6 : 63) <= 62 ? 1 : 0;
     auto kern = k_admm_chain<T, NC>;
     int dev = 0, optin = 0, nsm = 0;
     UOI_CUDA(cudaGetDevice(&dev));
@@ -1060,7 +1288,21 @@ bool launch_chain_nc(const AdmmDev<T>& d, int32_t* chain_next, int nw, int cs, b
     }
     const int per = std::max(1, std::min((int)ceil_div(nchains, NC), resident / std::max(1, d.G)));
     cfg.gridDim = dim3((unsigned)(cs * per), (unsigned)d.G);
-    UOI_CUDA(cudaLaunchKernelEx(&cfg, kern, d, chain_next, geo));
+    int32_t* em = chain_next + d.G;                  // exponents of the streamed M
+    if constexpr (sizeof(T) == 8) {
+        if (!geo.ldm) {
+            // the solve is M's last reader: its entries turn into their digits in place
+            double* M = const_cast<double*>(d.M);
+            const int64_t pp = (int64_t)d.p * d.p;
+            k_chain_exponent<<<d.G, 256, 0, s>>>(M, d.p, em);
+            UOI_CHECK_LAUNCH();
+            k_chain_digits<<<dim3((unsigned)std::min<int64_t>(ceil_div(pp, 1024), 1024), (unsigned)d.G), 256, 0, s>>>(
+                M, pp, em, geo.bits);
+            UOI_CHECK_LAUNCH();
+            count_launch(2);
+        }
+    }
+    UOI_CUDA(cudaLaunchKernelEx(&cfg, kern, d, chain_next, geo, (const int32_t*)em));
     UOI_CHECK_LAUNCH();
     count_launch();
     return true;
@@ -1075,7 +1317,7 @@ bool try_chain(const AdmmDev<T>& d, int32_t* chain_next, cudaStream_t s)
     int cs = 1;
     if (total < NSM)
         cs = (int)std::max<int64_t>(1, std::min<int64_t>({ CH_CLUSTER_MAX, GPC_FIT / total, d.p / 32 }));
-    constexpr int NW_S = sizeof(T) == 8 ? 4 : 8;  // warps with M in shared memory
+    const int NW_S = sizeof(T) == 8 && d.p <= 96 ? 4 : 8;   // warps with M in shared memory
     for (; cs <= CH_CLUSTER_MAX; ++cs) {
         if (launch_chain_nc<T, 1>(d, chain_next, NW_S, cs, true, nchains, s)) return true;
         if constexpr (sizeof(T) == 8) {
@@ -1118,7 +1360,7 @@ void admm_solve(const AdmmProblem<T>& P, cudaStream_t s)
     if constexpr (sizeof(T) == 4)
         if (nchains > 4 && admm_solve_wide(P, s)) return;
     {
-        DevBuf next(sizeof(int32_t) * P.G, s);
+        DevBuf next(sizeof(int32_t) * 2 * P.G, s);
         UOI_CUDA(cudaMemsetAsync(next.ptr, 0, next.bytes, s));
         if (try_resident<T>(d, next.as<int32_t>(), s)) return;
     }

@@ -191,7 +191,7 @@ struct AdmmProblem {
     int32_t G = 0;            // groups (bootstraps) sharing p
     int64_t p = 0, r = 0;     // features, response columns per group
     int32_t q = 0;            // lambdas
-    const T* M = nullptr;     // G x p x p   (A_g^{-1}, symmetric)
+    const T* M = nullptr;     // G x p x p   (A_g^{-1}, symmetric); the FP64 solve may overwrite it
     const T* c = nullptr;     // G x r x p   (A_g^{-1} b_ge / n_g)
     const double* lambdas = nullptr;   // q (device)
     double rho = 1.0, abs_tol = 1e-6, rel_tol = 1e-6;
@@ -233,8 +233,8 @@ void admm_batch_destroy(AdmmBatch* b);
 void admm_batch_enter(AdmmBatch* b);
 void admm_batch_leave();
 bool admm_batch_try_join(const AdmmProblem<float>& P, cudaStream_t s);
-// Resident schedule only, with the caller's zeroed per-group chain counters
-// (G int32).  Returns false (launching nothing) when p is too large for it.
+// Chain or resident schedule only, with the caller's zeroed per-group words (2 G int32:
+// chain counters, then exponents).  Returns false (launching nothing) when p is too large for it.
 template <typename T>
 bool admm_solve_resident_with(const AdmmProblem<T>& P, int32_t* chain_next, cudaStream_t s);
 
