@@ -28,6 +28,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "fixed_dot.cuh"
 #include "kernels.h"
 
 namespace uoi {
@@ -266,7 +267,7 @@ struct ChainGeom {
     int32_t nrp;                     // rows of the largest CTA, a multiple of CH_RB
     int32_t kp;                      // k extent padded to a multiple of 2 * warps
     int32_t ldm;                     // row length of the shared copy of M, 0: M stays in global memory
-    int32_t bits;                    // FP64: ch_bits of the products one thread sums
+    int32_t bits;                    // FP64: fx_bits of the products one thread sums
     int32_t fits;                    // FP64: the sum of all p products fits 63 bits
     size_t smem;
 };
@@ -330,55 +331,9 @@ template <typename T> struct ChNumOf;
 template <> struct ChNumOf<float> { using type = float; };
 template <> struct ChNumOf<double> { using type = int2; };
 
-// Bits of Q and P below the sign, at most 56: `terms` products of their upper digits fit
-// 61 bits.
-inline int ch_bits(int terms)
-{
-    int lg = 0;
-    while ((1 << lg) < terms) ++lg;
-    return 28 + (61 - (lg < 5 ? 5 : lg)) / 2;
-}
-
-// rint(x 2^(bits - e)) for |x| < 2^e as two digits.
-__device__ __forceinline__ int2 ch_fixed(double x, int e, int bits)
-{
-    const long long b = __double_as_longlong(x);
-    const int ex = (int)((b >> 52) & 0x7FF);
-    long long q = b & 0xFFFFFFFFFFFFFll;
-    if (ex) q |= 1ll << 52;
-    const int sh = max(ex, 1) - 1075 + bits - e;          // at most bits - 53
-    if (sh >= 0) q <<= sh;
-    else if (sh < -54) q = 0;
-    else q = (q + (1ll << (-sh - 1))) >> -sh;
-    if (b < 0) q = -q;
-    const long long hi = (q + (1ll << 27)) >> 28;
-    return make_int2((int)hi, (int)(q - (hi << 28)));
-}
-
-// e with |x| < 2^e for values whose high word (without sign) is at most h.
-__device__ __forceinline__ int ch_exponent(uint32_t h) { return max((int)(h >> 20), 1) - 1022; }
-
-// High word of |x|, 1 for a subnormal that lies in the low word alone.
-__device__ __forceinline__ uint32_t ch_high(double x)
-{
-    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
-    return h == 0 && __double2loint(x) != 0 ? 1u : h;
-}
-
 // acc += m v.  FP64: exact 64-bit sums of the digits' products; value() is the sum in units
 // of 2^56, rounded.  FP32: the rounding errors of the product and of the sum go to a second
 // word.
-struct ChSumD {
-    using Out = long long;
-    long long hh = 0, mid = 0;
-    __device__ __forceinline__ void add(int2 m, int2 v)
-    {
-        hh += (long long)m.x * v.x;
-        mid += (long long)m.x * v.y;
-        mid += (long long)m.y * v.x;
-    }
-    __device__ __forceinline__ long long value() const { return hh + ((mid + (1ll << 27)) >> 28); }
-};
 struct ChSumF {
     using Out = float;
     float a = 0.f, c = 0.f;
@@ -392,7 +347,7 @@ struct ChSumF {
     __device__ __forceinline__ float value() const { return a + c; }
 };
 template <typename T> struct ChSumOf;
-template <> struct ChSumOf<double> { using type = ChSumD; };
+template <> struct ChSumOf<double> { using type = FxSum; };
 template <> struct ChSumOf<float> { using type = ChSumF; };
 
 // NB blocks of one warp: out[(block * 16 + row)] of each slot (row stride `ostr` per
@@ -473,15 +428,15 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
     if constexpr (F64) {
         if (geo.ldm) {
             uint32_t h = 0;
-            for (int i = threadIdx.x; i < p; i += blockDim.x) h = max(h, ch_high(Mg[(size_t)i * p + i]));
+            for (int i = threadIdx.x; i < p; i += blockDim.x) h = max(h, fx_high(Mg[(size_t)i * p + i]));
             h = __reduce_max_sync(0xffffffffu, h);
             if (lane == 0) s_redm[warp] = h;
             __syncthreads();
             for (int w = 0; w < NW; ++w) h = max(h, s_redm[w]);
-            em = ch_exponent(h);
+            em = fx_exponent(h);
             for (int k = warp; k < p; k += NW)
                 for (int i = lane; i < nrows; i += 32)
-                    Ms[(size_t)k * geo.ldm + i] = ch_fixed(Mg[(size_t)k * p + row0 + i], em, geo.bits);
+                    Ms[(size_t)k * geo.ldm + i] = fx_digits(Mg[(size_t)k * p + row0 + i], em, geo.bits);
         } else {
             em = m_exp[g];
         }
@@ -499,9 +454,9 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
     }
     auto digits = [&](int buf, int s, uint32_t h) {
         if constexpr (F64) {
-            const int ev = h == 0 ? 0 : ch_exponent(h);
+            const int ev = h == 0 ? 0 : fx_exponent(h);
             const T* src = V + ((size_t)buf * NC + s) * kp;
-            for (int k = threadIdx.x; k < kp; k += blockDim.x) Vi[s * kp + k] = ch_fixed(src[k], ev, geo.bits);
+            for (int k = threadIdx.x; k < kp; k += blockDim.x) Vi[s * kp + k] = fx_digits(src[k], ev, geo.bits);
             // M = Q 2^(em - bits), V = P 2^(ev - bits), sums in units of 2^56; NaN if V holds Inf or NaN
             const int x = em + ev - 2 * geo.bits + 56;
             if (h >= 0x7FF00000u) rs[s] = __longlong_as_double(0x7FF8000000000000ll);
@@ -551,7 +506,7 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
             for (int k = threadIdx.x; k < p; k += blockDim.x) {
                 const T v0 = init ? (T)P.z0[col0 * p + k] - (T)P.u0[col0 * p + k] : T(0);
                 Vn[k] = v0;
-                if constexpr (F64) h = max(h, ch_high(v0));
+                if constexpr (F64) h = max(h, fx_high(v0));
             }
             if constexpr (F64) {
                 if (init) {                              // the largest value of the start, over the block
@@ -649,7 +604,7 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
                     const T zn = ch_threshold(v, kap);
                     const T un = v - zn;
                     const T vn = zn - un;
-                    if constexpr (F64) big = max(big, ch_high(vn));
+                    if constexpr (F64) big = max(big, fx_high(vn));
                     const T d = x - zn, dz = zn - zp;
                     zs[o] = zn;
                     us[o] = un;
@@ -823,13 +778,13 @@ __global__ void k_chain_exponent(const double* M, int p, int32_t* em)
     __shared__ uint32_t red[8];
     const double* m = M + (size_t)blockIdx.x * p * p;
     uint32_t h = 0;
-    for (int i = threadIdx.x; i < p; i += blockDim.x) h = max(h, ch_high(m[(size_t)i * p + i]));
+    for (int i = threadIdx.x; i < p; i += blockDim.x) h = max(h, fx_high(m[(size_t)i * p + i]));
     h = __reduce_max_sync(0xffffffffu, h);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = h;
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int w = 1; w < 8; ++w) h = max(h, red[w]);
-        em[blockIdx.x] = ch_exponent(h);
+        em[blockIdx.x] = fx_exponent(h);
     }
 }
 
@@ -838,7 +793,7 @@ __global__ void k_chain_digits(double* M, int64_t pp, const int32_t* em, int bit
     double* m = M + (size_t)blockIdx.y * pp;
     const int e = em[blockIdx.y];
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < pp; i += (int64_t)gridDim.x * blockDim.x) {
-        const int2 d = ch_fixed(m[i], e, bits);
+        const int2 d = fx_digits(m[i], e, bits);
         m[i] = __hiloint2double(d.y, d.x);                   // the pair's first member in the low word
     }
 }
@@ -1255,7 +1210,7 @@ bool launch_chain_nc(const AdmmDev<T>& d, int32_t* chain_next, int nw, int cs, b
     geo.ldm = m_smem ? (sizeof(T) == 4 && geo.nrp % 32 == 0 ? geo.nrp + CH_RB : geo.nrp) : 0;
     geo.smem = sizeof(T) * ((size_t)geo.ldm * geo.kp + (size_t)(sizeof(T) == 8 ? 3 : 2) * NC * geo.kp +
                             (size_t)(nw + 5) * NC * geo.nrp);
-    geo.bits = ch_bits(geo.kp / (2 * nw));
+    geo.bits = fx_bits(geo.kp / (2 * nw));
     geo.fits = 2 * (geo.bits - 28) + (geo.kp <= 64 ? 6 : 63) <= 62 ? 1 : 0;
     auto kern = k_admm_chain<T, NC>;
     int dev = 0, optin = 0, nsm = 0;

@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "fixed_dot.cuh"
 #include "kernels.h"
 
 namespace uoi {
@@ -24,7 +25,9 @@ namespace uoi {
 namespace {
 
 constexpr int OLS_SMEM_MAX = 160;   // supports up to this size factor in shared memory (FP64 path)
-constexpr int OLS_SMALL = 128;      // mixed path: supports up to this size form the small class
+// mixed path: a warp, a CTA with 4 x 4 or 8 x 8 register tiles, a CTA with a blocked factor
+constexpr int OLS_CLASSES = 4;
+constexpr int OLS_CLASS_MAX[OLS_CLASSES] = { 32, 64, 128, 0x7fffffff };
 // ADMM at lambda = 0 for singular supports: rho relative to the largest diagonal
 // (directions with eigenvalue >> rho converge in a few steps), the stopping
 // test on the relative change, and the iteration cap.
@@ -46,6 +49,7 @@ struct OlsArgs {
     double* scratch;                         // global factor scratch (per CTA), or null
     int64_t solves;
     int smax;                                // max support size
+    int s_lo;                                // mixed pass: solves with fewer or more than smax are another kernel's
     bool use_smem;
     const int32_t* list;                     // solve indices to run (null: 0 .. solves-1)
     // Moments restricted to the union U of the family supports: Gt, Ge are
@@ -57,13 +61,55 @@ struct OlsArgs {
     int32_t* fb_list;                        // mixed pass: solves left to the FP64 kernel
     int32_t* fb_count;
     float* fscratch;                         // mixed pass: global packed factor (per CTA), or null
-    const int32_t* je_list;                  // mixed loss pass: the (j*r + e) it covers (else all)
-    int32_t n_je;
-    // mixed loss pass with je_list: when set, CTAs take solves in order from this
-    // counter (preset to 0), support-major (t = rank of je in je_list * B2 + k), so a
-    // list sorted by decreasing support size runs the largest factors first
+    // mixed loss pass: the (j*r + e) it covers, taken in order from the counter `next`
+    // (preset to 0), support-major (t = rank of je in je_list * B2 + k), so a list sorted
+    // by decreasing support size runs the largest factors first
+    const int32_t* je_list;
     unsigned long long* next;
 };
+
+// The t-th solve of a mixed pass: bootstrap k, lambda j, response e, and its index in the
+// numbering of k_ols (for the FP64 hand-over).
+struct OlsSolve { int k, j, e; int64_t tg; };
+__device__ __forceinline__ OlsSolve ols_solve(const OlsArgs& a, int64_t t)
+{
+    OlsSolve o;
+    if (a.jstar) {
+        o.k = (int)(t / a.r); o.e = (int)(t % a.r); o.j = a.jstar[o.k];
+        o.tg = t;
+    } else {
+        const int32_t je = a.je_list[t / a.B2];
+        o.k = (int)(t % a.B2); o.j = (int)(je / a.r); o.e = (int)(je % a.r);
+        o.tg = ((int64_t)o.k * a.q + o.j) * a.r + o.e;
+    }
+    return o;
+}
+
+// Set bits of W words (bits below p) in increasing order, plus `base`, the first `cap` to idx,
+// and their number, by one warp: a word per lane, offsets by a prefix sum of their counts.
+__device__ __forceinline__ int warp_support(const uint64_t* bits, int W, int64_t p, int lane, int* idx, int cap,
+                                            int base = 0)
+{
+    int cnt = 0;
+    for (int w0 = 0; w0 < W; w0 += 32) {
+        const int wi = w0 + lane;
+        uint64_t word = wi < W ? bits[wi] : 0;
+        if (p < (int64_t)(wi + 1) * 64) word &= (1ull << (p & 63)) - 1ull;
+        const int c = __popcll(word);
+        int pos = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, pos, o);
+            if (lane >= o) pos += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, pos, 31);
+        for (pos += cnt - c; word; word &= word - 1, ++pos)
+            if (pos < cap) idx[pos] = base + wi * 64 + __ffsll((long long)word) - 1;
+        cnt += total;
+    }
+    __syncwarp();
+    return cnt;
+}
 
 __global__ void __launch_bounds__(256) k_ols(OlsArgs a)
 {
@@ -224,12 +270,21 @@ __global__ void __launch_bounds__(256) k_ols(OlsArgs a)
     }
 }
 
-// Mixed-precision form of the same solve: Cholesky of G'_k[S,S] rounded to FP32
-// (packed lower triangle), then iterative refinement with FP64 residuals
-// r = b - G x until the correction is at FP64 rounding level, so the result
-// agrees with an FP64 factorisation to ~kappa * 1e-16.  A solve whose FP32
-// pivots fall below 1e-3 of the largest diagonal (where FP32 cannot certify the
-// 1e-12 singularity test) or whose refinement stalls is queued for k_ols.
+// Mixed-precision form of the same solve: an FP32 inverse or factor of G'_k[S,S], then iterative
+// refinement with FP64 residuals r = b - G x until the correction is at FP64 rounding level, so
+// the result agrees with an FP64 factorisation to ~kappa * 1e-16.  A solve whose FP32 pivots
+// fall below 1e-3 of the largest diagonal (where FP32 cannot certify the 1e-12 singularity
+// test) or whose refinement stalls is queued for k_ols.
+//
+// Up to 128 columns (k_ols_warp, k_ols_block) the solve is a symmetric Gauss-Jordan sweep in
+// registers, which leaves -G^{-1}: a refinement step is then a matrix-vector product instead of
+// two substitutions, whose s dependent steps were most of a small solve's time.  The pivots are
+// those of the Cholesky factor.  G is scaled by a power of two below 1 and kept as exact
+// integers (fixed_dot.cuh) for the residuals: the FP64 pipe would take 19 clocks per 32 entries
+// and the gather of G from L2 would be repeated at each step.
+// Measured (all solves of a fit, against one CTA with a packed factor for every size): VAR
+// p = 192, 30 bootstraps x 32 lambdas (supports of a few to 30 columns): 4.1 -> 0.25 ms;
+// 4999 x 301, 24 x 32 (15 to 111 columns): 0.43 -> 0.13 ms.
 constexpr float OLS_F32_PIVOT = 1e-3f;
 constexpr int OLS_REFINE_MAX = 8;
 
@@ -305,11 +360,385 @@ __device__ __forceinline__ double block_sum(double v, double* red, int lane, int
     return t;
 }
 
-// PB: k chunk of the trailing update's 4 x 4 register tiles; MINB: CTAs per SM
-// the registers must allow (small supports want many).
-template <int PB, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_ols_mixed(OlsArgs a)
+// Tests of one refinement step on dmx = max |correction|, xmx = max |x| (FP32 is enough for
+// them).  Converged: the correction is at the level of FP64 rounding of the residual, or it no
+// longer shrinks (the residual is rounding noise).  1: done, -1: not to be had, 0: go on.
+__device__ __forceinline__ int ols_converged(int itr, float dmx, float xmx, float prev)
 {
+    if (itr > 0 && (dmx <= 1e-14f * xmx || (dmx > 0.5f * prev && dmx <= 1e-12f * xmx))) return 1;
+    if (itr == OLS_REFINE_MAX) return dmx <= 1e-12f * xmx ? 1 : -1;
+    return 0;
+}
+
+// Solves of at most 32 columns, one per warp: lane i holds row i of the swept matrix.
+// Bound by issue slots and the latency of a few hundred dependent steps; a warp per solve keeps
+// 16 or more in flight on an SM, and needs no block barrier.  The line at 32 is the warp's width.
+constexpr int OLS_WARPS = 4;
+struct OlsWarpSmem {
+    int2 xd[32];
+    double xb[32];
+    float buf[2][32];
+    int idx[32];
+};
+__global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    OlsWarpSmem& m = reinterpret_cast<OlsWarpSmem*>(smem_raw)[warp];
+    int2* Gd = reinterpret_cast<int2*>(smem_raw + sizeof(OlsWarpSmem) * OLS_WARPS) + (size_t)warp * a.smax * a.smax;
+    const int64_t wid = (int64_t)blockIdx.x * OLS_WARPS + warp, nwarps = (int64_t)gridDim.x * OLS_WARPS;
+    auto fetch = [&](int64_t t) -> int64_t {
+        if (!a.next) return t < 0 ? wid : t + nwarps;
+        unsigned long long v = 0;
+        if (lane == 0) v = atomicAdd(a.next, 1ull);
+        return (int64_t)__shfl_sync(0xffffffffu, v, 0);
+    };
+    for (int64_t t = fetch(-1); t < a.solves; t = fetch(t)) {
+        const OlsSolve o = ols_solve(a, t);
+        __syncwarp();
+        const int s = warp_support(a.family + ((int64_t)o.j * a.r + o.e) * a.W, a.W, a.p, lane, m.idx, a.smax);
+        if (s < a.s_lo || s > a.smax) continue;
+        const bool in = lane < s;
+        const int my = in ? a.upos[m.idx[lane]] : 0;
+        __syncwarp();
+        m.idx[lane] = my;
+        __syncwarp();
+        const double* Gk = a.Gt + (size_t)o.k * a.pu * a.pu;
+        const double dg = in ? __ldg(Gk + (size_t)my * a.pu + my) : 0.0;
+        const double b = in ? __ldg(a.Bt + ((size_t)o.k * a.pu + my) * a.r + o.e) : 0.0;
+        const uint32_t hg = __reduce_max_sync(0xffffffffu, fx_high(dg));
+        const uint32_t hb = __reduce_max_sync(0xffffffffu, fx_high(b));
+        const int em = fx_exponent(hg), eb = fx_exponent(hb);
+        bool bad = hb >= 0x7FF00000u;                        // Inf or NaN; G's entries at 2^em or above below
+        float g[32];
+        const float unit = __uint_as_float((uint32_t)(127 + 28 - bits) << 23);
+#pragma unroll
+        for (int c0 = 0; c0 < 32; c0 += 8) {
+            if (c0 < s) {
+                double v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    v[i] = in && c0 + i < s ? __ldg(Gk + (size_t)m.idx[c0 + i] * a.pu + my) : 0.0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int2 d = fx_digits(v[i], em, bits);
+                    bad |= (fx_high(v[i]) >> 20) > (hg >> 20) || fx_high(v[i]) >= 0x7FF00000u;
+                    if (in && c0 + i < s) Gd[(c0 + i) * s + lane] = d;
+                    g[c0 + i] = (float)d.x * unit;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) g[c0 + i] = 0.f;
+            }
+        }
+        bool ok = !__any_sync(0xffffffffu, bad);
+        float dmax = 0.f;
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+            if (lane == c) dmax = g[c];
+        dmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(dmax, 0.f))));
+        const float thr = OLS_F32_PIVOT * dmax;
+        // sweep of column c: g_ij -= g_ic g_cj / d, row and column c times 1 / d, g_cc = -1 / d.
+        // Row c is column c (symmetry), and in lane c the same update with 1 - 1/d for g_ic / d
+        // leaves g_cj / d.
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+            if (c < s && ok) {                               // the same in every lane
+                const float d = __shfl_sync(0xffffffffu, g[c], c);
+                if (!(d > thr)) ok = false;
+                else {
+                    float* row = m.buf[c & 1];
+                    row[lane] = g[c];
+                    __syncwarp();
+                    const float inv = __frcp_rn(d), q = g[c] * inv;
+                    const float f = lane == c ? 1.f - inv : q;
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4)
+                        if (j < s) {
+                            const float4 r = *reinterpret_cast<const float4*>(row + j);
+                            g[j] -= f * r.x; g[j + 1] -= f * r.y; g[j + 2] -= f * r.z; g[j + 3] -= f * r.w;
+                        }
+                    g[c] = lane == c ? -inv : q;
+                }
+            }
+        }
+        const double bs = b * fx_pow2(-eb);                  // x comes out times 2^(em - eb)
+        double x = 0.0;
+        bool done = false;
+        if (ok) {
+            float w = f64_to_f32_int(bs), prev = 0.f;
+            for (int itr = 0; itr <= OLS_REFINE_MAX; ++itr) {
+                __syncwarp();
+                m.buf[0][lane] = w;
+                __syncwarp();
+                float y0 = 0.f, y1 = 0.f;
+#pragma unroll
+                for (int c = 0; c < 32; c += 4)
+                    if (c < s) {
+                        const float4 r = *reinterpret_cast<const float4*>(m.buf[0] + c);
+                        y0 += g[c] * r.x; y1 += g[c + 1] * r.y; y0 += g[c + 2] * r.z; y1 += g[c + 3] * r.w;
+                    }
+                const float y = -(y0 + y1);
+                x += (double)y;
+                const uint32_t hx = __reduce_max_sync(0xffffffffu, fx_high(x));
+                const float dmx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(y))));
+                const float xmx = __uint_as_float(
+                    __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(f64_to_f32_int(x)))));
+                const int st = ols_converged(itr, dmx, xmx, prev);
+                if (st) { done = st > 0; break; }
+                prev = dmx;
+                const int ev = hx ? fx_exponent(hx) : 0;
+                m.xd[lane] = fx_digits(x, ev, bits);
+                __syncwarp();
+                FxSum sum;
+                if (in)
+#pragma unroll 4
+                    for (int c = 0; c < s; ++c) sum.add(Gd[c * s + lane], m.xd[c]);
+                w = f64_to_f32_int(fma(-fx_pow2(ev - 2 * bits + 56), (double)sum.value(), bs));
+            }
+        }
+        if (s > 0 && !done) {
+            if (lane == 0) a.fb_list[atomicAdd(a.fb_count, 1)] = (int32_t)o.tg;
+            continue;
+        }
+        x = scalbn(x, eb - em);
+        if (a.jstar) {
+            if (in) a.chosen[((size_t)o.k * a.r + o.e) * a.p + a.ucols[my]] = x;
+            continue;
+        }
+        m.xb[lane] = x;
+        __syncwarp();
+        const double* Ge = a.Ge + (size_t)o.k * a.pu * a.pu;
+        double acc = 0.0, part = 0.0;
+        if (in) {
+#pragma unroll 8
+            for (int c = 0; c < s; ++c) acc += __ldg(Ge + (size_t)m.idx[c] * a.pu + my) * m.xb[c];
+            part = x * (acc - 2.0 * a.Be[((size_t)o.k * a.pu + my) * a.r + o.e]);
+        }
+        const double tot = warp_sum(part);
+        if (lane == 0) {
+            a.losses[o.tg] = a.yye[(size_t)o.k * a.r + o.e] + tot;
+            if (a.singular) a.singular[o.tg] = 0;
+        }
+    }
+}
+
+// Solves of at most 16 T columns, one CTA each: thread (ty, tx) holds entries (ty + 16 u,
+// tx + 16 v) of the swept matrix.  One barrier per swept column (column c through two
+// alternating buffers); residuals by threads = (row, part of the columns).  Bound by the s
+// barriers of the sweep (about 200 clocks each at T = 4, 350 at T = 8).  T = 8 ends where the
+// integers of G[S,S] fill an SM's shared memory (128 columns) and the tile its registers.
+template <int T>
+struct OlsBlockSmem {
+    double bs[16 * T], x[16 * T];
+    long long part[256];
+    int2 xd[16 * T];
+    float buf[2][16 * T], w[16 * T], y[16 * T];
+    int idx[16 * T];
+    uint32_t red[3][8];
+    double redd[8];
+    int64_t next;
+    int count;
+};
+template <int T>
+__global__ void __launch_bounds__(256, T == 4 ? 4 : 2) k_ols_block(OlsArgs a)
+{
+    constexpr int R = 16 * T, PARTS = 256 / R;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    OlsBlockSmem<T>& m = *reinterpret_cast<OlsBlockSmem<T>*>(smem_raw);
+    int2* Gd = reinterpret_cast<int2*>(smem_raw + sizeof(OlsBlockSmem<T>));
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tx = tid & 15, ty = tid >> 4;
+    constexpr int bits = 55;                                 // sums of 128 products fit
+    constexpr float unit = 1.f / (float)(1 << (bits - 28));
+    auto fetch = [&](int64_t t) -> int64_t {
+        if (!a.next) return t < 0 ? (int64_t)blockIdx.x : t + gridDim.x;
+        __syncthreads();
+        if (tid == 0) m.next = (int64_t)atomicAdd(a.next, 1ull);
+        __syncthreads();
+        return m.next;
+    };
+    // maxima of up to three words over the block
+    auto block_max3 = [&](uint32_t& p0, uint32_t& p1, uint32_t& p2) {
+        p0 = __reduce_max_sync(0xffffffffu, p0);
+        p1 = __reduce_max_sync(0xffffffffu, p1);
+        p2 = __reduce_max_sync(0xffffffffu, p2);
+        if (lane == 0) { m.red[0][warp] = p0; m.red[1][warp] = p1; m.red[2][warp] = p2; }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            p0 = max(p0, m.red[0][i]);
+            p1 = max(p1, m.red[1][i]);
+            p2 = max(p2, m.red[2][i]);
+        }
+    };
+    for (int64_t t = fetch(-1); t < a.solves; t = fetch(t)) {
+        const OlsSolve o = ols_solve(a, t);
+        __syncthreads();                                     // the last solve's shared memory is free
+        if (warp == 0) {
+            const int c = warp_support(a.family + ((int64_t)o.j * a.r + o.e) * a.W, a.W, a.p, lane, m.idx,
+                                       a.smax);
+            if (lane == 0) m.count = c;
+        }
+        __syncthreads();
+        const int s = m.count;
+        if (s < a.s_lo || s > a.smax) continue;
+        int my = 0;
+        if (tid < s) my = a.upos[m.idx[tid]];
+        __syncthreads();
+        if (tid < s) m.idx[tid] = my;
+        const double* Gk = a.Gt + (size_t)o.k * a.pu * a.pu;
+        const double dg = tid < s ? __ldg(Gk + (size_t)my * a.pu + my) : 0.0;
+        const double b = tid < s ? __ldg(a.Bt + ((size_t)o.k * a.pu + my) * a.r + o.e) : 0.0;
+        uint32_t hg = fx_high(dg), hb = fx_high(b), zero = 0;
+        block_max3(hg, hb, zero);                            // its barrier: idx is complete
+        const int em = fx_exponent(hg), eb = fx_exponent(hb);
+        bool bad = hb >= 0x7FF00000u;
+        for (int c = warp; c < s; c += 8) {
+            const double* row = Gk + (size_t)m.idx[c] * a.pu;
+            double v[R / 32];
+#pragma unroll
+            for (int i = 0; i < R / 32; ++i) v[i] = lane + 32 * i < s ? __ldg(row + m.idx[lane + 32 * i]) : 0.0;
+#pragma unroll
+            for (int i = 0; i < R / 32; ++i) {
+                bad |= (fx_high(v[i]) >> 20) > (hg >> 20) || fx_high(v[i]) >= 0x7FF00000u;
+                if (lane + 32 * i < s) Gd[c * s + lane + 32 * i] = fx_digits(v[i], em, bits);
+            }
+        }
+        const double bs = b * fx_pow2(-eb);
+        if (tid < R) {
+            m.bs[tid] = bs;
+            m.x[tid] = 0.0;
+            m.w[tid] = f64_to_f32_int(bs);                   // zero past s
+            m.xd[tid] = make_int2(0, 0);
+        }
+        bool ok = __syncthreads_or(bad) == 0;
+        float g[T][T];
+#pragma unroll
+        for (int u = 0; u < T; ++u)
+#pragma unroll
+            for (int v = 0; v < T; ++v) {
+                const int i = ty + 16 * u, j = tx + 16 * v;
+                g[u][v] = i < s && j < s ? (float)Gd[j * s + i].x * unit : 0.f;
+            }
+        float dmax = 0.f;
+        for (int c = 0; c < s; ++c) dmax = fmaxf(dmax, (float)Gd[c * s + c].x * unit);
+        const float thr = OLS_F32_PIVOT * dmax;
+#pragma unroll
+        for (int v0 = 0; v0 < T; ++v0) {
+            for (int l = 0; l < 16 && ok; ++l) {
+                const int c = 16 * v0 + l;
+                if (c >= s) break;
+                float* col = m.buf[c & 1];
+                if (tx == l) {
+#pragma unroll
+                    for (int u = 0; u < T; ++u) col[ty + 16 * u] = g[u][v0];
+                }
+                __syncthreads();
+                const float d = col[c];
+                if (!(d > thr)) { ok = false; break; }
+                const float inv = __frcp_rn(d);
+                float r[T], f[T];
+#pragma unroll
+                for (int v = 0; v < T; ++v) r[v] = col[tx + 16 * v];
+#pragma unroll
+                for (int u = 0; u < T; ++u) {
+                    const float q = col[ty + 16 * u] * inv;
+                    f[u] = ty + 16 * u == c ? 1.f - inv : q;
+#pragma unroll
+                    for (int v = 0; v < T; ++v) g[u][v] -= f[u] * r[v];
+                    if (tx == l) g[u][v0] = ty + 16 * u == c ? -inv : q;
+                }
+            }
+        }
+        bool done = false;
+        double x = 0.0;                                      // threads below s
+        if (ok) {
+            float prev = 0.f;
+            for (int itr = 0; itr <= OLS_REFINE_MAX; ++itr) {
+                __syncthreads();                             // w
+                float r[T];
+#pragma unroll
+                for (int v = 0; v < T; ++v) r[v] = m.w[tx + 16 * v];
+#pragma unroll
+                for (int u = 0; u < T; ++u) {
+                    float y = 0.f;
+#pragma unroll
+                    for (int v = 0; v < T; ++v) y -= g[u][v] * r[v];
+#pragma unroll
+                    for (int k = 8; k > 0; k >>= 1) y += __shfl_xor_sync(0xffffffffu, y, k);
+                    if (tx == 0) m.y[ty + 16 * u] = y;
+                }
+                __syncthreads();
+                uint32_t hx = 0, hd = 0, hm = 0;
+                if (tid < s) {
+                    const float y = m.y[tid];
+                    x += (double)y;
+                    hx = fx_high(x);
+                    hd = __float_as_uint(fabsf(y));
+                    hm = __float_as_uint(fabsf(f64_to_f32_int(x)));
+                }
+                block_max3(hx, hd, hm);
+                const float dmx = __uint_as_float(hd);
+                const int st = ols_converged(itr, dmx, __uint_as_float(hm), prev);
+                if (st) { done = st > 0; break; }
+                prev = dmx;
+                const int ev = hx ? fx_exponent(hx) : 0;
+                if (tid < s) m.xd[tid] = fx_digits(x, ev, bits);
+                __syncthreads();
+                const int row = tid % R, part = tid / R;
+                if (row < s) {
+                    FxSum sum;
+#pragma unroll 4
+                    for (int c = part; c < s; c += PARTS) sum.add(Gd[c * s + row], m.xd[c]);
+                    m.part[tid] = sum.value();
+                }
+                __syncthreads();
+                if (tid < s) {
+                    long long q = 0;
+#pragma unroll
+                    for (int k = 0; k < PARTS; ++k) q += m.part[k * R + tid];
+                    m.w[tid] = f64_to_f32_int(fma(-fx_pow2(ev - 2 * bits + 56), (double)q, m.bs[tid]));
+                }
+            }
+        }
+        if (!done) {                                         // s >= s_lo > 0
+            if (tid == 0) a.fb_list[atomicAdd(a.fb_count, 1)] = (int32_t)o.tg;
+            continue;
+        }
+        x = scalbn(x, eb - em);
+        if (a.jstar) {
+            if (tid < s) a.chosen[((size_t)o.k * a.r + o.e) * a.p + a.ucols[my]] = x;
+            continue;
+        }
+        if (tid < s) m.x[tid] = x;
+        __syncthreads();
+        // x' Ge x - 2 x' be
+        const double* Ge = a.Ge + (size_t)o.k * a.pu * a.pu;
+        double part = tid < s ? -2.0 * x * a.Be[((size_t)o.k * a.pu + my) * a.r + o.e] : 0.0;
+        const int row = tid % R;
+        if (row < s) {
+            const int col = m.idx[row];
+            double acc = 0.0;
+#pragma unroll 8
+            for (int c = tid / R; c < s; c += PARTS) acc += __ldg(Ge + (size_t)m.idx[c] * a.pu + col) * m.x[c];
+            part += m.x[row] * acc;
+        }
+        part = warp_sum(part);
+        if (lane == 0) m.redd[warp] = part;
+        __syncthreads();
+        if (tid == 0) {
+            double tot = 0.0;
+            for (int w = 0; w < 8; ++w) tot += m.redd[w];
+            a.losses[o.tg] = a.yye[(size_t)o.k * a.r + o.e] + tot;
+            if (a.singular) a.singular[o.tg] = 0;
+        }
+    }
+}
+
+// Supports of more than 128 columns: packed FP32 Cholesky factor.
+__global__ void __launch_bounds__(256) k_ols_mixed(OlsArgs a)
+{
+    constexpr int PB = 8;                               // k chunk of the trailing update's register tiles
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int sm2 = (a.smax + 1) & ~1;
     int* idx = reinterpret_cast<int*>(smem_raw);                        // smax ints
@@ -333,32 +762,18 @@ __global__ void __launch_bounds__(256, MINB) k_ols_mixed(OlsArgs a)
     };
 
     for (int64_t t = fetch(-1); t < a.solves; t = fetch(t)) {
-        int k, j, e;
-        if (a.jstar) { k = (int)(t / a.r); e = (int)(t % a.r); j = a.jstar[k]; }
-        else if (a.je_list) {
-            int32_t je;
-            if (a.next) { k = (int)(t % a.B2); je = a.je_list[t / a.B2]; }
-            else { k = (int)(t / a.n_je); je = a.je_list[t % a.n_je]; }
-            j = (int)(je / a.r); e = (int)(je % a.r);
-        } else { k = (int)(t / ((int64_t)a.q * a.r)); const int64_t rem = t % ((int64_t)a.q * a.r);
-               j = (int)(rem / a.r); e = (int)(rem % a.r);
-               if (a.dup && a.dup[rem] != j) continue; }
-        // the solve's index in the numbering of k_ols (for the FP64 hand-over)
-        const int64_t tg = a.jstar ? t : ((int64_t)k * a.q + j) * a.r + e;
-        const uint64_t* bits = a.family + ((int64_t)j * a.r + e) * a.W;
+        const OlsSolve o = ols_solve(a, t);
+        const int k = o.k, j = o.j, e = o.e;
+        const int64_t tg = o.tg;
         if (warp == 0) {
-            int cnt = 0;
-            for (int64_t i0 = 0; i0 < a.p; i0 += 32) {
-                const int64_t i = i0 + lane;
-                const bool in = i < a.p && ((bits[i >> 6] >> (i & 63)) & 1ull);
-                const unsigned bal = __ballot_sync(0xffffffffu, in);
-                if (in) idx[cnt + __popc(bal & ((1u << lane) - 1u))] = a.upos[i];
-                cnt += __popc(bal);
-            }
-            if (lane == 0) s_count = cnt;
+            const int c = warp_support(a.family + ((int64_t)j * a.r + e) * a.W, a.W, a.p, lane, idx, a.smax);
+            if (lane == 0) s_count = c;
         }
         __syncthreads();
         const int s = s_count;
+        if (s < a.s_lo || s > a.smax) { __syncthreads(); continue; }
+        for (int x = threadIdx.x; x < s; x += blockDim.x) idx[x] = a.upos[idx[x]];
+        __syncthreads();
         const double* Gk = a.Gt + (size_t)k * a.pu * a.pu;
         const double* Bk = a.Bt + (size_t)k * a.pu * a.r;
         // gather the packed lower triangle in FP32, b in FP64
@@ -638,38 +1053,112 @@ __global__ void k_support_max(const uint64_t* fam, int64_t count, int W, int32_t
     }
 }
 
+// Lane = lambda, each adding its responses in order; ties go to the smallest j.
 __global__ void k_argmin(const double* losses, int32_t q, int64_t r, int32_t* jstar)
 {
-    const int k = blockIdx.x;
-    if (threadIdx.x != 0) return;
-    int best = 0;
+    const int k = blockIdx.x, lane = threadIdx.x;
+    int best = 0x7fffffff;
     double bv = 0.0;
-    for (int j = 0; j < q; ++j) {
+    bool nan0 = false;
+    for (int j = lane; j < q; j += 32) {
         double s = 0.0;
+#pragma unroll 8
         for (int64_t e = 0; e < r; ++e) s += losses[((int64_t)k * q + j) * r + e];
-        if (j == 0 || s < bv) { bv = s; best = j; }
+        if (j == 0) nan0 = s != s;
+        if (s == s && (best == 0x7fffffff || s < bv)) { bv = s; best = j; }
     }
-    jstar[k] = best;
+    // a NaN at j = 0 is never improved on, one at a later j never chosen
+    nan0 = __shfl_sync(0xffffffffu, nan0 ? 1 : 0, 0) != 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        if (ob != 0x7fffffff && (best == 0x7fffffff || ov < bv || (ov == bv && ob < best))) { bv = ov; best = ob; }
+    }
+    if (nan0) best = 0;
+    if (lane == 0) jstar[k] = best;
 }
 
-__global__ void k_bagging(const double* chosen, int32_t B2, int64_t count, int32_t mode, double* out)
+__device__ void bag_sorted(double* v, int n, double* out)    // by insertion, in place
 {
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < count;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        if (mode == UOI_BAG_MEAN) {
+    for (int k = 1; k < n; ++k) {
+        const double x = v[k * 33];
+        int t = k;
+        while (t > 0 && v[(t - 1) * 33] > x) { v[t * 33] = v[(t - 1) * 33]; --t; }
+        v[t * 33] = x;
+    }
+    *out = (n & 1) ? v[n / 2 * 33] : 0.5 * (v[(n / 2 - 1) * 33] + v[n / 2 * 33]);
+}
+
+// Mean: one thread per coefficient.  Median: 32 coefficients per CTA through shared memory,
+// a warp per coefficient; each lane holds up to four of the B2 <= 128 values and counts those
+// before them (by value, then by bootstrap) on integer keys that order as the values do.
+__global__ void __launch_bounds__(256) k_bagging(const double* chosen, int32_t B2, int64_t count, int32_t mode,
+                                                 double* out)
+{
+    if (mode == UOI_BAG_MEAN) {
+        for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < count;
+             c += (int64_t)gridDim.x * blockDim.x) {
             double s = 0.0;
             for (int k = 0; k < B2; ++k) s += chosen[(int64_t)k * count + c];
             out[c] = s / (double)B2;
-        } else {
-            double v[128];
-            const int n = B2 < 128 ? B2 : 128;
-            for (int k = 0; k < n; ++k) {            // insertion sort
-                const double x = chosen[(int64_t)k * count + c];
-                int t = k;
-                while (t > 0 && v[t - 1] > x) { v[t] = v[t - 1]; --t; }
-                v[t] = x;
+        }
+        return;
+    }
+    __shared__ double v[128 * 33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = B2 < 128 ? B2 : 128;
+    for (int64_t c0 = blockIdx.x * (int64_t)32; c0 < count; c0 += (int64_t)gridDim.x * 32) {
+        __syncthreads();
+        for (int k = warp; k < n; k += 8)
+            if (c0 + lane < count) v[k * 33 + lane] = chosen[(int64_t)k * count + c0 + lane];
+        __syncthreads();
+        for (int i = warp; i < 32 && c0 + i < count; i += 8) {
+            double x[4];
+            long long key[4];
+            bool zero = true, nan = false;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = lane + 32 * u;
+                x[u] = k < n ? v[k * 33 + i] : 0.0;
+                const long long b = __double_as_longlong(x[u]), mag = b & 0x7FFFFFFFFFFFFFFFll;
+                zero &= b == 0;
+                nan |= mag > 0x7FF0000000000000ll;
+                key[u] = b < 0 ? -mag : mag;
             }
-            out[c] = (n & 1) ? v[n / 2] : 0.5 * (v[n / 2 - 1] + v[n / 2]);
+            if (__all_sync(0xffffffffu, zero)) {             // outside every chosen support
+                if (lane == 0) out[c0 + i] = 0.0;
+                continue;
+            }
+            if (__any_sync(0xffffffffu, nan)) {
+                if (lane == 0) bag_sorted(v + i, n, out + c0 + i);
+                continue;
+            }
+            int before[4] = { 0, 0, 0, 0 };
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const int m = min(32, n - 32 * w);
+                for (int l = 0; l < m; ++l) {
+                    const long long o = __shfl_sync(0xffffffffu, key[w], l);
+                    const int k = 32 * w + l;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (32 * u < n) before[u] += o < key[u] || (o == key[u] && k < lane + 32 * u) ? 1 : 0;
+                }
+            }
+            // the values of rank n / 2 and n / 2 - 1, each held by one lane
+            double hi = 0.0, lo = 0.0;
+            bool has_hi = false, has_lo = false;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (lane + 32 * u >= n) continue;
+                if (before[u] == n / 2) { hi = x[u]; has_hi = true; }
+                if (before[u] == n / 2 - 1) { lo = x[u]; has_lo = true; }
+            }
+            const unsigned bh = __ballot_sync(0xffffffffu, has_hi), bl = __ballot_sync(0xffffffffu, has_lo);
+            hi = __shfl_sync(0xffffffffu, hi, __ffs(bh) - 1);
+            if (!(n & 1)) hi = 0.5 * (__shfl_sync(0xffffffffu, lo, __ffs(bl) - 1) + hi);
+            if (lane == 0) out[c0 + i] = hi;
         }
     }
 }
@@ -718,108 +1207,128 @@ void launch_ols_fp64(OlsArgs a, cudaStream_t s)
     }
 }
 
-// Mixed pass: FP32 factor + FP64 refinement for every solve (ols_mixed_start,
-// asynchronous on s), then the FP64 kernel for the solves it handed back
-// (ols_mixed_finish, which waits for the count).
-struct OlsMixedRun {
-    OlsArgs a{};                  // solves = 0 until started: finish does nothing
-    DevBuf fscratch, fbl, fbc;
-};
-
-void ols_mixed_start(OlsArgs a, cudaStream_t s, OlsMixedRun& R)
+// Mixed pass: launches the kernel of class `cls` (OLS_CLASS_MAX) over a.solves; those it hands
+// back go to a.fb_list.
+void launch_ols_class(OlsArgs a, int cls, DevBuf& fscratch, cudaStream_t s)
 {
-    R.a = a;
     if (a.solves == 0) return;
-    const int sm2 = (a.smax + 1) & ~1;
-    const size_t base = sizeof(int) * sm2 + 2 * sizeof(double) * sm2 + 32 * sizeof(double) +
-                        2 * sizeof(float) * sm2;
-    const size_t lbytes = sizeof(float) * (size_t)a.smax * (a.smax + 1) / 2;
-    const size_t cap = 227 * 1024 - 64;
-    const bool in_smem = base + lbytes <= cap;
-    const size_t smem = base + (in_smem ? lbytes : 0);
-    // small supports: narrow panels and few registers, many CTAs per SM (their
-    // steps are short and latency-bound); large ones: wide register tiles
-    const bool small = a.smax <= OLS_SMALL;
-    const void* kern = small ? (const void*)k_ols_mixed<2, 4> : (const void*)k_ols_mixed<8, 1>;
-    allow_max_dynamic_smem(kern);
-    int dev = 0, nsm = 0, per = 0;
+    a.s_lo = cls == 0 ? 0 : OLS_CLASS_MAX[cls - 1] + 1;
+    a.smax = std::max(1, std::min(a.smax, OLS_CLASS_MAX[cls]));
+    int dev = 0, nsm = 0, per = 0, threads = 256;
     UOI_CUDA(cudaGetDevice(&dev));
     UOI_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    UOI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 256, smem));
-    const int grid = (int)std::min<int64_t>(a.solves, (int64_t)nsm * std::max(1, per));
-    if (!in_smem) {
-        R.fscratch.alloc(lbytes * (size_t)grid, s);
-        R.a.fscratch = R.fscratch.as<float>();
+    const void* kern;
+    size_t smem;
+    int64_t work = a.solves;
+    const size_t digits = sizeof(int2) * (size_t)a.smax * a.smax;
+    if (cls == 0) {
+        kern = (const void*)k_ols_warp;
+        threads = 32 * OLS_WARPS;
+        smem = OLS_WARPS * (sizeof(OlsWarpSmem) + digits);
+        work = ceil_div(a.solves, OLS_WARPS);
+    } else if (cls == 1) {
+        kern = (const void*)k_ols_block<4>;
+        smem = sizeof(OlsBlockSmem<4>) + digits;
+    } else if (cls == 2) {
+        kern = (const void*)k_ols_block<8>;
+        smem = sizeof(OlsBlockSmem<8>) + digits;
+    } else {
+        kern = (const void*)k_ols_mixed;
+        const int sm2 = (a.smax + 1) & ~1;
+        const size_t base = sizeof(int) * sm2 + 2 * sizeof(double) * sm2 + 32 * sizeof(double) +
+                            2 * sizeof(float) * sm2;
+        const size_t lbytes = sizeof(float) * (size_t)a.smax * (a.smax + 1) / 2;
+        const bool in_smem = base + lbytes <= 227 * 1024 - 64;
+        smem = base + (in_smem ? lbytes : 0);
+        if (!in_smem) {
+            allow_max_dynamic_smem(kern);
+            UOI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem));
+            fscratch.alloc(lbytes * (size_t)std::min<int64_t>(work, (int64_t)nsm * std::max(1, per)), s);
+            a.fscratch = fscratch.as<float>();
+        }
     }
-    R.fbl.alloc(sizeof(int32_t) * (size_t)std::max<int64_t>(a.solves, (int64_t)a.B2 * a.q * a.r), s);
-    R.fbc.alloc(sizeof(int32_t), s);
-    UOI_CUDA(cudaMemsetAsync(R.fbc.ptr, 0, sizeof(int32_t), s));
-    R.a.fb_list = R.fbl.as<int32_t>();
-    R.a.fb_count = R.fbc.as<int32_t>();
-    if (small) k_ols_mixed<2, 4><<<grid, 256, smem, s>>>(R.a);
-    else k_ols_mixed<8, 1><<<grid, 256, smem, s>>>(R.a);
+    allow_max_dynamic_smem(kern);
+    UOI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem));
+    const int grid = (int)std::min<int64_t>(work, (int64_t)nsm * std::max(1, per));
+    if (cls == 0) k_ols_warp<<<grid, threads, smem, s>>>(a, fx_bits(32));
+    else if (cls == 1) k_ols_block<4><<<grid, threads, smem, s>>>(a);
+    else if (cls == 2) k_ols_block<8><<<grid, threads, smem, s>>>(a);
+    else k_ols_mixed<<<grid, threads, smem, s>>>(a);
     UOI_CHECK_LAUNCH();
     count_launch();
 }
 
-int64_t ols_mixed_finish(OlsMixedRun& R, cudaStream_t s)
+// Work on `side` between the constructor and done() follows what s has queued and precedes
+// what s queues afterwards (also when an exception leaves the scope: the buffers go back to
+// their pool in the order of s).
+struct SideJoin {
+    cudaStream_t side, s;
+    cudaEvent_t ev = nullptr;
+    SideJoin(cudaStream_t side_, cudaStream_t s_) : side(side_), s(s_)
+    {
+        if (side == s) return;
+        UOI_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        UOI_CUDA(cudaEventRecord(ev, s));
+        UOI_CUDA(cudaStreamWaitEvent(side, ev, 0));
+    }
+    SideJoin(const SideJoin&) = delete;
+    SideJoin& operator=(const SideJoin&) = delete;
+    void done()
+    {
+        if (!ev) return;
+        UOI_CUDA(cudaEventRecord(ev, side));
+        UOI_CUDA(cudaStreamWaitEvent(s, ev, 0));
+        cudaEventDestroy(ev);
+        ev = nullptr;
+    }
+    ~SideJoin()
+    {
+        if (!ev) return;
+        if (cudaEventRecord(ev, side) == cudaSuccess) cudaStreamWaitEvent(s, ev, 0);
+        cudaEventDestroy(ev);
+    }
+};
+
+// The FP64 kernel for the solves that the mixed pass handed back (waits for their count).
+int64_t finish_ols(OlsArgs a, int smax, cudaStream_t s)
 {
-    if (R.a.solves == 0) return 0;
     int32_t nfb = 0;
-    UOI_CUDA(cudaMemcpyAsync(&nfb, R.fbc.ptr, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    UOI_CUDA(cudaMemcpyAsync(&nfb, a.fb_count, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     UOI_CUDA(cudaStreamSynchronize(s));
     if (nfb > 0) {
-        OlsArgs a = R.a;
-        a.list = R.fbl.as<int32_t>();
+        a.smax = smax;
+        a.list = a.fb_list;
         a.solves = nfb;
-        a.fscratch = nullptr;
         launch_ols_fp64(a, s);
     }
     return nfb;
 }
 
-int64_t launch_ols_mixed(OlsArgs a, cudaStream_t s)
+// U = union over (j, e) of the family supports, compacted in increasing order.  One block:
+// every thread ORs one word over its share of the members, then warp 0 lists the set bits.
+constexpr int UNION_WORDS = 1024;
+__global__ void __launch_bounds__(UNION_WORDS) k_union_cols(const uint64_t* fam, int64_t count, int W, int64_t p,
+                                                            int32_t* cols, int32_t* n_out)
 {
-    OlsMixedRun R;
-    ols_mixed_start(a, s, R);
-    return ols_mixed_finish(R, s);
-}
-
-int64_t run_ols(OlsArgs a, cudaStream_t s)
-{
-    a.smax = std::max(1, (int)family_support_max(a, s));
-    if (a.smax > 46000) throw Error(UOI_ERR_UNSUPPORTED, "OLS support larger than 46000 columns");
-    return launch_ols_mixed(a, s);
-}
-
-// U = union over (j, e) of the family supports, compacted in increasing order.
-__global__ void k_union_cols(const uint64_t* fam, int64_t count, int W, int64_t p, int32_t* cols,
-                             int32_t* n_out)
-{
-    __shared__ int base;
-    if (threadIdx.x == 0) base = 0;
-    __syncthreads();
+    __shared__ unsigned long long word[UNION_WORDS];
     const int lane = threadIdx.x & 31;
-    for (int w = 0; w < W; ++w) {
-        // one block: OR of word w over all family members
-        uint64_t acc = 0;
-        for (int64_t t = threadIdx.x; t < count; t += blockDim.x) acc |= fam[t * W + w];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, o);
-        __shared__ uint64_t wred[32];
-        if (lane == 0) wred[threadIdx.x >> 5] = acc;
+    int n = 0;                                               // columns listed so far (warp 0)
+    for (int w0 = 0; w0 < W; w0 += UNION_WORDS) {
+        const int wc = min(W - w0, UNION_WORDS), shares = UNION_WORDS / wc;
+        const int w = threadIdx.x % wc, share = threadIdx.x / wc;
+        word[threadIdx.x] = 0;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            uint64_t u = 0;
-            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) u |= wred[i];
-            for (int b = 0; b < 64; ++b) {
-                const int64_t i = (int64_t)w * 64 + b;
-                if (i < p && ((u >> b) & 1ull)) cols[base++] = (int32_t)i;
-            }
-        }
+        unsigned long long acc = 0;
+        if (share < shares)
+#pragma unroll 4
+            for (int64_t t = share; t < count; t += shares) acc |= fam[t * W + w0 + w];
+        if (acc) atomicOr(&word[w], acc);
+        __syncthreads();
+        if (threadIdx.x < 32)
+            n += warp_support((const uint64_t*)word, wc, p - (int64_t)w0 * 64, lane, cols + n, 0x7fffffff, w0 * 64);
         __syncthreads();
     }
-    if (threadIdx.x == 0) *n_out = base;
+    if (threadIdx.x == 0) *n_out = n;
 }
 
 }  // namespace
@@ -838,7 +1347,7 @@ int32_t union_columns(const uint64_t* family, int64_t count, int64_t p, int32_t*
                       cudaStream_t s)
 {
     DevBuf n(sizeof(int32_t), s);
-    k_union_cols<<<1, 256, 0, s>>>(family, count, (int)((p + 63) / 64), p, cols, n.as<int32_t>());
+    k_union_cols<<<1, UNION_WORDS, 0, s>>>(family, count, (int)((p + 63) / 64), p, cols, n.as<int32_t>());
     UOI_CHECK_LAUNCH();
     count_launch();
     int32_t h = 0;
@@ -948,57 +1457,52 @@ int64_t ols_losses(const double* Gt, const double* Bt, const double* Ge, const d
     UOI_CUDA(cudaMemcpyAsync(hsz.data(), sizes.ptr, sizeof(int32_t) * qr, cudaMemcpyDeviceToHost, s));
     UOI_CUDA(cudaMemcpyAsync(hdup.data(), dup.ptr, sizeof(int32_t) * qr, cudaMemcpyDeviceToHost, s));
     UOI_CUDA(cudaStreamSynchronize(s));
-    std::vector<int32_t> small_je, large_je;
-    int32_t smax_small = 1, smax_large = 1;
+    std::vector<int32_t> lists[OLS_CLASSES];
+    int32_t smax = 1;
     for (int64_t t = 0; t < qr; ++t) {
         if (hdup[t] != (int32_t)(t / r)) continue;
-        if (hsz[t] <= OLS_SMALL) { small_je.push_back((int32_t)t); smax_small = std::max(smax_small, hsz[t]); }
-        else { large_je.push_back((int32_t)t); smax_large = std::max(smax_large, hsz[t]); }
+        int cls = 0;
+        while (hsz[t] > OLS_CLASS_MAX[cls]) ++cls;
+        lists[cls].push_back((int32_t)t);
+        smax = std::max(smax, hsz[t]);
     }
-    if (std::max(smax_small, smax_large) > 46000)
-        throw Error(UOI_ERR_UNSUPPORTED, "OLS support larger than 46000 columns");
-    int64_t nfb = 0;
-    // largest supports first within each class, taken from a counter as CTAs free up
-    // (the factor costs grow as the cube of the support size)
-    auto by_size = [&](int32_t x, int32_t y) { return hsz[(size_t)x] > hsz[(size_t)y]; };
-    std::stable_sort(small_je.begin(), small_je.end(), by_size);
-    std::stable_sort(large_je.begin(), large_je.end(), by_size);
-    DevBuf ctr(sizeof(unsigned long long) * 2, s);
+    if (smax > 46000) throw Error(UOI_ERR_UNSUPPORTED, "OLS support larger than 46000 columns");
+    DevBuf ctr(sizeof(unsigned long long) * OLS_CLASSES, s), fbc(sizeof(int32_t), s);
+    DevBuf fbl(sizeof(int32_t) * (size_t)std::max<int64_t>(a.solves, 1), s);
     UOI_CUDA(cudaMemsetAsync(ctr.ptr, 0, ctr.bytes, s));
-    // the two classes run side by side: the large class on s, the small one on a
+    UOI_CUDA(cudaMemsetAsync(fbc.ptr, 0, fbc.bytes, s));
+    a.fb_list = fbl.as<int32_t>();
+    a.fb_count = fbc.as<int32_t>();
+    // largest supports first within each class, taken from a counter as CTAs or warps
+    // free up (the factor costs grow as the cube of the support size)
+    std::vector<int32_t> order;
+    int64_t start[OLS_CLASSES + 1] = {};
+    int classes = 0, top = 0;
+    for (int cls = 0; cls < OLS_CLASSES; ++cls) {
+        std::stable_sort(lists[cls].begin(), lists[cls].end(),
+                         [&](int32_t x, int32_t y) { return hsz[(size_t)x] > hsz[(size_t)y]; });
+        order.insert(order.end(), lists[cls].begin(), lists[cls].end());
+        start[cls + 1] = (int64_t)order.size();
+        if (!lists[cls].empty()) { ++classes; top = cls; }
+    }
+    DevBuf jl(sizeof(int32_t) * std::max<size_t>(order.size(), 1), s);
+    UOI_CUDA(cudaMemcpyAsync(jl.ptr, order.data(), sizeof(int32_t) * order.size(), cudaMemcpyHostToDevice, s));
+    // the classes run side by side: the one of the largest supports on s, the others on a
     // second stream that starts after everything s has queued so far
-    cudaStream_t side = (small_je.empty() || large_je.empty()) ? s : side_stream();
-    cudaEvent_t ready = nullptr, side_done = nullptr;
-    if (side != s) {
-        UOI_CUDA(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
-        UOI_CUDA(cudaEventCreateWithFlags(&side_done, cudaEventDisableTiming));
-        UOI_CUDA(cudaEventRecord(ready, s));
-        UOI_CUDA(cudaStreamWaitEvent(side, ready, 0));
-    }
-    OlsMixedRun runs[2];
-    DevBuf jl[2];
-    for (int cls = 0; cls < 2; ++cls) {
-        const std::vector<int32_t>& lst = cls == 0 ? small_je : large_je;
-        if (lst.empty()) continue;
-        cudaStream_t cs = cls == 0 ? side : s;
-        jl[cls].alloc(sizeof(int32_t) * lst.size(), cs);
-        UOI_CUDA(cudaMemcpyAsync(jl[cls].ptr, lst.data(), sizeof(int32_t) * lst.size(), cudaMemcpyHostToDevice, cs));
+    DevBuf fscratch;
+    cudaStream_t side = classes < 2 ? s : side_stream();
+    SideJoin join(side, s);
+    for (int cls = OLS_CLASSES - 1; cls >= 0; --cls) {
+        if (lists[cls].empty()) continue;
         OlsArgs b = a;
-        b.je_list = jl[cls].as<int32_t>();
-        b.n_je = (int32_t)lst.size();
+        b.je_list = jl.as<int32_t>() + start[cls];
         b.next = ctr.as<unsigned long long>() + cls;
-        b.solves = (int64_t)B2 * b.n_je;
-        b.smax = cls == 0 ? smax_small : smax_large;
-        ols_mixed_start(b, cs, runs[cls]);
+        b.solves = (int64_t)B2 * (int64_t)lists[cls].size();
+        b.smax = hsz[(size_t)lists[cls][0]];
+        launch_ols_class(b, cls, fscratch, cls == top ? s : side);
     }
-    for (int cls = 1; cls >= 0; --cls) nfb += ols_mixed_finish(runs[cls], cls == 0 ? side : s);
-    if (side != s) {
-        // everything that follows on s (the duplicates' losses, the argmin) sees the side's results
-        UOI_CUDA(cudaEventRecord(side_done, side));
-        UOI_CUDA(cudaStreamWaitEvent(s, side_done, 0));
-        cudaEventDestroy(ready);
-        cudaEventDestroy(side_done);
-    }
+    join.done();
+    const int64_t nfb = finish_ols(a, smax, s);
     const unsigned gf = (unsigned)std::min<int64_t>(ceil_div(a.solves, 256), 4096);
     k_fill_duplicates<<<gf, 256, 0, s>>>(dup.as<int32_t>(), B2, q, r, losses, singular);
     UOI_CHECK_LAUNCH();
@@ -1026,13 +1530,23 @@ int64_t ols_chosen(const double* Gt, const double* Bt, const uint64_t* family, c
     a.p = p; a.r = r; a.q = q; a.B2 = B2; a.W = (int32_t)((p + 63) / 64);
     a.jstar = jstar; a.chosen = chosen;
     a.solves = (int64_t)B2 * r;
-    return run_ols(a, s);
+    const int smax = std::max(1, (int)family_support_max(a, s));
+    if (smax > 46000) throw Error(UOI_ERR_UNSUPPORTED, "OLS support larger than 46000 columns");
+    DevBuf fbl(sizeof(int32_t) * (size_t)a.solves, s), fbc(sizeof(int32_t), s), fscratch;
+    UOI_CUDA(cudaMemsetAsync(fbc.ptr, 0, fbc.bytes, s));
+    a.fb_list = fbl.as<int32_t>();
+    a.fb_count = fbc.as<int32_t>();
+    a.smax = smax;
+    // the sizes of the chosen supports are on the device: each class runs its own and skips the rest
+    for (int cls = 0; cls < OLS_CLASSES && (cls == 0 || smax > OLS_CLASS_MAX[cls - 1]); ++cls)
+        launch_ols_class(a, cls, fscratch, s);
+    return finish_ols(a, smax, s);
 }
 
 void bagging(const double* chosen, int32_t B2, int64_t count, int32_t mode, double* out,
              cudaStream_t s)
 {
-    k_bagging<<<(unsigned)std::min<int64_t>(ceil_div(count, 128), 4096), 128, 0, s>>>(
+    k_bagging<<<(unsigned)std::min<int64_t>(ceil_div(count, 32), 4096), 256, 0, s>>>(
         chosen, B2, count, mode, out);
     UOI_CHECK_LAUNCH();
     count_launch();
