@@ -319,11 +319,15 @@ void selection_admm(int precision, const double* Xd, int64_t ldx, const double* 
     int t0 = tm ? tm->mark() : 0;
     std::optional<NvtxRange> stage;
     stage.emplace("uoi:selection:moments");
-    // mixed form, large p: the block inverse on tensor cores; when nothing but the
+    // mixed form: the block inverse on tensor cores; when nothing but the
     // FP32 system reads G (no intercept elimination, no learned start), the Gram's
     // lower triangle is enough and the system is built from it
+    // (up to 192 columns one CTA inverts a system: 24 systems, factor stage 0.23 -> 0.12 ms
+    // at p = 65, 0.31 -> 0.14 at 128, 0.45 -> 0.33 at 192, the same errors; between them the
+    // block recursion would be quicker too, 0.74 -> 0.55 at 301, but its products lose a
+    // little to the FP32 factor)
     bool tc_inverse = false;
-    if constexpr (sizeof(T) == 4) tc_inverse = p >= 512 && inverse_tc_available();
+    if constexpr (sizeof(T) == 4) tc_inverse = (p <= 192 || p >= 512) && inverse_tc_available();
     const bool lower_only = tc_inverse && !icpt && !ws && precision == UOI_PREC_MIXED && gram_tc_available();
     DevBuf G(sizeof(double) * (size_t)(B * p * p), s), Bm(sizeof(double) * (size_t)(B * p * r), s);
     DevBuf nk(sizeof(double) * B, s);
@@ -354,20 +358,45 @@ void selection_admm(int precision, const double* Xd, int64_t ldx, const double* 
     DevBuf A(sizeof(T) * (size_t)(B * p * p), s);
     DevBuf M(sizeof(T) * (size_t)(B * p * p), s);
     DevBuf c(sizeof(T) * (size_t)(B * p * r), s);
+    bool inverted = false;
     if constexpr (sizeof(T) == 4) {
-        // mixed form, large p: block inverse with tensor-core GEMMs
+        // mixed form: block inverse with tensor-core GEMMs
         if (tc_inverse) {
-            if (lower_only)
-                build_system_lower(G.as<double>(), nk.as<double>(), rho, p, B, A.as<float>(), s);
-            else
-                build_system<float>(G.as<double>(), nk.as<double>(), rho, p, B, A.as<float>(), s);
-            if (!ws) G.release();
+            auto build = [&] {
+                if (lower_only)
+                    build_system_lower(G.as<double>(), nk.as<double>(), rho, p, B, A.as<float>(), s);
+                else
+                    build_system<float>(G.as<double>(), nk.as<double>(), rho, p, B, A.as<float>(), s);
+            };
+            build();
             spd_inverse_tc(A.as<float>(), p, B, M.as<float>(), st.as<DevStatus>(), s);
-            check_status(st.as<DevStatus>(), s, "inverse of G/n + rho I");
+            DevStatus h{};
+            UOI_CUDA(cudaMemcpyAsync(&h, st.ptr, sizeof(h), cudaMemcpyDeviceToHost, s));
+            UOI_CUDA(cudaStreamSynchronize(s));
+            if (h.code != 0 && p < 512) {
+                // a system at the edge of FP32: the Cholesky factor decides
+                UOI_CUDA(cudaMemsetAsync(st.ptr, 0, st.bytes, s));
+                build();
+                cholesky_inplace<float>(A.as<float>(), p, B, st.as<DevStatus>(), s);
+                check_status(st.as<DevStatus>(), s, "Cholesky of G/n + rho I");
+                DevBuf Linv(sizeof(float) * (size_t)(B * p * p), s);
+                spd_inverse_from_factor<float>(A.as<float>(), p, B, Linv.as<float>(), M.as<float>(), s);
+            } else if (h.code != 0) {
+                check_status(st.as<DevStatus>(), s, "inverse of G/n + rho I");
+            }
+            if (!ws) G.release();
             rhs_from_inverse<float>(M.as<float>(), Bm.as<double>(), nk.as<double>(), p, r, B, c.as<float>(), s);
+            inverted = true;
         }
     }
-    if (!tc_inverse) {
+    if constexpr (sizeof(T) == 8) {
+        if (inverse_newton(G.as<double>(), nk.as<double>(), rho, p, B, A.as<double>(), M.as<double>(), s)) {
+            rhs_from_inverse<double>(M.as<double>(), Bm.as<double>(), nk.as<double>(), p, r, B, c.as<double>(), s);
+            if (!ws) G.release();
+            inverted = true;
+        }
+    }
+    if (!inverted) {
         build_and_factor<T>(G.as<double>(), nk.as<double>(), rho, p, B, A.as<T>(), st.as<DevStatus>(), s);
         if (!ws) G.release();
         check_status(st.as<DevStatus>(), s, "Cholesky of G/n + rho I");
@@ -1155,13 +1184,17 @@ int uoi_ws_dataset(const double* X, const double* Y, int64_t n, int64_t p, int64
         weight_sums(wd, nullptr, n, B, nk.as<double>(), s);
         DevBuf st(sizeof(DevStatus), s);
         UOI_CUDA(cudaMemsetAsync(st.ptr, 0, st.bytes, s));
-        build_and_factor<double>(G.as<double>(), nk.as<double>(), rho, p, B, A.as<double>(),
-                                 st.as<DevStatus>(), s);
-        check_status(st.as<DevStatus>(), s, "Cholesky of G/n + rho I");
-        DevBuf Linv(sizeof(double) * (size_t)(B * p * p), s), M(sizeof(double) * (size_t)(B * p * p), s);
-        DevBuf c(sizeof(double) * (size_t)(B * p * r), s);
-        inverse_and_rhs<double>(A.as<double>(), Bm.as<double>(), nk.as<double>(), p, r, B,
-                                Linv.as<double>(), M.as<double>(), c.as<double>(), s);
+        DevBuf M(sizeof(double) * (size_t)(B * p * p), s), c(sizeof(double) * (size_t)(B * p * r), s);
+        if (inverse_newton(G.as<double>(), nk.as<double>(), rho, p, B, A.as<double>(), M.as<double>(), s)) {
+            rhs_from_inverse<double>(M.as<double>(), Bm.as<double>(), nk.as<double>(), p, r, B, c.as<double>(), s);
+        } else {
+            build_and_factor<double>(G.as<double>(), nk.as<double>(), rho, p, B, A.as<double>(),
+                                     st.as<DevStatus>(), s);
+            check_status(st.as<DevStatus>(), s, "Cholesky of G/n + rho I");
+            DevBuf Linv(sizeof(double) * (size_t)(B * p * p), s);
+            inverse_and_rhs<double>(A.as<double>(), Bm.as<double>(), nk.as<double>(), p, r, B,
+                                    Linv.as<double>(), M.as<double>(), c.as<double>(), s);
+        }
         DevBuf zs(sizeof(double) * (size_t)rows, s), us(sizeof(double) * (size_t)rows, s);
         AdmmProblem<double> P;
         P.G = B; P.p = p; P.r = r; P.q = q;

@@ -518,6 +518,8 @@ template void spd_inverse_from_factor<float>(const float*, int64_t, int32_t, flo
                                              cudaStream_t);
 template void rhs_from_inverse<float>(const float*, const double*, const double*, int64_t, int64_t,
                                       int32_t, float*, cudaStream_t, float*);
+template void rhs_from_inverse<double>(const double*, const double*, const double*, int64_t, int64_t,
+                                       int32_t, double*, cudaStream_t, double*);
 template void inverse_and_rhs<double>(const double*, const double*, const double*, int64_t,
                                       int64_t, int32_t, double*, double*, double*, cudaStream_t, double*);
 template void inverse_and_rhs<float>(const float*, const double*, const double*, int64_t,

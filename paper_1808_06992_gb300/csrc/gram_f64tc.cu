@@ -77,12 +77,14 @@ struct OzArgs {
     uint64_t wait_ns = tc::kWaitLimitNs;
 };
 
-// Four consecutive TMEM columns of each of the 7 accumulators (64 columns apart).
-__device__ __forceinline__ void oz_load4(uint32_t taddr, float (&v)[OZ_S][4])
+// Four consecutive TMEM columns of each of the NA accumulators (64 columns apart).
+template <int NA>
+__device__ __forceinline__ void oz_load4(uint32_t taddr, float (&v)[NA][4])
 {
-    uint32_t r[OZ_S][4];
+    uint32_t r[8][4];
+    if constexpr (NA < 8) r[7][0] = r[7][1] = r[7][2] = r[7][3] = 0;
 #pragma unroll
-    for (int o = 0; o < OZ_S; ++o)
+    for (int o = 0; o < NA; ++o)
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                      : "=r"(r[o][0]), "=r"(r[o][1]), "=r"(r[o][2]), "=r"(r[o][3])
                      : "r"(taddr + (uint32_t)(o * OZ_TN)));
@@ -91,9 +93,10 @@ __device__ __forceinline__ void oz_load4(uint32_t taddr, float (&v)[OZ_S][4])
                    "+r"(r[1][2]), "+r"(r[1][3]), "+r"(r[2][0]), "+r"(r[2][1]), "+r"(r[2][2]), "+r"(r[2][3]),
                    "+r"(r[3][0]), "+r"(r[3][1]), "+r"(r[3][2]), "+r"(r[3][3]), "+r"(r[4][0]), "+r"(r[4][1]),
                    "+r"(r[4][2]), "+r"(r[4][3]), "+r"(r[5][0]), "+r"(r[5][1]), "+r"(r[5][2]), "+r"(r[5][3]),
-                   "+r"(r[6][0]), "+r"(r[6][1]), "+r"(r[6][2]), "+r"(r[6][3]));
+                   "+r"(r[6][0]), "+r"(r[6][1]), "+r"(r[6][2]), "+r"(r[6][3]), "+r"(r[7][0]), "+r"(r[7][1]),
+                   "+r"(r[7][2]), "+r"(r[7][3]));
 #pragma unroll
-    for (int o = 0; o < OZ_S; ++o)
+    for (int o = 0; o < NA; ++o)
 #pragma unroll
         for (int t = 0; t < 4; ++t) v[o][t] = __uint_as_float(r[o][t]);
 }
@@ -101,6 +104,8 @@ __device__ __forceinline__ void oz_load4(uint32_t taddr, float (&v)[OZ_S][4])
 // grid (tiles, items, row splits): one tile of one item over a range of its chunks.
 // Warp 0: TMA producer (ring of two stages of 32 rows, all slices of A and of B in one
 // copy each); warp 1: MMA issuer; warps 2-9 drain the accumulators after every chunk.
+// NA orders are kept: 7, or 8 for residuals (T_lo then in units 2^-8 as large).
+template <int NA>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
 k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, OzArgs a)
 {
@@ -178,10 +183,12 @@ k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 #pragma unroll 1
                     for (int u = 0; u < OZ_S; ++u) {
                         const uint64_t A = smem_desc_sw64(st + u * (OZ_TM * OZ_TK * 2)) + adv;
-                        const uint32_t acc = (q > 0 || ks > 0 || u > 0) ? 1u : 0u;
-                        for (int t = 0; t + u < OZ_S; ++t)
+                        // the first product of an order starts its sum: slice 0 of A, slice 1 for order 7
+                        const bool started = q > 0 || ks > 0;
+                        for (int t = 0; t < OZ_S && t + u < NA; ++t)
                             mma_bf16(tmem + (uint32_t)((u + t) * OZ_TN), A,
-                                     smem_desc_sw64(st + OZ_A_BYTES + t * (OZ_TN * OZ_TK * 2)) + adv, idesc, acc);
+                                     smem_desc_sw64(st + OZ_A_BYTES + t * (OZ_TN * OZ_TK * 2)) + adv, idesc,
+                                     started || u > (u + t >= OZ_S ? 1 : 0) ? 1u : 0u);
                     }
                 }
                 mma_commit(&empty_bar[s]);
@@ -210,8 +217,8 @@ k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             const int sh = a.cshift[(int64_t)item * a.max_chunks + c0 + c];
 #pragma unroll
             for (int cb = 0; cb < NCOL; cb += 4) {
-                float v[OZ_S][4];
-                oz_load4(taddr + (uint32_t)cb, v);
+                float v[NA][4];
+                oz_load4<NA>(taddr + (uint32_t)cb, v);
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     // S_0 2^8 + S_1 and S_2 2^8 + S_3 fit 32 bits (|S_o| <= (o + 1) 2^21)
@@ -219,7 +226,9 @@ k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     const int p23 = __float2int_rn(v[2][t]) * 256 + __float2int_rn(v[3][t]);
                     const long long p56 = (long long)__float2int_rn(v[5][t]) * 256 + __float2int_rn(v[6][t]);
                     hi[cb + t] += ((long long)p01 * 65536 + p23) << sh;
-                    lo[cb + t] += ((long long)__float2int_rn(v[4][t]) * 65536 + p56) << sh;
+                    long long p46 = (long long)__float2int_rn(v[4][t]) * 65536 + p56;
+                    if constexpr (NA == 8) p46 = p46 * 256 + __float2int_rn(v[7][t]);
+                    lo[cb + t] += p46 << sh;
                 }
             }
             tc_fence_before();
@@ -399,10 +408,11 @@ __device__ __forceinline__ uint32_t oz_digit(uint32_t word, int byte)
 // Gathers the listed rows, takes their digits and writes them transposed:
 // out[((item * 7 + s) * pz_pad + col) * n_pad + t].  A block covers 128 listed rows x 32
 // columns: rows are read along X's rows, the 56-bit values turned over in shared memory.
+// gsx, gsy: distance of the items' operands (0: all items read the same X and Y).
 constexpr int OZ_LD = OZ_CHUNK + 2;
 __global__ void __launch_bounds__(256)
-k_oz_split(const double* __restrict__ X, int64_t ldx, const double* __restrict__ Y, int64_t ldy, int32_t pz_x,
-           int32_t pz, const int32_t* __restrict__ rows, int64_t cap, const OzItem* items, const uint32_t* cmax,
+k_oz_split(const double* __restrict__ X, int64_t ldx, int64_t gsx, const double* __restrict__ Y, int64_t ldy,
+           int64_t gsy, int32_t pz_x, int32_t pz, const int32_t* __restrict__ rows, int64_t cap, const OzItem* items, const uint32_t* cmax,
            int64_t n_pad, int32_t pz_pad, __nv_bfloat16* out)
 {
     __shared__ long long tile[32][OZ_LD];
@@ -413,6 +423,8 @@ k_oz_split(const double* __restrict__ X, int64_t ldx, const double* __restrict__
     const int c = blockIdx.z * 32 + lane;
     const int e = c < pz ? oz_exponent(cmax[(int64_t)item * pz + c]) : 0;
     const int32_t* rl = rows + (int64_t)item * cap + t0;
+    X += item * gsx;
+    Y += item * gsy;
     double x[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -487,6 +499,69 @@ k_oz_finish(const long long* T, int32_t ntiles, const int32_t* tiles, const uint
     }
 }
 
+// Residuals of approximate inverses: the same products with one pair of square matrices per
+// item (X = A_k, Y = M_k, every row once).  The order 7 is kept too: the products it drops
+// are the largest error of a sum whose terms cancel, and a Newton step cannot go below it
+// (without it c = M b came out at 1.4e-14 for p = 400, with it at the level of b).
+
+// One list of the rows 0 .. n - 1 for every item, and the items' entry counts.
+__global__ void k_oz_all_rows(int32_t n, int32_t n_pad, int32_t B, int32_t* rows, OzItem* items)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < n_pad) rows[t] = t < n ? t : -1;
+    if (t < B) {
+        items[t].weight = (unsigned long long)n;
+        items[t].entries = n_pad;
+    }
+}
+
+// Largest high words of the columns of A_k and of M_k (a slice of the rows per block z).
+__global__ void __launch_bounds__(128)
+k_oz_colmax_pair(const double* __restrict__ A, const double* __restrict__ M, int32_t p, uint32_t* cmax,
+                 int32_t* nonfinite)
+{
+    const int item = blockIdx.y, c = blockIdx.x * 128 + threadIdx.x;
+    if (c >= 2 * p) return;
+    const int r0 = (int)((int64_t)p * blockIdx.z / gridDim.z), r1 = (int)((int64_t)p * (blockIdx.z + 1) / gridDim.z);
+    const double* src = (c < p ? A + c : M + (c - p)) + (int64_t)item * p * p;
+    uint32_t h = 0;
+#pragma unroll 8
+    for (int t = r0; t < r1; ++t) {
+        const double x = __ldg(src + (int64_t)t * p);
+        const uint32_t w = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+        h = max(h, w == 0 && __double2loint(x) != 0 ? 1u : w);
+    }
+    if (h >= 0x7FF00000u) atomicExch(nonfinite, 1);
+    if (h) atomicMax(&cmax[(int64_t)item * 2 * p + c], h);
+}
+
+// R = I - A M in FP32 and the sums of |R| over each row, 64 x 64 at a time (rows of the
+// sums are M's columns).
+__global__ void __launch_bounds__(256)
+k_oz_residual(const long long* T, int32_t ntiles, const int32_t* tiles, const uint32_t* cmax, int32_t p, float* R,
+              float* rowsum)
+{
+    const int item = blockIdx.y;
+    const int ti = tiles[2 * blockIdx.x], tj = tiles[2 * blockIdx.x + 1];
+    const long long* t = T + ((int64_t)item * ntiles + blockIdx.x) * (2 * OZ_TILE) + blockIdx.z * 64;
+    const uint32_t* cm = cmax + (int64_t)item * 2 * p;
+    const int i0 = ti * OZ_TM + blockIdx.z * 64 - p, j0 = tj * OZ_TN;      // column of M, row of A
+    if (i0 + 63 < 0 || i0 >= p) return;
+    for (int x = threadIdx.x; x < 64 * 64; x += 256) {
+        const int i = i0 + (x & 63), j = j0 + (x >> 6);
+        float v = 0.f;
+        if (i >= 0 && i < p && j < p) {
+            const long long hi = t[(int64_t)(x >> 6) * OZ_TM + (x & 63)];
+            const long long lo = t[OZ_TILE + (int64_t)(x >> 6) * OZ_TM + (x & 63)];
+            const int e = oz_exponent(cm[p + i]) + oz_exponent(cm[j]);
+            v = f64_to_f32_int((i == j ? 1.0 : 0.0) - scalbn(fma((double)lo, 0x1p-32, (double)hi), e - 38));
+            R[((int64_t)item * p + j) * p + i] = v;
+        }
+        const float sum = warp_sum(fabsf(v));            // a warp lies within one row
+        if ((threadIdx.x & 31) == 0 && j < p) atomicAdd(&rowsum[(int64_t)item * p + j], sum);
+    }
+}
+
 // Slices of one operand: box of all 7 slices of box_rows columns x 32 sample rows.
 CUtensorMap oz_map(void* base, int64_t n_pad, int64_t pz_pad, int64_t depth, int box_rows)
 {
@@ -503,6 +578,65 @@ CUtensorMap oz_map(void* base, int64_t n_pad, int64_t pz_pad, int64_t depth, int
 }
 
 }  // namespace
+
+// R_k = I - A_k M_k (FP32, p x p each) with FP64-accurate products, and the row sums of
+// |R_k|; flags[0] becomes 1 if an entry is NaN or Inf, flags[1] a pipeline error.
+void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float* R, float* rowsum, int32_t* flags,
+                  cudaStream_t s)
+{
+    const int32_t pz_x = (int32_t)p, pz = 2 * pz_x;
+    const int32_t pz_pad = (int32_t)ceil_div(pz, OZ_TM) * OZ_TM;
+    const int32_t n_pad = (int32_t)ceil_div(p, OZ_CHUNK) * OZ_CHUNK, max_chunks = n_pad / OZ_CHUNK;
+    std::vector<int32_t> tiles;
+    for (int ti = pz_x / OZ_TM; ti * OZ_TM < pz; ++ti)
+        for (int tj = 0; tj * OZ_TN < pz_x; ++tj) { tiles.push_back(ti); tiles.push_back(tj); }
+    const int ntiles = (int)tiles.size() / 2;
+    const size_t per_item = (size_t)OZ_S * pz_pad * n_pad * sizeof(__nv_bfloat16);
+    const size_t t_item = sizeof(long long) * 2 * OZ_TILE * (size_t)ntiles;
+    const int group = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, (8ull << 30) / (per_item + t_item)));
+    DevBuf tl(sizeof(int32_t) * tiles.size(), s), rows(sizeof(int32_t) * (size_t)n_pad, s);
+    DevBuf items(sizeof(OzItem) * (size_t)B, s), cmax(sizeof(uint32_t) * (size_t)B * pz, s);
+    DevBuf cshift(sizeof(int32_t) * (size_t)group * max_chunks, s);
+    DevBuf zt(per_item * group, s), T(t_item * group, s);
+    UOI_CUDA(cudaMemcpyAsync(tl.ptr, tiles.data(), sizeof(int32_t) * tiles.size(), cudaMemcpyHostToDevice, s));
+    UOI_CUDA(cudaMemsetAsync(cmax.ptr, 0, cmax.bytes, s));
+    UOI_CUDA(cudaMemsetAsync(cshift.ptr, 0, cshift.bytes, s));
+    UOI_CUDA(cudaMemsetAsync(rowsum, 0, sizeof(float) * (size_t)(B * p), s));
+    k_oz_all_rows<<<(unsigned)ceil_div(std::max<int64_t>(n_pad, B), 256), 256, 0, s>>>(pz_x, n_pad, B, rows.as<int32_t>(),
+                                                                                      items.as<OzItem>());
+    UOI_CHECK_LAUNCH();
+    UOI_CUDA(cudaFuncSetAttribute(k_gram_f64tc<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
+    for (int b0 = 0; b0 < B; b0 += group) {
+        const int nb = std::min(group, B - b0);
+        const int64_t o = (int64_t)b0 * p * p;
+        uint32_t* cm = cmax.as<uint32_t>() + (int64_t)b0 * pz;
+        const unsigned cb = (unsigned)ceil_div(pz, 128);
+        k_oz_colmax_pair<<<dim3(cb, (unsigned)nb, (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(p, 32), 1216 / (cb * nb)))),
+                           128, 0, s>>>(A + o, M + o, pz_x, cm, flags);
+        UOI_CHECK_LAUNCH();
+        k_oz_split<<<dim3((unsigned)nb, (unsigned)max_chunks, (unsigned)(pz_pad / 32)), 256, 0, s>>>(
+            A + o, p, p * p, M + o, p, p * p, pz_x, pz, rows.as<int32_t>(), 0, items.as<OzItem>(), cm, n_pad, pz_pad,
+            zt.as<__nv_bfloat16>());
+        UOI_CHECK_LAUNCH();
+        const int splits = (int)std::max<int64_t>(
+            1, std::min<int64_t>(max_chunks, 152 / std::max<int64_t>(1, (int64_t)ntiles * nb)));
+        if (splits > 1) UOI_CUDA(cudaMemsetAsync(T.ptr, 0, t_item * nb, s));
+        OzArgs a;
+        a.pz = pz; a.pz_x = pz_x; a.ntiles = ntiles;
+        a.tiles = tl.as<int32_t>(); a.items = items.as<OzItem>();
+        a.cshift = cshift.as<int32_t>(); a.max_chunks = max_chunks;
+        a.T = T.as<long long>(); a.err = flags + 1;
+        k_gram_f64tc<8><<<dim3((unsigned)ntiles, (unsigned)nb, (unsigned)splits), OZ_THREADS, OZ_SMEM, s>>>(
+            oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TM),
+            oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TN), a);
+        UOI_CHECK_LAUNCH();
+        k_oz_residual<<<dim3((unsigned)ntiles, (unsigned)nb, 2), 256, 0, s>>>(T.as<long long>(), ntiles, tl.as<int32_t>(),
+                                                                             cm, pz_x, R + o, rowsum + (int64_t)b0 * p);
+        UOI_CHECK_LAUNCH();
+        count_launch(4);
+    }
+    count_launch();
+}
 
 void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t m, int64_t p, int64_t r,
                  const uint32_t* w, const uint8_t* mask, int32_t B, double* G, double* Bm, int b_only,
@@ -556,7 +690,7 @@ void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int
     const size_t t_item = sizeof(long long) * 2 * OZ_TILE * (size_t)ntiles;
     const int group = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, (16ull << 30) / (per_item + t_item)));
     DevBuf zt(per_item * group, s), T(t_item * group, s);
-    UOI_CUDA(cudaFuncSetAttribute(k_gram_f64tc, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
+    UOI_CUDA(cudaFuncSetAttribute(k_gram_f64tc<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
     for (int b0 = 0; b0 < B; b0 += group) {
         const int nb = std::min(group, B - b0);
         // few tiles: split the rows until every SM has one (integer sums: any split
@@ -564,7 +698,7 @@ void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int
         const int splits = (int)std::max<int64_t>(
             1, std::min<int64_t>(max_chunks, 152 / std::max<int64_t>(1, (int64_t)ntiles * nb)));
         k_oz_split<<<dim3((unsigned)nb, (unsigned)max_chunks, (unsigned)(pz_pad / 32)), 256, 0, s>>>(
-            X, ldx, Y, ldy, pz_x, pz, rows.as<int32_t>() + (int64_t)b0 * n_pad, n_pad, items.as<OzItem>() + b0,
+            X, ldx, 0, Y, ldy, 0, pz_x, pz, rows.as<int32_t>() + (int64_t)b0 * n_pad, n_pad, items.as<OzItem>() + b0,
             cmax.as<uint32_t>() + (int64_t)b0 * pz, n_pad, pz_pad, zt.as<__nv_bfloat16>());
         UOI_CHECK_LAUNCH();
         if (splits > 1) UOI_CUDA(cudaMemsetAsync(T.ptr, 0, t_item * nb, s));
@@ -573,7 +707,7 @@ void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int
         a.tiles = tl.as<int32_t>(); a.items = items.as<OzItem>() + b0;
         a.cshift = cshift.as<int32_t>() + (int64_t)b0 * max_chunks; a.max_chunks = max_chunks;
         a.T = T.as<long long>(); a.err = flags.as<int32_t>() + 1;
-        k_gram_f64tc<<<dim3((unsigned)ntiles, (unsigned)nb, (unsigned)splits), OZ_THREADS, OZ_SMEM, s>>>(
+        k_gram_f64tc<7><<<dim3((unsigned)ntiles, (unsigned)nb, (unsigned)splits), OZ_THREADS, OZ_SMEM, s>>>(
             oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TM),
             oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TN), a);
         UOI_CHECK_LAUNCH();

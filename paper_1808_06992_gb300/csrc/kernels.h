@@ -176,6 +176,16 @@ bool inverse_tc_available();
 void spd_inverse_tc(const float* A, int64_t p, int32_t G, float* M, DevStatus* status, cudaStream_t s);
 // The calling host thread's second stream (estimate.cu).
 cudaStream_t side_stream();
+// M_k = (G_k/n_k + rho I)^{-1} in FP64 accuracy by Newton's iteration from the FP32 inverse
+// (inverse_f64.cu); A: B x p x p scratch.  false (nothing usable in M) when the size is not
+// its own or the iteration does not settle: the caller then takes the FP64 factor.
+constexpr int64_t INVERSE_NEWTON_MIN = 64;
+bool inverse_newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A, double* M,
+                    cudaStream_t s);
+// R_k = I - A_k M_k with FP64-accurate products (gram_f64tc.cu); flags: non-finite entry, error.
+void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float* R, float* rowsum, int32_t* flags,
+                  cudaStream_t s);
+
 // M_k = A_k^{-1} from the factor L (lower triangle of A), then
 // c_k[e][i] = (M_k Bm_k)[i][e] / nk[k].
 template <typename T>
