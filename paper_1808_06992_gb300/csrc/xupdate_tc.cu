@@ -27,7 +27,7 @@
 // Grid: (row tiles of 128, chain tiles of NT <= 64, groups), two CTAs per SM so
 // that one CTA's prologue and epilogue overlap the other's stream of M.  Warp 0:
 // TMA producer (ring of 4 stages of k = 32); warp 1: TMEM allocation and MMA
-// issue; warps 2-5: epilogue (one TMEM lane quarter each).
+// issue; warps 2-9: epilogue (two per TMEM lane quarter, half of the chains each).
 // Waits are bounded (~1 s) and report UOI_ERR_TIMEOUT.
 #include <cuda_fp16.h>
 
@@ -57,8 +57,9 @@ constexpr int XT_STAGES = 4;                           // ring slots
 constexpr int XT_A_BYTES = XT_TM * XT_TK * 2;          // 8 KB per piece
 constexpr int XT_STAGE_MAX = XT_PIECES * XT_A_BYTES + XT_PIECES * XT_NT_MAX * XT_TK * 2;   // 24 KB
 constexpr int XT_SMEM = XT_STAGES * XT_STAGE_MAX + 1024;
-constexpr int XT_THREADS = 192;
-constexpr uint32_t XT_TMEM_COLS = 256;                 // A1[0] at 0, A1[1] at 64, A2 at 128
+constexpr int XT_EPI_WARPS = 8;                        // two per TMEM lane quarter
+constexpr int XT_THREADS = 64 + 32 * XT_EPI_WARPS;
+constexpr uint32_t XT_TMEM_COLS = 256;                 // A1[0] at 0, A1[1] at 64, A2 at 128, folded sums at 192
 constexpr int XT_CHUNK_STAGES = 4;                     // drain h.H every 128 k
 constexpr int XT_SCALE_EXP = 10;                       // scaled magnitudes stay below 2^10
 
@@ -85,12 +86,6 @@ struct XtArgs {
     uint64_t wait_ns = tc::kWaitLimitNs;   // limit of every bounded mbarrier wait
 };
 
-// 4-byte asynchronous copy global -> shared (completion waited for by the issuing thread).
-__device__ __forceinline__ void cp_async4(uint32_t dst, const float* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-
 __device__ __forceinline__ void split2(float x, __half& h, __half& l)
 {
     h = __float2half_rn(x);
@@ -107,12 +102,11 @@ __device__ __forceinline__ float pow2_scale(float bound)
 }
 
 // One CTA of the x-update: row tile rt, chain tile ct of group g, with a ring of
-// STAGES slots (at least 4: the epilogue stages z, u and c in the idle ring).
+// STAGES slots.
 template <int STAGES>
 __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUtensorMap* tmV, const XtArgs& a,
                                              int rt, int ct, int g)
 {
-    static_assert(3 * XT_NT_MAX * XT_TM * 4 <= STAGES * XT_STAGE_MAX, "epilogue staging fits the ring");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ uint64_t full_bar[STAGES], empty_bar[STAGES], accf_bar[2], acce_bar[2], done_bar;
     __shared__ uint32_t tmem_base;
@@ -146,7 +140,7 @@ __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUten
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&accf_bar[b], 1); mbar_init(&acce_bar[b], 128); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&accf_bar[b], 1); mbar_init(&acce_bar[b], 32 * XT_EPI_WARPS); }
         mbar_init(&done_bar, 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -232,12 +226,16 @@ __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUten
         mbar_wait(&done_bar, 0, &dummy, a.wait_ns);
     } else if (warp >= 2) {
         // ---------------- epilogue ----------------
+        // rows of TMEM lane quarter `quad`; the tile's chains are shared by two warps,
+        // columns h0 .. h0 + ncol - 1 (at most 32, a multiple of 8) for this one
         const int quad = warp & 3;
         const int i = i0 + quad * 32 + lane;
+        const int hw = (a.NT / 2 + 7) & ~7, half = (warp - 2) >> 2;
+        const int h0 = half * hw, ncol = min(hw, a.NT - h0);
         const uint32_t lanes = (uint32_t)(quad * 32) << 16;
         {
             // per-chain scalars of the update, read once instead of per row, while the
-            // products run; then a barrier of the four epilogue warps
+            // products run; then a barrier of the epilogue warps
             const int n = threadIdx.x - 64;
             if (n < XT_NT_MAX) {
                 const int chain = n0 + n;
@@ -248,12 +246,12 @@ __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUten
                 s_vw[n] = mine ? a.vs_w[sl] : 0.f;
                 s_coff[n] = g * a.r + (a.warm ? chain : chain % a.r);
             }
-            asm volatile("bar.sync 1, 128;" ::: "memory");
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * XT_EPI_WARPS) : "memory");
         }
         const float rinv_row = i < a.p ? a.row_inv[(int64_t)g * a.ppad + i] : 0.f;
-        float acc[64], cmp[64];
+        float acc[32], cmp[32];
 #pragma unroll
-        for (int t = 0; t < 64; ++t) { acc[t] = 0.f; cmp[t] = 0.f; }
+        for (int t = 0; t < 32; ++t) { acc[t] = 0.f; cmp[t] = 0.f; }
         for (int c = 0; c < nchunks; ++c) {
             const int b = c & 1;
             const bool okw = mbar_wait(&accf_bar[b], (c >> 1) & 1, &abort_flag, a.wait_ns);
@@ -265,16 +263,16 @@ __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUten
             tc_fence_after();
 #pragma unroll
             for (int cb = 0; cb < 2; ++cb) {
-                if (cb * 32 >= a.NT) break;
-                float v[32];
-                tmem_ld32(tmem + lanes + (uint32_t)(b * 64 + cb * 32), v);
+                if (cb * 16 >= ncol) break;
+                float v[16];
+                tmem_ld16(tmem + lanes + (uint32_t)(b * 64 + h0 + cb * 16), v);
 #pragma unroll
-                for (int t = 0; t < 32; ++t) {
-                    const float x = v[t], sa = acc[cb * 32 + t];
+                for (int t = 0; t < 16; ++t) {
+                    const float x = v[t], sa = acc[cb * 16 + t];
                     const float sum = sa + x;
                     const float bv = sum - sa;
-                    cmp[cb * 32 + t] += (sa - (sum - bv)) + (x - bv);
-                    acc[cb * 32 + t] = sum;
+                    cmp[cb * 16 + t] += (sa - (sum - bv)) + (x - bv);
+                    acc[cb * 16 + t] = sum;
                 }
             }
             tc_fence_before();
@@ -282,7 +280,7 @@ __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUten
         }
         // fold the compensation terms (frees their registers for the epilogue)
 #pragma unroll
-        for (int t = 0; t < 64; ++t) acc[t] += cmp[t];
+        for (int t = 0; t < 32; ++t) acc[t] += cmp[t];
         // small products, once all MMAs are done
         {
             int dummy = 0;
@@ -292,52 +290,41 @@ __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUten
         tc_fence_after();
         const bool rowok = i < a.p && !abort_flag;
         const float rinv = rowok ? rinv_row : 0.f;
-        // The ring is idle now: stage this row's z, u and c of every live chain in
-        // it with asynchronous copies, all in flight at once, so the update below
-        // reads shared memory instead of waiting on DRAM once per group of chains.
-        // Each thread copies (and later reads) only its own row: no barrier needed.
-        float* stg = reinterpret_cast<float*>(smem_raw + (sbase - smem_u32(smem_raw)));   // [3][NT][128]
-        const int r128 = quad * 32 + lane;
-        if (rowok) {
-            for (int n = 0; n < a.NT; ++n) {
-                if (!s_live[n]) continue;
-                const int64_t o = ((int64_t)g * a.nchains + n0 + n) * a.p + i;
-                cp_async4(smem_u32(stg + (0 * a.NT + n) * XT_TM + r128), a.z + o);
-                cp_async4(smem_u32(stg + (1 * a.NT + n) * XT_TM + r128), a.u + o);
-                cp_async4(smem_u32(stg + (2 * a.NT + n) * XT_TM + r128), a.c + (int64_t)s_coff[n] * a.p + i);
+        // z, u and c of this row for eight chains, read one group ahead of the update
+        float zp[8], uo[8], cc[8];
+        auto fetch = [&](int nb, float (&z8)[8], float (&u8)[8], float (&c8)[8]) {
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const bool act = rowok && s_live[nb + t];
+                const int64_t o = ((int64_t)g * a.nchains + n0 + nb + t) * a.p + i;
+                z8[t] = act ? a.z[o] : 0.f;
+                u8[t] = act ? a.u[o] : 0.f;
+                c8[t] = act ? __ldg(a.c + (int64_t)s_coff[nb + t] * a.p + i) : 0.f;
             }
-        }
-        // The folded sums go back to TMEM, into the first drain buffer (columns
-        // 0..NT-1, idle once all products are done), so that the update below is a
-        // rolled loop over groups of 8 chains with one copy of its body: each pass
-        // reads 8 columns of h.H and of the small products.
-#pragma unroll
-        for (int cb = 0; cb < 2; ++cb) {
-            if (cb * 32 >= a.NT) break;
-            float w[32];
-#pragma unroll
-            for (int t = 0; t < 32; ++t) w[t] = acc[cb * 32 + t];
-            tmem_st32(tmem + lanes + (uint32_t)(cb * 32), w);
-        }
-        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+        };
+        if (ncol > 0) fetch(h0, zp, uo, cc);
+        // The folded sums go to free TMEM columns (192 + 32 half), so that the update
+        // below is a rolled loop over groups of 8 chains with one copy of its body: each
+        // pass reads 8 columns of h.H and of the small products.
+        const uint32_t fold = tmem + lanes + 192u + (uint32_t)(32 * half);
+        tmem_st32(fold, acc);
 #pragma unroll 1
-        for (int nb = 0; nb < a.NT; nb += 8) {                       // first chain of the group of 8
+        for (int nb = h0; nb < h0 + ncol; nb += 8) {                 // first chain of the group of 8
             float hv[8];                                             // h.H + small products
             {
                 float hh[8], v2[8];
-                tmem_ld8x2(tmem + lanes + (uint32_t)nb, tmem + lanes + (uint32_t)(128 + nb), hh, v2);
+                tmem_ld8x2(fold + (uint32_t)(nb - h0), tmem + lanes + (uint32_t)(128 + nb), hh, v2);
 #pragma unroll
                 for (int t = 0; t < 8; ++t) hv[t] = hh[t] + v2[t];
             }
-            {
-                float zp[8], uo[8], cc[8];
+            float zn8[8], un8[8], cn8[8];
+            if (nb + 8 < h0 + ncol) {
+                fetch(nb + 8, zn8, un8, cn8);
+            } else {
 #pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const bool act = rowok && s_live[nb + t];
-                    zp[t] = act ? stg[(0 * a.NT + nb + t) * XT_TM + r128] : 0.f;
-                    uo[t] = act ? stg[(1 * a.NT + nb + t) * XT_TM + r128] : 0.f;
-                    cc[t] = act ? stg[(2 * a.NT + nb + t) * XT_TM + r128] : 0.f;
-                }
+                for (int t = 0; t < 8; ++t) { zn8[t] = 0.f; un8[t] = 0.f; cn8[t] = 0.f; }
+            }
+            {
                 float pr[5][8];
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
@@ -390,6 +377,8 @@ __device__ __forceinline__ void xupdate_tile(const CUtensorMap* tmM, const CUten
                     if ((lane & 3) == 0) red[quad][nb + b4 * 4 + b3 * 2 + b2][qq] = w2;
                 }
             }
+#pragma unroll
+            for (int t = 0; t < 8; ++t) { zp[t] = zn8[t]; uo[t] = un8[t]; cc[t] = cn8[t]; }
         }
     }
     tc_fence_before();
