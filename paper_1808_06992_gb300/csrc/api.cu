@@ -322,8 +322,8 @@ void selection_admm(int precision, const double* Xd, int64_t ldx, const double* 
     // mixed form: the block inverse on tensor cores; when nothing but the
     // FP32 system reads G (no intercept elimination, no learned start), the Gram's
     // lower triangle is enough and the system is built from it
-    // (up to 192 columns one CTA inverts a system: 24 systems, factor stage 0.23 -> 0.12 ms
-    // at p = 65, 0.31 -> 0.14 at 128, 0.45 -> 0.33 at 192, the same errors; between them the
+    // (up to 192 columns one CTA inverts a system: 24 systems, factor stage 0.23 -> 0.08 ms
+    // at p = 65, 0.31 -> 0.10 at 128, 0.45 -> 0.16 at 192, the same errors; between them the
     // block recursion would be quicker too, 0.74 -> 0.55 at 301, but its products lose a
     // little to the FP32 factor)
     bool tc_inverse = false;

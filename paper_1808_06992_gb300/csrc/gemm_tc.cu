@@ -499,163 +499,99 @@ void gemm3(const Pieces& A, const Pieces& B, int32_t m, int32_t n, int32_t G, fl
     count_launch();
 }
 
-// In-place blocked Gauss-Jordan inverse of one SPD block per CTA (n <= INV_BASE =
-// 192), in steps of 32 pivots (no pivoting: the pivots are Schur-complement
-// diagonals, positive for SPD A).  1024 threads; thread (ty, tx) owns the
-// elements (ty + 32u, tx + 32w), u, w < R, in registers.  Step K works on row and
-// column block K (indices 32K .. 32K + 31):
-//   P = A_KK^{-1}                        (one warp, in registers, by shuffles)
-//   A_KJ <- P A_KJ             (J != K)  (block row K; each warp one of its rows)
-//   A_IJ <- A_IJ - A_IK A_KJ   (I, J != K; A_IK before the step, A_KJ after it)
-//   A_IK <- -A_IK P            (I != K)
-//   A_KK <- P
-// which leaves A^{-1} after the last step (the block form of the pivot-by-pivot
-// Gauss-Jordan elimination: the same products, four barriers per 32 pivots
-// instead of one per pivot).  Rows and columns past n hold zeros and the padded
-// part of the last diagonal block is inverted as the identity, so they never
-// reach the n x n result.  A pivot <= 0 sets status UOI_ERR_NOT_PD (where = g0 + group).
-constexpr int GJ_LD = 33;                              // shared rows: conflict-free columns
-template <int R>
-constexpr size_t gj_smem_bytes() { return sizeof(float) * (size_t)(3 * 32 * R * GJ_LD + 32 * GJ_LD); }
+// Inverse of one SPD block per CTA (n <= INV_BASE = 192) by symmetric Gauss-Jordan sweeps in
+// registers (no pivoting: the pivots are Schur-complement diagonals, positive for SPD A).
+// 256 threads; thread (ty, tx) owns the elements (sweep_index(ty, u), sweep_index(tx, w)),
+// u, w < T.  The sweep of column c,
+//   a_ij -= a_ic a_cj / d,  a_ic = a_ic / d,  a_cj = a_cj / d,  a_cc = -1 / d,   d = a_cc,
+// needs column c alone (row c is its mirror), which its owners put in one of two alternating
+// buffers: one barrier per pivot.  After n sweeps -A^{-1} is left.  Rows and columns past n
+// hold zeros and stay zero.  A pivot <= 0 sets status UOI_ERR_NOT_PD (where = g0 + group).
+//
+// Few blocks are inverted at a time (one per system and chain), so the length of one block's
+// chain counts: 128 pivots of about 270 clocks, of which 130 are the multiply-adds at one warp
+// instruction per clock and scheduler; four consecutive elements per thread make the column a
+// few 16-byte reads.  Against blocked elimination in steps of 32 pivots with 1024 threads
+// (one warp inverts the diagonal block while 31 wait), 24 blocks: n = 128 88 -> 42 us, n = 192
+// 262 -> 94 us; factor stage of 24 systems p = 128 0.14 -> 0.10 ms, p = 192 0.33 -> 0.16 ms.
+__device__ __forceinline__ int sweep_index(int t, int u) { return (u >> 2) * 64 + t * 4 + (u & 3); }
 
-// P = inverse of the bk x bk diagonal block whose row k, column l is at
-// D[k * GJ_LD + l] (identity past bk), by one warp: lane l holds column l in
-// registers and each of the 32 pivots is one round of shuffles.  Returns false
-// when a pivot is not positive.  Not inlined, so that the caller's register tile
-// is saved around it by the one warp that calls it instead of being squeezed.
-__device__ __noinline__ bool gj_invert_diag(const float* D, float* P, int bk)
+template <int T>
+__global__ void __launch_bounds__(256) k_spd_inverse_sweep(const float* A, int64_t lda, int64_t gsa, float* M,
+                                                           int64_t ldm, int64_t gsm, int n, int g0, DevStatus* st)
 {
-    const int tx = threadIdx.x & 31;
-    float d[32];
+    __shared__ __align__(16) float buf[2][16 * T];
+    const int gi = blockIdx.x, tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const float* a = A + (int64_t)gi * gsa;
+    float g[T][T];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) d[k] = (k < bk && tx < bk) ? D[k * GJ_LD + tx] : (k == tx ? 1.f : 0.f);
-    bool ok = true;
+    for (int u = 0; u < T; ++u)
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        const float piv = __shfl_sync(0xffffffffu, d[k], k);
-        ok = ok && piv > 0.f;
-        const float inv = 1.f / piv;
-        const float r = (tx == k) ? inv : d[k] * inv;           // row k / pivot
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const float c = __shfl_sync(0xffffffffu, d[i], k);   // column k
-            d[i] = (i == k) ? r : fmaf(-c, r, tx == k ? 0.f : d[i]);
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 32; ++k) P[k * GJ_LD + tx] = d[k];
-    return ok;
-}
-
-template <int R>
-__global__ void __launch_bounds__(1024) k_spd_inverse_blocked(const float* A, int64_t lda, int64_t gsa,
-                                                              float* M, int64_t ldm, int64_t gsm, int n,
-                                                              int g0, DevStatus* st)
-{
-    extern __shared__ float sm[];
-    float* colK = sm;                           // [32R][LD]: colK[i][k] = A(i, 32K + k) before step K
-    float* rowT = colK + 32 * R * GJ_LD;        // [32R][LD]: rowT[j][k] = A(32K + k, j) before step K
-    float* rowN = rowT + 32 * R * GJ_LD;        // [32R][LD]: rowN[j][k] = (P A_K.)(k, j)
-    float* P = rowN + 32 * R * GJ_LD;           // [32][LD]:  P[k][l] = (A_KK^{-1})(k, l)
-    __shared__ int bad;
-    const int g = blockIdx.x;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const float* a = A + (int64_t)g * gsa;
-    float v[R][R];
-#pragma unroll
-    for (int u = 0; u < R; ++u)
-#pragma unroll
-        for (int w = 0; w < R; ++w) {
-            const int i = ty + 32 * u, j = tx + 32 * w;
-            v[u][w] = (i < n && j < n) ? a[(int64_t)i * lda + j] : 0.f;
-        }
-    if (threadIdx.x == 0) bad = 0;
-    const int nblk = (n + 31) / 32;
-#pragma unroll
-    for (int K = 0; K < R; ++K) {
-        if (K >= nblk) break;
-        __syncthreads();                        // the last step's readers are done
-#pragma unroll
-        for (int u = 0; u < R; ++u) colK[(ty + 32 * u) * GJ_LD + tx] = v[u][K];
-#pragma unroll
-        for (int w = 0; w < R; ++w) rowT[(tx + 32 * w) * GJ_LD + ty] = v[K][w];
-        __syncthreads();
-        if (ty == 0) {
-            const bool ok = gj_invert_diag(colK + 32 * K * GJ_LD, P, min(32, n - 32 * K));
-            if (!ok && tx == 0) bad = 1;
-        }
-        __syncthreads();
-        if (bad) {
-            if (threadIdx.x == 0) dev_fail(st, UOI_ERR_NOT_PD, g0 + g);
-            return;                             // same decision in every thread
-        }
-        // block row K: this warp's row 32K + ty becomes row ty of P A_K.
-#pragma unroll
-        for (int w = 0; w < R; ++w)
-            if (w != K) v[K][w] = 0.f;
-#pragma unroll 2
-        for (int k = 0; k < 32; ++k) {
-            const float pk = P[ty * GJ_LD + k];
-#pragma unroll
-            for (int w = 0; w < R; ++w)
-                if (w != K) v[K][w] = fmaf(pk, rowT[(tx + 32 * w) * GJ_LD + k], v[K][w]);
+        for (int w = 0; w < T; ++w) {
+            const int i = sweep_index(ty, u), j = sweep_index(tx, w);
+            g[u][w] = (i < n && j < n) ? a[(int64_t)i * lda + j] : 0.f;
         }
 #pragma unroll
-        for (int w = 0; w < R; ++w)
-            if (w != K) rowN[(tx + 32 * w) * GJ_LD + ty] = v[K][w];
-        v[K][K] = P[ty * GJ_LD + tx];
-        __syncthreads();
-        // every other block row: A_IJ -= A_IK (P A_KJ), A_IK = -A_IK P
-#pragma unroll
-        for (int u = 0; u < R; ++u)
-            if (u != K) v[u][K] = 0.f;
+    for (int h = 0; h < T / 4; ++h)
 #pragma unroll 1
-        for (int k = 0; k < 32; ++k) {
-            float r[R];
+        for (int o = 0; o < 16; ++o) {
+            if (64 * h + 4 * o >= n) break;
 #pragma unroll
-            for (int w = 0; w < R; ++w)
-                r[w] = (w == K) ? P[k * GJ_LD + tx] : rowN[(tx + 32 * w) * GJ_LD + k];
+            for (int q = 0; q < 4; ++q) {
+                const int c = 64 * h + 4 * o + q, m = 4 * h + q;       // column c: element m of thread column o
+                if (c >= n) break;
+                float* col = buf[q & 1];
+                if (tx == o) {
 #pragma unroll
-            for (int u = 0; u < R; ++u) {
-                if (u == K) continue;
-                const float c = colK[(ty + 32 * u) * GJ_LD + k];
+                    for (int k = 0; k < T / 4; ++k)
+                        *reinterpret_cast<float4*>(col + 64 * k + 4 * ty) =
+                            make_float4(g[4 * k][m], g[4 * k + 1][m], g[4 * k + 2][m], g[4 * k + 3][m]);
+                }
+                __syncthreads();
+                const float d = col[c];
+                if (!(d > 0.f)) {                                      // the same in every thread
+                    if (threadIdx.x == 0) dev_fail(st, UOI_ERR_NOT_PD, g0 + gi);
+                    return;
+                }
+                const float inv = 1.f / d;
+                float r[T], f[T];
 #pragma unroll
-                for (int w = 0; w < R; ++w) v[u][w] = fmaf(-c, r[w], v[u][w]);
+                for (int k = 0; k < T / 4; ++k) {
+                    const float4 x = *reinterpret_cast<const float4*>(col + 64 * k + 4 * tx);
+                    const float4 y = *reinterpret_cast<const float4*>(col + 64 * k + 4 * ty);
+                    r[4 * k] = x.x; r[4 * k + 1] = x.y; r[4 * k + 2] = x.z; r[4 * k + 3] = x.w;
+                    f[4 * k] = y.x * inv; f[4 * k + 1] = y.y * inv; f[4 * k + 2] = y.z * inv; f[4 * k + 3] = y.w * inv;
+                }
+                const bool myrow = ty == o;
+#pragma unroll
+                for (int u = 0; u < T; ++u) {
+                    if (u == m) {
+                        const float fu = myrow ? -inv : f[u];
+#pragma unroll
+                        for (int w = 0; w < T; ++w) g[u][w] = fmaf(-fu, r[w], myrow ? 0.f : g[u][w]);
+                    } else {
+#pragma unroll
+                        for (int w = 0; w < T; ++w) g[u][w] = fmaf(-f[u], r[w], g[u][w]);
+                    }
+                    if (tx == o) g[u][m] = u == m && myrow ? -inv : f[u];
+                }
             }
         }
-    }
-    float* mo = M + (int64_t)g * gsm;
+    float* mo = M + (int64_t)gi * gsm;
 #pragma unroll
-    for (int u = 0; u < R; ++u)
+    for (int u = 0; u < T; ++u)
 #pragma unroll
-        for (int w = 0; w < R; ++w) {
-            const int i = ty + 32 * u, j = tx + 32 * w;
-            if (i < n && j < n) mo[(int64_t)i * ldm + j] = v[u][w];
+        for (int w = 0; w < T; ++w) {
+            const int i = sweep_index(ty, u), j = sweep_index(tx, w);
+            if (i < n && j < n) mo[(int64_t)i * ldm + j] = -g[u][w];
         }
-}
-
-template <int R>
-void launch_inverse_blocked(const float* A, int64_t ldA, int64_t gsA, float* Mout, int64_t ldM, int64_t gsM,
-                            int64_t n, int32_t G, int32_t g0, DevStatus* st, cudaStream_t s)
-{
-    static std::once_flag once;
-    std::call_once(once, [] {
-        UOI_CUDA(cudaFuncSetAttribute(k_spd_inverse_blocked<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)gj_smem_bytes<R>()));
-    });
-    k_spd_inverse_blocked<R><<<(unsigned)G, 1024, gj_smem_bytes<R>(), s>>>(A, ldA, gsA, Mout, ldM, gsM,
-                                                                           (int)n, g0, st);
 }
 
 void inv_base(const float* A, int64_t ldA, int64_t gsA, float* Mout, int64_t ldM, int64_t gsM,
               int64_t n, int32_t G, int32_t g0, DevStatus* st, cudaStream_t s)
 {
-    if (n <= 64)
-        launch_inverse_blocked<2>(A, ldA, gsA, Mout, ldM, gsM, n, G, g0, st, s);
-    else if (n <= 128)
-        launch_inverse_blocked<4>(A, ldA, gsA, Mout, ldM, gsM, n, G, g0, st, s);
-    else
-        launch_inverse_blocked<6>(A, ldA, gsA, Mout, ldM, gsM, n, G, g0, st, s);
+    const auto kern = n <= 64 ? k_spd_inverse_sweep<4> : n <= 128 ? k_spd_inverse_sweep<8> : k_spd_inverse_sweep<12>;
+    kern<<<(unsigned)G, 256, 0, s>>>(A, ldA, gsA, Mout, ldM, gsM, (int)n, g0, st);
     UOI_CHECK_LAUNCH();
     count_launch();
 }
