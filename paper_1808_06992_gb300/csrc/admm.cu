@@ -254,7 +254,9 @@ __global__ void __launch_bounds__(256, 1) k_admm_resident(AdmmDev<T> P, int32_t*
 // at 64 clocks, two block barriers, the exchange); past L2 the stream of M.
 // Measured (one call; one warp per chain or two launches per iteration, then this schedule
 // with FP64 products, then as it is): 200 x 50, 20 chains, 598 iterations each: 12.7, 2.3,
-// 1.65 ms; p = 400, 20 chains: 38, 6.9, 3.8 ms; p = 1000 (M 160 MB): 124, 52, 26 ms;
+// 1.65 ms; p = 400, 20 chains: 38, 6.9, 3.8 ms; p = 1000 (M 160 MB): 124, 52, 14 ms
+// (26 ms with 8 and 3 blocks per pass instead of 6 and 5: a pass of few blocks has few
+// loads in flight);
 // p = 150, 128 chains: 110, 5.1, 3.0 ms.
 constexpr int CH_RB = 16;            // rows per block
 constexpr int CH_NB = 8;             // blocks accumulated together
@@ -367,7 +369,7 @@ __device__ __forceinline__ void ch_product(const typename ChNumOf<T>::type* m, s
     // p - 1 repeat the last
     const size_t step = (size_t)kstep * ld;
     const Num* mk = m + (size_t)min(k0, p - 1) * ld;
-#pragma unroll(NB > 4 || !SHARED ? 2 : 4)
+#pragma unroll(NB > (SHARED ? 4 : 6) ? 2 : 4)
     for (int k = k0; k < kp; k += kstep, mk += step) {
         const Num* mr = SHARED ? mk : m + (size_t)min(k, p - 1) * ld;
         Num v[NC], x[NB];
@@ -539,7 +541,9 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
             Sum* pw = part + (size_t)warp * NC * nrp;
             const size_t ld = geo.ldm ? (size_t)geo.ldm : (size_t)p;
             const Num* base = geo.ldm ? Ms : Mi + row0;
-            constexpr int CB = NC == 1 ? CH_NB : CH_NB / 2;
+            // blocks per pass over k, as equal as they come: loads in flight hide a streamed M's latency
+            constexpr int CB_MAX = NC == 1 ? CH_NB : CH_NB / 2;
+            const int CB = geo.ldm ? CB_MAX : (nblk + (nblk + CB_MAX - 1) / CB_MAX - 1) / ((nblk + CB_MAX - 1) / CB_MAX);
             for (int c0 = 0; c0 < nblk; c0 += CB) {
                 const int row = c0 * CH_RB + ri;
                 const Num* m = base + min(row, nrows - 1);
