@@ -130,7 +130,7 @@ extern "C" int lasso_admm_batch_noalloc(const double* X, const double* Y, int64_
         const size_t need = 3 * (sizeof(double) * (size_t)(B * p * p) + 256) +
                             2 * (sizeof(double) * (size_t)(B * p * r) + 256) +
                             sizeof(double) * (size_t)(B * p) + 256 +
-                            sizeof(double) * B + 2 * sizeof(int32_t) * B + sizeof(DevStatus) +
+                            sizeof(double) * B + sizeof(int32_t) * B + sizeof(DevStatus) +
                             (size_t)ncol + sizeof(int32_t) + 6 * 256;
         if (need > kScratchBytes)
             throw Error(UOI_ERR_INVALID_ARG, "problem needs more than the 16 MiB no-allocation scratch");
@@ -144,7 +144,7 @@ extern "C" int lasso_admm_batch_noalloc(const double* X, const double* Y, int64_
         double* c = cv.take<double>((size_t)(B * p * r));
         double* bs = cv.take<double>((size_t)(B * p));
         double* nk = cv.take<double>((size_t)B);
-        int32_t* chains = cv.take<int32_t>((size_t)(2 * B));
+        int32_t* chains = cv.take<int32_t>((size_t)B);
         DevStatus* st = cv.take<DevStatus>(1);
         uint8_t* conv = cv.take<uint8_t>((size_t)ncol);
         int32_t* noncon = cv.take<int32_t>(1);
@@ -152,7 +152,7 @@ extern "C" int lasso_admm_batch_noalloc(const double* X, const double* Y, int64_
             throw Error(UOI_ERR_INVALID_ARG, "problem needs more than the 16 MiB no-allocation scratch");
 
         // the array keeps the previous call's contents: clear what must start at zero
-        UOI_CUDA(cudaMemsetAsync(chains, 0, sizeof(int32_t) * 2 * B, s));
+        UOI_CUDA(cudaMemsetAsync(chains, 0, sizeof(int32_t) * B, s));
         UOI_CUDA(cudaMemsetAsync(st, 0, sizeof(DevStatus), s));
         UOI_CUDA(cudaMemsetAsync(noncon, 0, sizeof(int32_t), s));
 
