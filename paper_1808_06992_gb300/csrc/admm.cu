@@ -1409,6 +1409,7 @@ template <typename T>
 bool admm_solve_resident_with(const AdmmProblem<T>& P, int32_t* chain_next, cudaStream_t s)
 {
     if (P.G <= 0 || P.p <= 0 || P.r <= 0 || P.q <= 0) return true;
+    if (P.p > 128) return false;                     // up to here M fits in shared memory: no exponents
     const AdmmDev<T> d = to_dev(P);
     return try_resident<T>(d, chain_next, s);
 }

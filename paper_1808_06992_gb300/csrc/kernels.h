@@ -243,8 +243,8 @@ void admm_batch_destroy(AdmmBatch* b);
 void admm_batch_enter(AdmmBatch* b);
 void admm_batch_leave();
 bool admm_batch_try_join(const AdmmProblem<float>& P, cudaStream_t s);
-// Chain or resident schedule only, with the caller's zeroed per-group words (2 G int32:
-// chain counters, then exponents).  Returns false (launching nothing) when p is too large for it.
+// One-launch schedule only, with the caller's zeroed per-group chain counters (G int32).
+// Returns false (launching nothing) when p > 128.
 template <typename T>
 bool admm_solve_resident_with(const AdmmProblem<T>& P, int32_t* chain_next, cudaStream_t s);
 
