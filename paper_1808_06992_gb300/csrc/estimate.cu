@@ -3,8 +3,8 @@
 //
 // For estimation bootstrap k and family member S_j (per response e):
 //   beta = argmin || W^{1/2} (y_e - X_S b) ||   from G'_k[S,S] (FP64 moments):
-//   FP32 Cholesky + FP64 iterative refinement, FP64 Cholesky where FP32 is
-//   not safe (see k_ols_mixed)
+//   FP32 inverse or Cholesky + FP64-accurate iterative refinement, FP64 Cholesky
+//   where FP32 is not safe (see k_ols_warp, k_ols_block, k_ols_mixed)
 //   L_kje = sum_{t in E^k} (y_te - x_t beta)^2
 //         = y_E'y_E - 2 beta' (X_E'y_E)_S + beta' G^E_k[S,S] beta
 // j*_k = argmin_j sum_e L_kje (ties -> smallest j); beta*_e = median (or mean)
