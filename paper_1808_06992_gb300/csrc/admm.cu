@@ -523,7 +523,9 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
         }
         __syncthreads();
     };
-    __syncthreads();                                         // s_kappa
+    // s_kappa and V, and every CTA of the cluster has started: only then may rank 0 store into the
+    // others' shared memory
+    ch_barrier(cs);
     fetch((1u << NC) - 1u, 0);
 
     const int slot = warp % NC, wi = warp / NC, nwi = NW / NC;   // this warp's slot in the row-wise steps
