@@ -454,7 +454,7 @@ k_admm_wide(const __grid_constant__ CUtensorMap tmM, WideArgs a)
                             nv[kk] = v;
                             const float d = x - zn, dz = zn - zp;
                             n5[0] += d * d; n5[1] += dz * dz; n5[2] += x * x; n5[3] += zn * zn; n5[4] += un * un;
-                            vs[k2] = (zn - un) * sw;
+                            vs[k2] = sw != 0.f ? (zn - un) * sw : 0.f;   // an ended chain's NaN or Inf stays its own
                         }
                         const __half2 h = __floats2half2_rn(vs[0], vs[1]);
                         const float2 hf = __half22float2(h);
