@@ -279,9 +279,11 @@ __global__ void __launch_bounds__(256) k_ols(OlsArgs a)
 // Up to 128 columns (k_ols_warp, k_ols_block) the solve is a symmetric Gauss-Jordan sweep in
 // registers, which leaves -G^{-1}: a refinement step is then a matrix-vector product instead of
 // two substitutions, whose s dependent steps were most of a small solve's time.  The pivots are
-// those of the Cholesky factor.  G is scaled by a power of two below 1 and kept as exact
-// integers (fixed_dot.cuh) for the residuals: the FP64 pipe would take 19 clocks per 32 entries
-// and the gather of G from L2 would be repeated at each step.
+// those of the Cholesky factor.  Rows and columns of G are scaled by powers of two 2^-e_i that
+// bring its diagonal to [1/4, 1) (exact; one scale for all of G lost the bits of its small
+// columns), and the result is kept as integers (fixed_dot.cuh) for the residuals: the FP64
+// pipe would take 19 clocks per 32 entries and the gather of G from L2 would be repeated at
+// each step.
 // Measured (all solves of a fit, against one CTA with a packed factor for every size): VAR
 // p = 192, 30 bootstraps x 32 lambdas (supports of a few to 30 columns): 4.1 -> 0.25 ms;
 // 4999 x 301, 24 x 32 (15 to 111 columns): 0.43 -> 0.13 ms.
@@ -370,6 +372,33 @@ __device__ __forceinline__ int ols_converged(int itr, float dmx, float xmx, floa
     return 0;
 }
 
+// e with d 2^(-2 e) in [1/4, 1) for d > 0 with high word h.
+__device__ __forceinline__ int ols_scale(uint32_t h) { return (fx_exponent(h) + 1) >> 1; }
+
+// Whether |v| 2^-e is 1 or more, or v is Inf or NaN.
+__device__ __forceinline__ bool ols_exceeds(double v, int e)
+{
+    const uint32_t h = fx_high(v);
+    return h >= 0x7FF00000u || (h != 0 && fx_exponent(h) > e);
+}
+
+// Least pivot of a scaled column: OLS_F32_PIVOT of the largest diagonal (high word hg) before
+// scaling, in the scale of a column with exponent e.
+__device__ __forceinline__ float ols_pivot(uint32_t hg, int e)
+{
+    const float top = __uint_as_float(0x3F000000u | (hg & 0xFFFFFu) << 3);       // hg's value over 2^fx_exponent
+    return hg == 0 ? 1.f : ldexpf(OLS_F32_PIVOT * top, min(fx_exponent(hg) - 2 * e, 100));
+}
+
+// Exponent of v 2^-e as a number that grows with it (0 for v = 0, past any other for Inf or NaN).
+constexpr uint32_t OLS_EXP_BIAS = 16384, OLS_EXP_NONFINITE = 0x7FFFFFFF;
+__device__ __forceinline__ uint32_t ols_exponent_key(double v, int e)
+{
+    const uint32_t h = fx_high(v);
+    return h >= 0x7FF00000u ? OLS_EXP_NONFINITE : h == 0 ? 0u : (uint32_t)(fx_exponent(h) - e + (int)OLS_EXP_BIAS);
+}
+__device__ __forceinline__ int ols_key_exponent(uint32_t k) { return k == 0 ? 0 : (int)k - (int)OLS_EXP_BIAS; }
+
 // Solves of at most 32 columns, one per warp: lane i holds row i of the swept matrix.
 // Bound by issue slots and the latency of a few hundred dependent steps; a warp per solve keeps
 // 16 or more in flight on an SM, and needs no block barrier.  The line at 32 is the warp's width.
@@ -378,7 +407,7 @@ struct OlsWarpSmem {
     int2 xd[32];
     double xb[32];
     float buf[2][32];
-    int idx[32];
+    int idx[32], ex[32];
 };
 __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits)
 {
@@ -407,9 +436,12 @@ __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits
         const double dg = in ? __ldg(Gk + (size_t)my * a.pu + my) : 0.0;
         const double b = in ? __ldg(a.Bt + ((size_t)o.k * a.pu + my) * a.r + o.e) : 0.0;
         const uint32_t hg = __reduce_max_sync(0xffffffffu, fx_high(dg));
-        const uint32_t hb = __reduce_max_sync(0xffffffffu, fx_high(b));
-        const int em = fx_exponent(hg), eb = fx_exponent(hb);
-        bool bad = hb >= 0x7FF00000u;                        // Inf or NaN; G's entries at 2^em or above below
+        const int e = ols_scale(fx_high(dg));
+        const uint32_t hb = __reduce_max_sync(0xffffffffu, ols_exponent_key(b, e));
+        const int eb = ols_key_exponent(hb);
+        m.ex[lane] = e;
+        __syncwarp();
+        bool bad = hb == OLS_EXP_NONFINITE;                  // scaled entries of G at 1 or above: below
         float g[32];
         const float unit = __uint_as_float((uint32_t)(127 + 28 - bits) << 23);
 #pragma unroll
@@ -421,8 +453,9 @@ __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits
                     v[i] = in && c0 + i < s ? __ldg(Gk + (size_t)m.idx[c0 + i] * a.pu + my) : 0.0;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const int2 d = fx_digits(v[i], em, bits);
-                    bad |= (fx_high(v[i]) >> 20) > (hg >> 20) || fx_high(v[i]) >= 0x7FF00000u;
+                    const int ev = e + m.ex[c0 + i];
+                    const int2 d = fx_digits(v[i], ev, bits);
+                    bad |= ols_exceeds(v[i], ev);
                     if (in && c0 + i < s) Gd[(c0 + i) * s + lane] = d;
                     g[c0 + i] = (float)d.x * unit;
                 }
@@ -432,12 +465,7 @@ __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits
             }
         }
         bool ok = !__any_sync(0xffffffffu, bad);
-        float dmax = 0.f;
-#pragma unroll
-        for (int c = 0; c < 32; ++c)
-            if (lane == c) dmax = g[c];
-        dmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(dmax, 0.f))));
-        const float thr = OLS_F32_PIVOT * dmax;
+        const float thr = ols_pivot(hg, e);                  // of this lane's column
         // sweep of column c: g_ij -= g_ic g_cj / d, row and column c times 1 / d, g_cc = -1 / d.
         // Row c is column c (symmetry), and in lane c the same update with 1 - 1/d for g_ic / d
         // leaves g_cj / d.
@@ -445,7 +473,7 @@ __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits
         for (int c = 0; c < 32; ++c) {
             if (c < s && ok) {                               // the same in every lane
                 const float d = __shfl_sync(0xffffffffu, g[c], c);
-                if (!(d > thr)) ok = false;
+                if (__any_sync(0xffffffffu, lane == c && !(d > thr))) ok = false;
                 else {
                     float* row = m.buf[c & 1];
                     row[lane] = g[c];
@@ -462,7 +490,7 @@ __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits
                 }
             }
         }
-        const double bs = b * fx_pow2(-eb);                  // x comes out times 2^(em - eb)
+        const double bs = scalbn(b, -e - eb);                // x comes out times 2^(e - eb)
         double x = 0.0;
         bool done = false;
         if (ok) {
@@ -501,7 +529,7 @@ __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits
             if (lane == 0) a.fb_list[atomicAdd(a.fb_count, 1)] = (int32_t)o.tg;
             continue;
         }
-        x = scalbn(x, eb - em);
+        x = scalbn(x, eb - e);
         if (a.jstar) {
             if (in) a.chosen[((size_t)o.k * a.r + o.e) * a.p + a.ucols[my]] = x;
             continue;
@@ -533,8 +561,8 @@ struct OlsBlockSmem {
     double bs[16 * T], x[16 * T];
     long long part[256];
     int2 xd[16 * T];
-    float buf[2][16 * T], w[16 * T], y[16 * T];
-    int idx[16 * T];
+    float buf[2][16 * T], w[16 * T], y[16 * T], thr[16 * T];
+    int idx[16 * T], ex[16 * T];
     uint32_t red[3][8];
     double redd[8];
     int64_t next;
@@ -589,10 +617,12 @@ __global__ void __launch_bounds__(256, T == 4 ? 4 : 2) k_ols_block(OlsArgs a)
         const double* Gk = a.Gt + (size_t)o.k * a.pu * a.pu;
         const double dg = tid < s ? __ldg(Gk + (size_t)my * a.pu + my) : 0.0;
         const double b = tid < s ? __ldg(a.Bt + ((size_t)o.k * a.pu + my) * a.r + o.e) : 0.0;
-        uint32_t hg = fx_high(dg), hb = fx_high(b), zero = 0;
-        block_max3(hg, hb, zero);                            // its barrier: idx is complete
-        const int em = fx_exponent(hg), eb = fx_exponent(hb);
-        bool bad = hb >= 0x7FF00000u;
+        const int e = ols_scale(fx_high(dg));
+        if (tid < R) m.ex[tid] = e;
+        uint32_t hg = fx_high(dg), hb = tid < s ? ols_exponent_key(b, e) : 0u, zero = 0;
+        block_max3(hg, hb, zero);                            // its barrier: idx and ex are complete
+        const int eb = ols_key_exponent(hb);
+        bool bad = hb == OLS_EXP_NONFINITE;
         for (int c = warp; c < s; c += 8) {
             const double* row = Gk + (size_t)m.idx[c] * a.pu;
             double v[R / 32];
@@ -600,13 +630,15 @@ __global__ void __launch_bounds__(256, T == 4 ? 4 : 2) k_ols_block(OlsArgs a)
             for (int i = 0; i < R / 32; ++i) v[i] = lane + 32 * i < s ? __ldg(row + m.idx[lane + 32 * i]) : 0.0;
 #pragma unroll
             for (int i = 0; i < R / 32; ++i) {
-                bad |= (fx_high(v[i]) >> 20) > (hg >> 20) || fx_high(v[i]) >= 0x7FF00000u;
-                if (lane + 32 * i < s) Gd[c * s + lane + 32 * i] = fx_digits(v[i], em, bits);
+                const int ev = m.ex[c] + m.ex[lane + 32 * i];
+                bad |= ols_exceeds(v[i], ev);
+                if (lane + 32 * i < s) Gd[c * s + lane + 32 * i] = fx_digits(v[i], ev, bits);
             }
         }
-        const double bs = b * fx_pow2(-eb);
+        const double bs = scalbn(b, -e - eb);
         if (tid < R) {
             m.bs[tid] = bs;
+            m.thr[tid] = ols_pivot(hg, e);
             m.x[tid] = 0.0;
             m.w[tid] = f64_to_f32_int(bs);                   // zero past s
             m.xd[tid] = make_int2(0, 0);
@@ -620,9 +652,6 @@ __global__ void __launch_bounds__(256, T == 4 ? 4 : 2) k_ols_block(OlsArgs a)
                 const int i = ty + 16 * u, j = tx + 16 * v;
                 g[u][v] = i < s && j < s ? (float)Gd[j * s + i].x * unit : 0.f;
             }
-        float dmax = 0.f;
-        for (int c = 0; c < s; ++c) dmax = fmaxf(dmax, (float)Gd[c * s + c].x * unit);
-        const float thr = OLS_F32_PIVOT * dmax;
 #pragma unroll
         for (int v0 = 0; v0 < T; ++v0) {
             for (int l = 0; l < 16 && ok; ++l) {
@@ -635,7 +664,7 @@ __global__ void __launch_bounds__(256, T == 4 ? 4 : 2) k_ols_block(OlsArgs a)
                 }
                 __syncthreads();
                 const float d = col[c];
-                if (!(d > thr)) { ok = false; break; }
+                if (!(d > m.thr[c])) { ok = false; break; }
                 const float inv = __frcp_rn(d);
                 float r[T], f[T];
 #pragma unroll
@@ -705,7 +734,7 @@ __global__ void __launch_bounds__(256, T == 4 ? 4 : 2) k_ols_block(OlsArgs a)
             if (tid == 0) a.fb_list[atomicAdd(a.fb_count, 1)] = (int32_t)o.tg;
             continue;
         }
-        x = scalbn(x, eb - em);
+        x = scalbn(x, eb - e);
         if (a.jstar) {
             if (tid < s) a.chosen[((size_t)o.k * a.r + o.e) * a.p + a.ucols[my]] = x;
             continue;
