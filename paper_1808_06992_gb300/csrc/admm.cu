@@ -239,14 +239,23 @@ __global__ void __launch_bounds__(256, 1) k_admm_resident(AdmmDev<T> P, int32_t*
 //             next iteration written into every CTA of the cluster;
 //   stop      the CTAs exchange five partial norms; one cluster barrier ends the
 //             iteration, after which every thread takes the same decision.
-// FP64 products run on the integer pipe.  M and V are taken to integers Q, P of up to 57 bits
-// with sign (a power of two above the group's largest entry of M, on its diagonal, and above
-// V's largest value at this step), split into balanced digits of 28 bits, and
-//   x - c = rho 2^(..) sum_k hi hi' 2^56 + (hi lo' + lo hi') 2^28      (+ lo lo', below 2^-58)
-// is summed exactly in 64 bits by three 32 x 32 + 64 -> 64 multiply-adds per entry.  This
-// part's FP64 pipe charges 19 clocks and SM per warp instruction, the integer pipe 1 per
-// multiply-add.  The error is that of rounding M and V, 2^-57 of their largest values, where
-// an FP64 dot product rounds every partial sum at 2^-53.  The rest of an iteration is FP64:
+// FP64 products run on the integer pipe (fixed_dot.cuh).  M and V are equilibrated first, by
+// powers of two and so exactly: with 2^(2 f_i) above M_ii, M^ = M_ij 2^(-f_i - f_j) has entries
+// below 1, and V^ = V_j 2^(f_j) is scaled by its largest value of this step.  (One scale for
+// all of M cost features whose columns are larger than others' their bits: 2^-57 of the
+// largest M_ii.)  Both become integers of h + l bits, and
+//   x_i - c_i = rho 2^(f_i + ..) sum_k hi hi' 2^(2 l) + (hi lo' + lo hi') 2^l   (+ lo lo', below the last bit)
+// is summed exactly in 64 bits by three 32 x 32 + 64 -> 64 multiply-adds per entry.  h comes
+// from the largest row sum R of |M^|, which bounds every sum by R 2^(2 h) (R is 1 to 4 where
+// the number of terms is 50 to 1000: 30 bits instead of 26 to 28), l from what is then left
+// for the terms of one thread: 57 to 60 bits in all.  This part's FP64 pipe charges 19 clocks
+// and SM per warp instruction, the integer pipe 1 per multiply-add.  The error is that of
+// rounding M^ and V^, 2^-58 to 2^-61 of 1 and of V^'s largest value, where an FP64 dot product
+// rounds every partial sum at 2^-53.  Against 80-bit iterates after 60 steps (a model of this
+// arithmetic on the CPU, p = 24..1000, columns of equal scale and up to 1e3 apart) the 2-norm
+// error of z is 0.2 to 0.7 times that of FP64 sums (1.3 times in one of eight), that of u 0.4 to
+// 1.0 times; where columns are 1e5 apart, entries of u far below its largest are off by 4e-13 of
+// themselves (2e-15 with FP64 sums).  The rest of an iteration is FP64:
 // no instruction of it may run on few lanes, and the norms are first taken in FP32 (from the
 // FP64 differences): only when those say that the stop test may pass are they formed in
 // FP64, so that decisions are those of the FP64 norms.
@@ -269,8 +278,7 @@ struct ChainGeom {
     int32_t nrp;                     // rows of the largest CTA, a multiple of CH_RB
     int32_t kp;                      // k extent padded to a multiple of 2 * warps
     int32_t ldm;                     // row length of the shared copy of M, 0: M stays in global memory
-    int32_t bits;                    // FP64: fx_bits of the products one thread sums
-    int32_t fits;                    // FP64: the sum of all p products fits 63 bits
+    int32_t lg_terms;                // FP64: log2 of the products one thread sums, rounded up
     size_t smem;
 };
 
@@ -333,8 +341,44 @@ template <typename T> struct ChNumOf;
 template <> struct ChNumOf<float> { using type = float; };
 template <> struct ChNumOf<double> { using type = int2; };
 
+// Digits of the FP64 products: sums of |M^ V^| are below 2^(lg_sum), one thread's have 2^lg_terms
+// terms; all sums of upper digits' products then stay within 2^62, and those of the mixed ones.
+struct ChDigits { int bits, lo; };
+__device__ __forceinline__ ChDigits ch_digits_for(int lg_sum, int lg_terms)
+{
+    const int h = min(30, (62 - lg_sum) / 2);
+    const int lo = min(30, 62 - h - max(lg_sum, lg_terms));
+    return { h + lo, lo };
+}
+
+// f with x 2^(-2 f) in [1/4, 1) for x > 0.
+__device__ __forceinline__ int ch_scale(double x) { return (fx_exponent(fx_high(x)) + 1) >> 1; }
+
+// |x| 2^-e in FP32, cut off to 23 bits (0 below 2^-126).
+__device__ __forceinline__ float ch_scaled32(double x, int e)
+{
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu, m = __funnelshift_l((uint32_t)__double2loint(x), h, 3) & 0x7FFFFFu;
+    const int ex = (int)(h >> 20) - e - 896;                 // exponent bias 1023 -> 127
+    return ex <= 0 ? 0.f : ex >= 255 ? __uint_as_float(0x7F800000u) : __uint_as_float((uint32_t)ex << 23 | m);
+}
+
+// log2, rounded up, of a bound on what sums of ch_scaled32 stand for.
+__device__ __forceinline__ int ch_log2_bound(float sum)
+{
+    const int e = (int)(__float_as_uint(sum * 1.001f + 1e-30f) >> 23) - 126;
+    return max(0, min(e, 40));
+}
+
+// Exponent of x 2^f as a number that grows with it: 0 for x = 0, past any other for Inf or NaN.
+constexpr uint32_t CH_KEY_BIAS = 16384, CH_KEY_NONFINITE = 0x7FFFFFFF;
+__device__ __forceinline__ uint32_t ch_key(double x, int f)
+{
+    const uint32_t h = fx_high(x);
+    return h >= 0x7FF00000u ? CH_KEY_NONFINITE : h == 0 ? 0u : (uint32_t)(fx_exponent(h) + f + (int)CH_KEY_BIAS);
+}
+
 // acc += m v.  FP64: exact 64-bit sums of the digits' products; value() is the sum in units
-// of 2^56, rounded.  FP32: the rounding errors of the product and of the sum go to a second
+// of 2^(2 lo), rounded.  FP32: the rounding errors of the product and of the sum go to a second
 // word.
 struct ChSumF {
     using Out = float;
@@ -346,7 +390,7 @@ struct ChSumF {
         c += (__fsub_rn(a, __fsub_rn(s, b)) + __fsub_rn(p, b)) + e;
         a = s;
     }
-    __device__ __forceinline__ float value() const { return a + c; }
+    __device__ __forceinline__ float value(int) const { return a + c; }
 };
 template <typename T> struct ChSumOf;
 template <> struct ChSumOf<double> { using type = FxSum; };
@@ -358,7 +402,7 @@ template <> struct ChSumOf<float> { using type = ChSumF; };
 template <typename T, int NB, int NC, bool SHARED>
 __device__ __forceinline__ void ch_product(const typename ChNumOf<T>::type* m, size_t ld, int p,
                                            const typename ChNumOf<T>::type* V, int kp, int k0, int kstep, int row,
-                                           int nrows, typename ChSumOf<T>::type::Out* out, int ostr)
+                                           int nrows, typename ChSumOf<T>::type::Out* out, int ostr, int lob)
 {
     using Num = typename ChNumOf<T>::type;
     typename ChSumOf<T>::type acc[NB][NC];
@@ -386,7 +430,7 @@ __device__ __forceinline__ void ch_product(const typename ChNumOf<T>::type* m, s
     for (int b = 0; b < NB; ++b)
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-            typename ChSumOf<T>::type::Out s = acc[b][c].value();
+            typename ChSumOf<T>::type::Out s = acc[b][c].value(lob);
             s += __shfl_xor_sync(0xffffffffu, s, CH_RB);
             if ((threadIdx.x & 31) < CH_RB) out[c * ostr + b * CH_RB] = s;
         }
@@ -394,7 +438,7 @@ __device__ __forceinline__ void ch_product(const typename ChNumOf<T>::type* m, s
 
 template <typename T, int NC>
 __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P, int32_t* chain_next, ChainGeom geo,
-                                                   const int32_t* m_exp)
+                                                   const int32_t* m_scale)
 {
     using Num = typename ChNumOf<T>::type;
     using Sum = typename ChSumOf<T>::type::Out;
@@ -405,7 +449,7 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
     __shared__ float s_norm[2][CH_CLUSTER_MAX][NC][5];
     __shared__ T s_redx[16][5], s_exact[CH_CLUSTER_MAX][NC][5];
     __shared__ int s_cid[NC];
-    __shared__ uint32_t s_max[2][CH_CLUSTER_MAX][NC], s_redm[16];   // largest high word of |V'|
+    __shared__ uint32_t s_max[2][CH_CLUSTER_MAX][NC], s_redm[16];   // largest exponent key of V^'
     const int p = P.p, cs = geo.cs, nrp = geo.nrp, kp = geo.kp;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, NW = blockDim.x >> 5;
     int rank = 0;
@@ -415,7 +459,8 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
     const int b0 = rank * nbt / cs, nblk = (rank + 1) * nbt / cs - b0;
     const int row0 = b0 * CH_RB, nrows = min(p - row0, nblk * CH_RB);
     const T* Mg = P.M + (size_t)g * p * p;
-    // shared memory: [M] | V, two buffers of NC | [FP64: V's digits] | partial products | z u c x z_prev
+    // shared memory: [M] | V, two buffers of NC | [FP64: V's digits] | partial products | z u c x z_prev |
+    // [FP64 with M: the rows' f]
     Num* Ms = reinterpret_cast<Num*>(smem_raw);
     T* V = reinterpret_cast<T*>(Ms + (size_t)geo.ldm * kp);
     Num* Vi = reinterpret_cast<Num*>(V + (size_t)2 * NC * kp);
@@ -426,44 +471,86 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
     T* xs = cv + NC * nrp;
     T* zq = xs + NC * nrp;
     const Num* Mi = reinterpret_cast<const Num*>(Mg);        // streamed M: digits already
-    int em = 0;                                              // |M| < 2^em
+    // FP64: f of the features k = threadIdx.x and + blockDim.x in registers (with M in shared
+    // memory there are no more), of this CTA's rows in rowf, of all in feat (streamed M)
+    int f0 = 0, f1 = 0, bits = 0, lob = 0;
+    int* rowf_s = reinterpret_cast<int*>(zq + NC * nrp);
+    const int* rowf = rowf_s;
+    const int* feat = nullptr;
     if constexpr (F64) {
+        const int ka = threadIdx.x, kb = threadIdx.x + blockDim.x;
         if (geo.ldm) {
-            uint32_t h = 0;
-            for (int i = threadIdx.x; i < p; i += blockDim.x) h = max(h, fx_high(Mg[(size_t)i * p + i]));
-            h = __reduce_max_sync(0xffffffffu, h);
-            if (lane == 0) s_redm[warp] = h;
+            if (ka < p) f0 = ch_scale(Mg[(size_t)ka * p + ka]);
+            if (kb < p) f1 = ch_scale(Mg[(size_t)kb * p + kb]);
+            for (int i = threadIdx.x; i < nrows; i += blockDim.x) rowf_s[i] = ch_scale(Mg[(size_t)(row0 + i) * p + row0 + i]);
             __syncthreads();
+            // the largest row sum of |M^|: over the columns k of a warp, the warps, the rows, the cluster
+            float* ps = reinterpret_cast<float*>(part) + (size_t)warp * nrp;
+            for (int i = lane; i < nrows; i += 32) {
+                float sum = 0.f;
+#pragma unroll 4
+                for (int k = warp; k < p; k += NW)
+                    sum += ch_scaled32(Mg[(size_t)k * p + row0 + i], rowf_s[i] + ch_scale(Mg[(size_t)k * p + k]));
+                ps[i] = sum;
+            }
+            __syncthreads();
+            float top = 0.f;
+            for (int i = threadIdx.x; i < nrows; i += blockDim.x) {
+                float sum = 0.f;
+                for (int w = 0; w < NW; ++w) sum += reinterpret_cast<float*>(part)[(size_t)w * nrp + i];
+                top = fmaxf(top, sum);
+            }
+            uint32_t h = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+            if (lane == 0) s_redm[warp] = h;
+            ch_barrier(cs);                                  // and every CTA of the cluster has started
             for (int w = 0; w < NW; ++w) h = max(h, s_redm[w]);
-            em = fx_exponent(h);
-            for (int k = warp; k < p; k += NW)
+            if (cs > 1) {
+                if (threadIdx.x < cs) ch_store_rank(&s_max[1][rank][0], (int)threadIdx.x, h);
+                ch_barrier(cs);
+                for (int k = 0; k < cs; ++k) h = max(h, s_max[1][k][0]);
+            }
+            const ChDigits d = ch_digits_for(ch_log2_bound(__uint_as_float(h)), geo.lg_terms);
+            bits = d.bits;
+            lob = d.lo;
+            for (int k = warp; k < p; k += NW) {
+                const int fk = ch_scale(Mg[(size_t)k * p + k]);
                 for (int i = lane; i < nrows; i += 32)
-                    Ms[(size_t)k * geo.ldm + i] = fx_digits(Mg[(size_t)k * p + row0 + i], em, geo.bits);
+                    Ms[(size_t)k * geo.ldm + i] = fx_digits(Mg[(size_t)k * p + row0 + i], fk + rowf_s[i], bits, lob);
+            }
         } else {
-            em = m_exp[g];
+            feat = m_scale + P.G + (size_t)g * p;
+            rowf = feat + row0;
+            if (ka < p) f0 = feat[ka];
+            if (kb < p) f1 = feat[kb];
+            const ChDigits d = ch_digits_for(ch_log2_bound(__int_as_float(m_scale[g])), geo.lg_terms);
+            bits = d.bits;
+            lob = d.lo;
         }
     } else if (geo.ldm) {
         for (int k = warp; k < kp; k += NW)
             for (int i = lane; i < nrows; i += 32)
                 Ms[(size_t)k * geo.ldm + i] = k < p ? Mg[(size_t)k * p + row0 + i] : T(0);
     }
-    // digits of V_slot from buffer `buf`, their scale in rs[slot]: x = c + rs (sum of digits)
-    T rs[NC];
+    auto feature_scale = [&](int k) {                        // f_k of a feature k this thread owns in V
+        return k >= p ? 0 : k == (int)threadIdx.x ? f0 : k == (int)(threadIdx.x + blockDim.x) ? f1 : feat[k];
+    };
+    // digits of V^_slot from buffer `buf`, their scale's exponent in re[slot]:
+    // x = c + rho 2^(re + f) (sum of digits)
+    constexpr int RE_NAN = 1 << 30;
+    int re[NC];
     int rho_e = 0;                                           // exponent field of rho (0: subnormal, scaled by scalbn)
     if constexpr (F64) {
         rho_e = (__double2hiint(P.rho) >> 20) & 0x7FF;
         if (rho_e == 0) rho_e = -100000;
     }
-    auto digits = [&](int buf, int s, uint32_t h) {
+    auto digits = [&](int buf, int s, uint32_t key) {
         if constexpr (F64) {
-            const int ev = h == 0 ? 0 : fx_exponent(h);
+            const int ev = key == 0 ? 0 : (int)key - (int)CH_KEY_BIAS;
             const T* src = V + ((size_t)buf * NC + s) * kp;
-            for (int k = threadIdx.x; k < kp; k += blockDim.x) Vi[s * kp + k] = fx_digits(src[k], ev, geo.bits);
-            // M = Q 2^(em - bits), V = P 2^(ev - bits), sums in units of 2^56; NaN if V holds Inf or NaN
-            const int x = em + ev - 2 * geo.bits + 56;
-            if (h >= 0x7FF00000u) rs[s] = __longlong_as_double(0x7FF8000000000000ll);
-            else if (x + rho_e > 0 && x + rho_e < 2046) rs[s] = __longlong_as_double(__double_as_longlong(P.rho) + ((long long)x << 52));
-            else rs[s] = scalbn(P.rho, x);
+            for (int k = threadIdx.x; k < kp; k += blockDim.x)
+                Vi[s * kp + k] = fx_digits(src[k], ev - feature_scale(k), bits, lob);
+            // M^ = Q 2^-bits, V^ = P 2^(ev - bits), sums in units of 2^(2 lob); NaN if V holds Inf or NaN
+            re[s] = key == CH_KEY_NONFINITE ? RE_NAN : ev - 2 * (bits - lob);
         }
     };
     for (int i = threadIdx.x; i < 2 * NC * kp; i += blockDim.x) V[i] = T(0);
@@ -508,7 +595,7 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
             for (int k = threadIdx.x; k < p; k += blockDim.x) {
                 const T v0 = init ? (T)P.z0[col0 * p + k] - (T)P.u0[col0 * p + k] : T(0);
                 Vn[k] = v0;
-                if constexpr (F64) h = max(h, fx_high(v0));
+                if constexpr (F64) h = max(h, ch_key(v0, feature_scale(k)));
             }
             if constexpr (F64) {
                 if (init) {                              // the largest value of the start, over the block
@@ -553,8 +640,8 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
                 const int k0 = 2 * warp + kk, ks = 2 * NW;
                 auto run = [&](auto nb) {
                     constexpr int NB = decltype(nb)::value;
-                    if (geo.ldm) ch_product<T, NB, NC, true>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp);
-                    else if constexpr (F64) ch_product<T, NB, NC, false>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp);
+                    if (geo.ldm) ch_product<T, NB, NC, true>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp, lob);
+                    else if constexpr (F64) ch_product<T, NB, NC, false>(m, ld, p, Vc, kp, k0, ks, row, nrows, o, nrp, lob);
                 };
                 switch (min(CB, nblk - c0)) {
                 case 1: run(std::integral_constant<int, 1>{}); break;
@@ -576,30 +663,30 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
         __syncthreads();
         // update
         {
-            T kap = T(0), scale = T(0);
+            T kap = T(0);
             bool on = false;
-            uint32_t big = 0;                                // largest high word of |V'|
+            int rexp = 0;
+            uint32_t big = 0;                                // largest exponent key of V^'
 #pragma unroll
             for (int s = 0; s < NC; ++s)
-                if (slot == s) { kap = kappa[s]; on = act[s]; scale = rs[s]; }
+                if (slot == s) { kap = kappa[s]; on = act[s]; rexp = re[s]; }
             float n5[5] = { 0.f, 0.f, 0.f, 0.f, 0.f };
             if (on)
                 for (int i = wi * 32 + lane; i < nrows; i += nwi * 32) {
                     const int o = slot * nrp + i;
                     T x;
+                    int fi = 0;
                     if constexpr (F64) {
-                        // partial sums below 2^62 each: their halves add up in 64 bits
-                        long long up = 0, dn = 0;
-                        if (geo.fits) {                      // and all of them below 2^63
-                            for (int w = 0; w < NW; ++w) dn += part[(size_t)w * NC * nrp + o];
-                        } else {
-                            for (int w = 0; w < NW; ++w) {
-                                const long long q = part[(size_t)w * NC * nrp + o];
-                                up += q >> 32;
-                                dn += (long long)(uint32_t)q;
-                            }
-                        }
-                        x = cv[o] + scale * fma((double)up, 4294967296.0, (double)dn);
+                        fi = rowf[i];
+                        long long sum = 0;                   // within 2^62, however it is split (ch_digits_for)
+                        for (int w = 0; w < NW; ++w) sum += part[(size_t)w * NC * nrp + o];
+                        const int xe = rexp + fi;
+                        T scale;
+                        if (rexp == RE_NAN) scale = __longlong_as_double(0x7FF8000000000000ll);
+                        else if (xe + rho_e > 0 && xe + rho_e < 2046)
+                            scale = __longlong_as_double(__double_as_longlong(P.rho) + ((long long)xe << 52));
+                        else scale = scalbn(P.rho, xe);
+                        x = cv[o] + scale * (double)sum;
                     } else {
                         T sum = part[o];
                         for (int w = 1; w < NW; ++w) sum += part[(size_t)w * NC * nrp + o];
@@ -610,7 +697,7 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
                     const T zn = ch_threshold(v, kap);
                     const T un = v - zn;
                     const T vn = zn - un;
-                    if constexpr (F64) big = max(big, fx_high(vn));
+                    if constexpr (F64) big = max(big, ch_key(vn, fi));
                     const T d = x - zn, dz = zn - zp;
                     zs[o] = zn;
                     us[o] = un;
@@ -778,29 +865,40 @@ __global__ void __launch_bounds__(NC == 1 ? 512 : 256) k_admm_chain(AdmmDev<T> P
     if (cs > 1) ch_barrier(cs);                              // no CTA leaves while another may store into it
 }
 
-// Streamed M of the FP64 chain schedule: exponent of each group, then digits in place.
-__global__ void k_chain_exponent(const double* M, int p, int32_t* em)
+// Streamed M of the FP64 chain schedule.  ms: G row-sum bounds (FP32 bits, zero before), then
+// G x p exponents f; then M turns into its digits in place.
+__global__ void __launch_bounds__(256) k_chain_scales(const double* M, int p, int G, int32_t* ms)
 {
-    __shared__ uint32_t red[8];
-    const double* m = M + (size_t)blockIdx.x * p * p;
-    uint32_t h = 0;
-    for (int i = threadIdx.x; i < p; i += blockDim.x) h = max(h, fx_high(m[(size_t)i * p + i]));
-    h = __reduce_max_sync(0xffffffffu, h);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = h;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) h = max(h, red[w]);
-        em[blockIdx.x] = fx_exponent(h);
-    }
+    const int g = blockIdx.y, i = blockIdx.x * 256 + threadIdx.x;
+    if (i < p) ms[G + (size_t)g * p + i] = ch_scale(M[((size_t)g * p + i) * p + i]);
 }
 
-__global__ void k_chain_digits(double* M, int64_t pp, const int32_t* em, int bits)
+__global__ void __launch_bounds__(256) k_chain_row_sums(const double* __restrict__ M, int p, int G, int32_t* ms)
 {
-    double* m = M + (size_t)blockIdx.y * pp;
-    const int e = em[blockIdx.y];
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < pp; i += (int64_t)gridDim.x * blockDim.x) {
-        const int2 d = fx_digits(m[i], e, bits);
-        m[i] = __hiloint2double(d.y, d.x);                   // the pair's first member in the low word
+    const int g = blockIdx.y, i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= p) return;
+    const double* m = M + ((size_t)g * p + i) * p;
+    const int32_t* f = ms + G + (size_t)g * p;
+    const int fi = f[i];
+    float sum = 0.f;
+#pragma unroll 4
+    for (int k = lane; k < p; k += 32) sum += ch_scaled32(m[k], fi + f[k]);
+    sum = warp_sum(sum);
+    if (lane == 0) atomicMax(&ms[g], __float_as_int(sum));
+}
+
+__global__ void __launch_bounds__(256) k_chain_digits(double* M, int p, int G, const int32_t* ms, int lg_terms)
+{
+    const int g = blockIdx.y;
+    const ChDigits d = ch_digits_for(ch_log2_bound(__int_as_float(ms[g])), lg_terms);
+    const int32_t* f = ms + G + (size_t)g * p;
+    for (int i = blockIdx.x; i < p; i += gridDim.x) {
+        double* m = M + ((size_t)g * p + i) * p;
+        const int fi = f[i];
+        for (int k = threadIdx.x; k < p; k += 256) {
+            const int2 v = fx_digits(m[k], fi + f[k], d.bits, d.lo);
+            m[k] = __hiloint2double(v.y, v.x);               // the pair's first member in the low word
+        }
     }
 }
 
@@ -1216,8 +1314,11 @@ bool launch_chain_nc(const AdmmDev<T>& d, int32_t* chain_next, int nw, int cs, b
     geo.ldm = m_smem ? (sizeof(T) == 4 && geo.nrp % 32 == 0 ? geo.nrp + CH_RB : geo.nrp) : 0;
     geo.smem = sizeof(T) * ((size_t)geo.ldm * geo.kp + (size_t)(sizeof(T) == 8 ? 3 : 2) * NC * geo.kp +
                             (size_t)(nw + 5) * NC * geo.nrp);
-    geo.bits = fx_bits(geo.kp / (2 * nw));
-    geo.fits = 2 * (geo.bits - 28) + (geo.kp <= 64 ? 6 : 63) <= 62 ? 1 : 0;
+    if (sizeof(T) == 8) {
+        if (m_smem && geo.kp > 2 * 32 * nw) return false;   // two features a thread (their f in registers)
+        if (m_smem) geo.smem += sizeof(int32_t) * (size_t)geo.nrp;
+        while ((1 << geo.lg_terms) < geo.kp / (2 * nw)) ++geo.lg_terms;
+    }
     auto kern = k_admm_chain<T, NC>;
     int dev = 0, optin = 0, nsm = 0;
     UOI_CUDA(cudaGetDevice(&dev));
@@ -1249,21 +1350,21 @@ bool launch_chain_nc(const AdmmDev<T>& d, int32_t* chain_next, int nw, int cs, b
     }
     const int per = std::max(1, std::min((int)ceil_div(nchains, NC), resident / std::max(1, d.G)));
     cfg.gridDim = dim3((unsigned)(cs * per), (unsigned)d.G);
-    int32_t* em = chain_next + d.G;                  // exponents of the streamed M
+    int32_t* ms = chain_next + d.G;                  // scales of the streamed M
     if constexpr (sizeof(T) == 8) {
         if (!geo.ldm) {
             // the solve is M's last reader: its entries turn into their digits in place
             double* M = const_cast<double*>(d.M);
-            const int64_t pp = (int64_t)d.p * d.p;
-            k_chain_exponent<<<d.G, 256, 0, s>>>(M, d.p, em);
+            k_chain_scales<<<dim3((unsigned)ceil_div(d.p, 256), (unsigned)d.G), 256, 0, s>>>(M, d.p, d.G, ms);
             UOI_CHECK_LAUNCH();
-            k_chain_digits<<<dim3((unsigned)std::min<int64_t>(ceil_div(pp, 1024), 1024), (unsigned)d.G), 256, 0, s>>>(
-                M, pp, em, geo.bits);
+            k_chain_row_sums<<<dim3((unsigned)ceil_div(d.p, 8), (unsigned)d.G), 256, 0, s>>>(M, d.p, d.G, ms);
             UOI_CHECK_LAUNCH();
-            count_launch(2);
+            k_chain_digits<<<dim3((unsigned)std::min(d.p, 1024), (unsigned)d.G), 256, 0, s>>>(M, d.p, d.G, ms, geo.lg_terms);
+            UOI_CHECK_LAUNCH();
+            count_launch(3);
         }
     }
-    UOI_CUDA(cudaLaunchKernelEx(&cfg, kern, d, chain_next, geo, (const int32_t*)em));
+    UOI_CUDA(cudaLaunchKernelEx(&cfg, kern, d, chain_next, geo, (const int32_t*)ms));
     UOI_CHECK_LAUNCH();
     count_launch();
     return true;
@@ -1321,8 +1422,9 @@ void admm_solve(const AdmmProblem<T>& P, cudaStream_t s)
     if constexpr (sizeof(T) == 4)
         if (nchains > 4 && admm_solve_wide(P, s)) return;
     {
-        DevBuf next(sizeof(int32_t) * 2 * P.G, s);
-        UOI_CUDA(cudaMemsetAsync(next.ptr, 0, next.bytes, s));
+        // chain counters and (FP64) row-sum bounds, zero, then the exponents of a streamed M
+        DevBuf next(sizeof(int32_t) * (size_t)P.G * (2 + (sizeof(T) == 8 ? (size_t)P.p : 0)), s);
+        UOI_CUDA(cudaMemsetAsync(next.ptr, 0, sizeof(int32_t) * 2 * (size_t)P.G, s));
         if (try_resident<T>(d, next.as<int32_t>(), s)) return;
     }
     if constexpr (sizeof(T) == 4) {
@@ -1411,7 +1513,7 @@ template <typename T>
 bool admm_solve_resident_with(const AdmmProblem<T>& P, int32_t* chain_next, cudaStream_t s)
 {
     if (P.G <= 0 || P.p <= 0 || P.r <= 0 || P.q <= 0) return true;
-    if (P.p > 128) return false;                     // up to here M fits in shared memory: no exponents
+    if (P.p > 128) return false;                     // up to here M fits in shared memory: no scales
     const AdmmDev<T> d = to_dev(P);
     return try_resident<T>(d, chain_next, s);
 }

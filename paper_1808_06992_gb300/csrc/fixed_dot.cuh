@@ -1,10 +1,11 @@
 // fixed_dot.cuh -- FP64 dot products as exact integer sums.
 //
 // sum_k m_k v_k with |m| < 2^em, |v| < 2^ev: both become integers of `bits` bits (rounded once,
-// 2^-bits of their bounds), each two balanced digits of 28 bits, and three 32 x 32 + 64 -> 64
-// multiply-adds per entry sum hi hi' 2^56 + (hi lo' + lo hi') 2^28 exactly (lo lo' lies below
-// the last bit kept).  The sum is value() * 2^(em + ev - 2 bits + 56).  One multiply-add takes
-// a warp 1 clock of its SM's integer pipes; an FP64 multiply-add takes 19.
+// 2^-bits of their bounds), each two balanced digits, the lower one of `lob` bits (28 unless
+// said otherwise), and three 32 x 32 + 64 -> 64 multiply-adds per entry sum
+// hi hi' 2^(2 lob) + (hi lo' + lo hi') 2^lob exactly (lo lo' lies below the last bit kept).  The
+// sum is value() * 2^(em + ev - 2 bits + 2 lob).  One multiply-add takes a warp 1 clock of its
+// SM's integer pipes; an FP64 multiply-add takes 19.
 #pragma once
 
 #include "common.cuh"
@@ -21,7 +22,7 @@ inline int fx_bits(int terms)
 }
 
 // rint(x 2^(bits - e)) for |x| < 2^e as two digits.
-__device__ __forceinline__ int2 fx_digits(double x, int e, int bits)
+__device__ __forceinline__ int2 fx_digits(double x, int e, int bits, int lob = 28)
 {
     const long long b = __double_as_longlong(x);
     const int ex = (int)((b >> 52) & 0x7FF);
@@ -32,8 +33,8 @@ __device__ __forceinline__ int2 fx_digits(double x, int e, int bits)
     else if (sh < -54) q = 0;
     else q = (q + (1ll << (-sh - 1))) >> -sh;
     if (b < 0) q = -q;
-    const long long hi = (q + (1ll << 27)) >> 28;
-    return make_int2((int)hi, (int)(q - (hi << 28)));
+    const long long hi = (q + (1ll << (lob - 1))) >> lob;
+    return make_int2((int)hi, (int)(q - (hi << lob)));
 }
 
 // e with |x| < 2^e for values whose high word (without sign) is at most h.
@@ -46,7 +47,7 @@ __device__ __forceinline__ uint32_t fx_high(double x)
     return h == 0 && __double2loint(x) != 0 ? 1u : h;
 }
 
-// Sum of products; value(): the sum in units of 2^56, rounded.
+// Sum of products; value(): the sum in units of 2^(2 lob), rounded.
 struct FxSum {
     using Out = long long;
     long long hh = 0, mid = 0;
@@ -56,7 +57,7 @@ struct FxSum {
         mid += (long long)m.x * v.y;
         mid += (long long)m.y * v.x;
     }
-    __device__ __forceinline__ long long value() const { return hh + ((mid + (1ll << 27)) >> 28); }
+    __device__ __forceinline__ long long value(int lob = 28) const { return hh + ((mid + (1ll << (lob - 1))) >> lob); }
 };
 
 // 2^e for any e that FP64 can hold (0 or Inf past its range).
