@@ -345,6 +345,12 @@ int uoi_selftest_wait(uint64_t limit_ns, int32_t arrive, double* waited_ms, void
  * returns UOI_OK, else skips the store and returns UOI_ERR_BOUNDS. */
 int uoi_selftest_index_check(int64_t index, int64_t extent, void* stream);
 
+/* Test support for calls on a device whose memory is short (the paper has no
+ * counterpart): until it is called again, every device allocation of more than
+ * `bytes` that this library makes on the calling host thread fails as it would on
+ * a full device (UOI_ERR_OOM where the call has no smaller way).  0 ends this. */
+int uoi_selftest_alloc_limit(uint64_t bytes);
+
 /* Text of a status code (static storage). */
 const char* uoi_status_string(int status);
 

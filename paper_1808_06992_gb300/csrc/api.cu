@@ -23,11 +23,14 @@ namespace uoi {
 
 thread_local int64_t g_launches = 0;
 thread_local bool g_fit_in_batch = false;
+thread_local int32_t g_fits_at_once = 1;
+thread_local uint64_t g_alloc_limit = 0;
 
 void DevBuf::alloc(size_t n, cudaStream_t s)
 {
     release();
     if (n == 0) n = 16;
+    if (g_alloc_limit && n > g_alloc_limit) throw Error(UOI_ERR_OOM, "allocation above the limit set for a test");
     UOI_CUDA(cudaMallocAsync(&ptr, n, s));
     bytes = n;
     stream = s;
@@ -39,6 +42,8 @@ void DevBuf::release()
     ptr = nullptr;
     bytes = 0;
 }
+
+size_t scratch_share(size_t total) { return total / (size_t)std::max<int32_t>(1, g_fits_at_once); }
 
 thread_local std::string g_last_error;
 
@@ -867,10 +872,12 @@ int uoi_lasso_fit_batch(int32_t count, const double* const* X, const double* con
         std::vector<std::string> detail((size_t)count);
         std::atomic<int32_t> next(0);
         int32_t wave_end = count;
+        int32_t at_once = 1;
         uoi::AdmmBatch* batch = nullptr;
         auto worker = [&]() {
             cudaSetDevice(dev);
             uoi::g_fit_in_batch = true;
+            uoi::g_fits_at_once = at_once;
             cudaStream_t ws = nullptr;
             if (cudaStreamCreateWithFlags(&ws, cudaStreamNonBlocking) != cudaSuccess) {
                 for (int32_t t; (t = next.fetch_add(1)) < wave_end;) {
@@ -903,6 +910,7 @@ int uoi_lasso_fit_batch(int32_t count, const double* const* X, const double* con
             const int nw = grouped ? w1 - w0 : std::max(1, std::min<int32_t>(streams, count));
             next = w0;
             wave_end = w1;
+            at_once = nw;
             batch = grouped ? uoi::admm_batch_create(w1 - w0) : nullptr;
             std::vector<std::thread> pool;
             for (int w = 0; w < nw; ++w) pool.emplace_back(worker);

@@ -37,6 +37,9 @@ inline void count_launch(int64_t n = 1) { g_launches += n; }
 // True on the worker threads of a batch of fits, whose fits share the device with
 // one another (a fit then adds no concurrency of its own).
 extern thread_local bool g_fit_in_batch;
+// Fits that may run at the same time as the calling thread's, itself included: 1, or the
+// workers of its batch.
+extern thread_local int32_t g_fits_at_once;
 
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 

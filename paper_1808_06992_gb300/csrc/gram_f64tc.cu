@@ -72,6 +72,8 @@ struct OzArgs {
     const OzItem* items;
     const int32_t* cshift;          // items x max_chunks: bit of the weight each chunk stands for
     int32_t max_chunks;
+    int32_t chunk0, range;          // this launch sums the chunks chunk0 .. chunk0 + range - 1
+    int32_t add;                    // into T as it is (zero before the first range)
     long long* T;                   // items x ntiles x 2 x OZ_TN x OZ_TM
     int32_t* err;
     uint64_t wait_ns = tc::kWaitLimitNs;
@@ -116,10 +118,10 @@ k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int item = blockIdx.y;
     const int ti = a.tiles[2 * blockIdx.x], tj = a.tiles[2 * blockIdx.x + 1];
-    const int chunks = a.items[item].entries / OZ_CHUNK;
+    const int chunks = min(max(a.items[item].entries / OZ_CHUNK - a.chunk0, 0), a.range);
     const int c0 = (int)((int64_t)chunks * blockIdx.z / gridDim.z);
     const int nc = (int)((int64_t)chunks * (blockIdx.z + 1) / gridDim.z) - c0;
-    if (nc <= 0 && gridDim.z > 1) return;                // nothing to add
+    if (nc <= 0 && a.add) return;                        // nothing to add
     const int nst = nc * (OZ_CHUNK / OZ_TK);
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     if (threadIdx.x == 0) {
@@ -214,7 +216,7 @@ k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 break;
             }
             tc_fence_after();
-            const int sh = a.cshift[(int64_t)item * a.max_chunks + c0 + c];
+            const int sh = a.cshift[(int64_t)item * a.max_chunks + a.chunk0 + c0 + c];
 #pragma unroll
             for (int cb = 0; cb < NCOL; cb += 4) {
                 float v[NA][4];
@@ -239,7 +241,7 @@ k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 #pragma unroll
             for (int t = 0; t < NCOL; ++t) {
                 const int64_t o = (int64_t)(half * NCOL + t) * OZ_TM;
-                if (gridDim.z == 1) {
+                if (!a.add) {
                     out[o] = hi[t];
                     out[OZ_TILE + o] = lo[t];
                 } else {
@@ -406,23 +408,25 @@ __device__ __forceinline__ uint32_t oz_digit(uint32_t word, int byte)
 }
 
 // Gathers the listed rows, takes their digits and writes them transposed:
-// out[((item * 7 + s) * pz_pad + col) * n_pad + t].  A block covers 128 listed rows x 32
-// columns: rows are read along X's rows, the 56-bit values turned over in shared memory.
+// out[((item * 7 + s) * pz_pad + col) * n_pad + t], t counted from row list entry chunk0 * 128.  A
+// block covers 128 listed rows x 32 columns: rows are read along X's rows, the 56-bit values
+// turned over in shared memory.
 // gsx, gsy: distance of the items' operands (0: all items read the same X and Y).
 constexpr int OZ_LD = OZ_CHUNK + 2;
 __global__ void __launch_bounds__(256)
 k_oz_split(const double* __restrict__ X, int64_t ldx, int64_t gsx, const double* __restrict__ Y, int64_t ldy,
            int64_t gsy, int32_t pz_x, int32_t pz, const int32_t* __restrict__ rows, int64_t cap, const OzItem* items, const uint32_t* cmax,
-           int64_t n_pad, int32_t pz_pad, __nv_bfloat16* out)
+           int64_t n_pad, int32_t pz_pad, int32_t chunk0, __nv_bfloat16* out)
 {
     __shared__ long long tile[32][OZ_LD];
     const int item = blockIdx.x;
     const int64_t t0 = (int64_t)blockIdx.y * OZ_CHUNK;
-    if (t0 >= items[item].entries) return;               // past this item's rows: never read
+    const int64_t r0 = (int64_t)chunk0 * OZ_CHUNK + t0;
+    if (r0 >= items[item].entries) return;               // past this item's rows: never read
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = blockIdx.z * 32 + lane;
     const int e = c < pz ? oz_exponent(cmax[(int64_t)item * pz + c]) : 0;
-    const int32_t* rl = rows + (int64_t)item * cap + t0;
+    const int32_t* rl = rows + (int64_t)item * cap + r0;
     X += item * gsx;
     Y += item * gsy;
     double x[16];
@@ -593,7 +597,7 @@ void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float*
     const int ntiles = (int)tiles.size() / 2;
     const size_t per_item = (size_t)OZ_S * pz_pad * n_pad * sizeof(__nv_bfloat16);
     const size_t t_item = sizeof(long long) * 2 * OZ_TILE * (size_t)ntiles;
-    const int group = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, (8ull << 30) / (per_item + t_item)));
+    const int group = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, scratch_share(8ull << 30) / (per_item + t_item)));
     DevBuf tl(sizeof(int32_t) * tiles.size(), s), rows(sizeof(int32_t) * (size_t)n_pad, s);
     DevBuf items(sizeof(OzItem) * (size_t)B, s), cmax(sizeof(uint32_t) * (size_t)B * pz, s);
     DevBuf cshift(sizeof(int32_t) * (size_t)group * max_chunks, s);
@@ -615,7 +619,7 @@ void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float*
                            128, 0, s>>>(A + o, M + o, pz_x, cm, flags);
         UOI_CHECK_LAUNCH();
         k_oz_split<<<dim3((unsigned)nb, (unsigned)max_chunks, (unsigned)(pz_pad / 32)), 256, 0, s>>>(
-            A + o, p, p * p, M + o, p, p * p, pz_x, pz, rows.as<int32_t>(), 0, items.as<OzItem>(), cm, n_pad, pz_pad,
+            A + o, p, p * p, M + o, p, p * p, pz_x, pz, rows.as<int32_t>(), 0, items.as<OzItem>(), cm, n_pad, pz_pad, 0,
             zt.as<__nv_bfloat16>());
         UOI_CHECK_LAUNCH();
         const int splits = (int)std::max<int64_t>(
@@ -624,7 +628,8 @@ void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float*
         OzArgs a;
         a.pz = pz; a.pz_x = pz_x; a.ntiles = ntiles;
         a.tiles = tl.as<int32_t>(); a.items = items.as<OzItem>();
-        a.cshift = cshift.as<int32_t>(); a.max_chunks = max_chunks;
+        a.cshift = cshift.as<int32_t>(); a.max_chunks = a.range = max_chunks;
+        a.chunk0 = 0; a.add = splits > 1;
         a.T = T.as<long long>(); a.err = flags + 1;
         k_gram_f64tc<8><<<dim3((unsigned)ntiles, (unsigned)nb, (unsigned)splits), OZ_THREADS, OZ_SMEM, s>>>(
             oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TM),
@@ -638,14 +643,17 @@ void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float*
     count_launch();
 }
 
-void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t m, int64_t p, int64_t r,
-                 const uint32_t* w, const uint8_t* mask, int32_t B, double* G, double* Bm, int b_only,
-                 cudaStream_t s)
+namespace {
+
+constexpr size_t OZ_SCRATCH = 16ull << 30;      // slices and sums in flight
+constexpr size_t OZ_SCRATCH_MIN = 16ull << 20;
+
+// The sliced moments with at most `budget` bytes of slices and sums (one chunk of rows of one item
+// at least); false (nothing usable written) for inputs that it does not take.
+bool moments_sliced(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t m, int64_t p, int64_t r,
+                    const uint32_t* w, const uint8_t* mask, int32_t B, double* G, double* Bm, int b_only,
+                    size_t budget, cudaStream_t s)
 {
-    if (!gram_tc_available() || m > 65535ll * OZ_MAX_ROWS) {
-        moments_fp64(X, ldx, Y, ldy, m, p, r, w, mask, B, G, Bm, b_only, s);
-        return;
-    }
     const int32_t pz_x = (int32_t)p, pz = (int32_t)(p + r);
     const int32_t pz_pad = (int32_t)ceil_div(pz, OZ_TM) * OZ_TM;
     DevBuf items(sizeof(OzItem) * (size_t)B, s), cmax(sizeof(uint32_t) * (size_t)B * pz, s);
@@ -668,10 +676,8 @@ void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int
     for (const OzItem& it : hi) { entries = std::max(entries, it.entries); weight = std::max(weight, it.weight); }
     if (nonfinite || weight > OZ_MAX_WEIGHT || entries / OZ_CHUNK > 65535) {
         // Inf and NaN propagate through the plain sums; heavier weights could pass 2^63
-        moments_fp64(X, ldx, Y, ldy, m, p, r, w, mask, B, G, Bm, b_only, s);
-        return;
+        return false;
     }
-    const int64_t n_pad = entries;
     const int32_t max_chunks = entries / OZ_CHUNK;
     // tiles of the lower triangle of G and of the B block (b_only: those with a row of Y)
     std::vector<int32_t> tiles;
@@ -682,45 +688,78 @@ void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int
     const int ntiles = (int)tiles.size() / 2;
     DevBuf tl(sizeof(int32_t) * tiles.size(), s);
     UOI_CUDA(cudaMemcpyAsync(tl.ptr, tiles.data(), sizeof(int32_t) * tiles.size(), cudaMemcpyHostToDevice, s));
-    DevBuf rows(sizeof(int32_t) * (size_t)(n_pad * B), s), cshift(sizeof(int32_t) * (size_t)B * max_chunks, s);
-    k_oz_lists<<<B, 1024, 0, s>>>(w, mask, m, n_pad, max_chunks, rows.as<int32_t>(), cshift.as<int32_t>());
+    DevBuf rows(sizeof(int32_t) * (size_t)entries * B, s), cshift(sizeof(int32_t) * (size_t)B * max_chunks, s);
+    k_oz_lists<<<B, 1024, 0, s>>>(w, mask, m, entries, max_chunks, rows.as<int32_t>(), cshift.as<int32_t>());
     UOI_CHECK_LAUNCH();
     count_launch();
-    const size_t per_item = (size_t)OZ_S * pz_pad * n_pad * sizeof(__nv_bfloat16);
+    // as many items at a time as the budget holds; an item that is larger alone in ranges of its
+    // rows (integer sums: any split gives the same bits)
+    const size_t per_chunk = (size_t)OZ_S * pz_pad * OZ_CHUNK * sizeof(__nv_bfloat16);
     const size_t t_item = sizeof(long long) * 2 * OZ_TILE * (size_t)ntiles;
-    const int group = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, (16ull << 30) / (per_item + t_item)));
-    DevBuf zt(per_item * group, s), T(t_item * group, s);
+    const int group = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, budget / (per_chunk * max_chunks + t_item)));
+    const int32_t range = (int32_t)std::max<int64_t>(
+        1, std::min<int64_t>(max_chunks, ((int64_t)(budget / group) - (int64_t)t_item) / (int64_t)per_chunk));
+    const int64_t n_pad = (int64_t)range * OZ_CHUNK;
+    DevBuf zt(per_chunk * range * group, s), T(t_item * group, s);
     UOI_CUDA(cudaFuncSetAttribute(k_gram_f64tc<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
     for (int b0 = 0; b0 < B; b0 += group) {
         const int nb = std::min(group, B - b0);
         // few tiles: split the rows until every SM has one (integer sums: any split
         // gives the same bits)
         const int splits = (int)std::max<int64_t>(
-            1, std::min<int64_t>(max_chunks, 152 / std::max<int64_t>(1, (int64_t)ntiles * nb)));
-        k_oz_split<<<dim3((unsigned)nb, (unsigned)max_chunks, (unsigned)(pz_pad / 32)), 256, 0, s>>>(
-            X, ldx, 0, Y, ldy, 0, pz_x, pz, rows.as<int32_t>() + (int64_t)b0 * n_pad, n_pad, items.as<OzItem>() + b0,
-            cmax.as<uint32_t>() + (int64_t)b0 * pz, n_pad, pz_pad, zt.as<__nv_bfloat16>());
-        UOI_CHECK_LAUNCH();
-        if (splits > 1) UOI_CUDA(cudaMemsetAsync(T.ptr, 0, t_item * nb, s));
+            1, std::min<int64_t>(range, 152 / std::max<int64_t>(1, (int64_t)ntiles * nb)));
+        const bool add = splits > 1 || range < max_chunks;
+        if (add) UOI_CUDA(cudaMemsetAsync(T.ptr, 0, t_item * nb, s));
         OzArgs a;
         a.pz = pz; a.pz_x = pz_x; a.ntiles = ntiles;
         a.tiles = tl.as<int32_t>(); a.items = items.as<OzItem>() + b0;
         a.cshift = cshift.as<int32_t>() + (int64_t)b0 * max_chunks; a.max_chunks = max_chunks;
         a.T = T.as<long long>(); a.err = flags.as<int32_t>() + 1;
-        k_gram_f64tc<7><<<dim3((unsigned)ntiles, (unsigned)nb, (unsigned)splits), OZ_THREADS, OZ_SMEM, s>>>(
-            oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TM),
-            oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TN), a);
-        UOI_CHECK_LAUNCH();
+        a.add = add; a.range = range;
+        const CUtensorMap mA = oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TM);
+        const CUtensorMap mB = oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TN);
+        for (a.chunk0 = 0; a.chunk0 < max_chunks; a.chunk0 += range) {
+            k_oz_split<<<dim3((unsigned)nb, (unsigned)std::min(range, max_chunks - a.chunk0), (unsigned)(pz_pad / 32)), 256, 0, s>>>(
+                X, ldx, 0, Y, ldy, 0, pz_x, pz, rows.as<int32_t>() + (int64_t)b0 * entries, entries, items.as<OzItem>() + b0,
+                cmax.as<uint32_t>() + (int64_t)b0 * pz, n_pad, pz_pad, a.chunk0, zt.as<__nv_bfloat16>());
+            UOI_CHECK_LAUNCH();
+            k_gram_f64tc<7><<<dim3((unsigned)ntiles, (unsigned)nb, (unsigned)splits), OZ_THREADS, OZ_SMEM, s>>>(mA, mB, a);
+            UOI_CHECK_LAUNCH();
+            count_launch(2);
+        }
         k_oz_finish<<<dim3((unsigned)ntiles, (unsigned)nb, 2), 256, 0, s>>>(
             T.as<long long>(), ntiles, tl.as<int32_t>(), cmax.as<uint32_t>() + (int64_t)b0 * pz, pz, pz_x, (int32_t)r,
             b_only ? nullptr : G + (size_t)b0 * p * p, Bm + (size_t)b0 * p * r);
         UOI_CHECK_LAUNCH();
-        count_launch(3);
+        count_launch();
     }
     int32_t h = 0;
     UOI_CUDA(cudaMemcpyAsync(&h, flags.as<int32_t>() + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     UOI_CUDA(cudaStreamSynchronize(s));
     if (h) throw Error(h, "tensor-core FP64 Gram: a bounded pipeline wait expired");
+    return true;
+}
+
+}  // namespace
+
+void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t m, int64_t p, int64_t r,
+                 const uint32_t* w, const uint8_t* mask, int32_t B, double* G, double* Bm, int b_only,
+                 cudaStream_t s)
+{
+    bool done = false;
+    if (gram_tc_available() && m <= 65535ll * OZ_MAX_ROWS) {
+        // less scratch where the device has no more, and the sums that need none at the end
+        for (size_t budget = std::max(scratch_share(OZ_SCRATCH), OZ_SCRATCH_MIN); budget >= OZ_SCRATCH_MIN; budget /= 4) {
+            try {
+                done = moments_sliced(X, ldx, Y, ldy, m, p, r, w, mask, B, G, Bm, b_only, budget, s);
+                break;
+            } catch (const Error& e) {
+                if (e.status != UOI_ERR_OOM) throw;
+                cudaGetLastError();
+            }
+        }
+    }
+    if (!done) moments_fp64(X, ldx, Y, ldy, m, p, r, w, mask, B, G, Bm, b_only, s);
 }
 
 }  // namespace uoi

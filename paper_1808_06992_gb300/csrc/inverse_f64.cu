@@ -120,15 +120,10 @@ constexpr int NEWTON_MAX = 8;
 constexpr float NEWTON_LAST = 0x1p-30f;
 constexpr size_t NEWTON_SCRATCH = 2ull << 30;   // FP32 copies of the systems in flight
 
-}  // namespace
-
-bool inverse_newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A, double* M,
-                    cudaStream_t s)
+bool newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A, double* M, cudaStream_t s)
 {
-    if (p < INVERSE_NEWTON_MIN || !inverse_tc_available()) return false;
     const size_t per = 3 * sizeof(float) * (size_t)(p * p);
-    if (per > NEWTON_SCRATCH) return false;
-    const int32_t group = (int32_t)std::min<size_t>((size_t)B, NEWTON_SCRATCH / per);
+    const int32_t group = (int32_t)std::max<size_t>(1, std::min<size_t>((size_t)B, scratch_share(NEWTON_SCRATCH) / per));
     const size_t words = (size_t)group * p * p;
     DevBuf ex(sizeof(int32_t) * (size_t)(group * p), s), rowsum(sizeof(float) * (size_t)(group * p), s);
     DevBuf a32(sizeof(float) * words, s), m32(sizeof(float) * words, s), r32(sizeof(float) * words, s);
@@ -184,6 +179,21 @@ bool inverse_newton(const double* G, const double* nk, double rho, int64_t p, in
         if (!done) return false;
     }
     return true;
+}
+
+}  // namespace
+
+bool inverse_newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A, double* M,
+                    cudaStream_t s)
+{
+    if (p < INVERSE_NEWTON_MIN || 3 * sizeof(float) * (size_t)(p * p) > NEWTON_SCRATCH || !inverse_tc_available()) return false;
+    try {
+        return newton(G, nk, rho, p, B, A, M, s);
+    } catch (const Error& e) {
+        if (e.status != UOI_ERR_OOM) throw;                  // the factor needs none of the scratch
+        cudaGetLastError();
+        return false;
+    }
 }
 
 }  // namespace uoi

@@ -67,6 +67,10 @@ struct DevBuf {
     template <typename T> T* as() const { return reinterpret_cast<T*>(ptr); }
 };
 
+// What one stage of a fit may take for scratch whose size is its own choice: `total` alone on the
+// device, an equal share of it on the workers of a batch.
+size_t scratch_share(size_t total);
+
 // Allow `kern` the largest dynamic shared memory the current device opts in to (its
 // static shared memory deducted).  Kernels launched with a size that varies by call
 // use this, so that every caller sets the same value and concurrent callers on
@@ -98,7 +102,8 @@ void moments_fp64(const double* X, int64_t ldx, const double* Y, int64_t ldy, in
                   int64_t p, int64_t r, const uint32_t* w, const uint8_t* mask, int32_t B,
                   double* G, double* Bm, int b_only, cudaStream_t s);
 // The same moments in FP64 accuracy on the tensor cores (gram_f64tc.cu), where they can
-// be used: else moments_fp64.  Allocates from the pool and waits for the stream.
+// be used: else moments_fp64.  Allocates from the pool (up to scratch_share of 16 GB; less, and
+// with none moments_fp64, where the device has no more) and waits for the stream.
 void moments_f64(const double* X, int64_t ldx, const double* Y, int64_t ldy, int64_t m, int64_t p, int64_t r,
                  const uint32_t* w, const uint8_t* mask, int32_t B, double* G, double* Bm, int b_only,
                  cudaStream_t s);

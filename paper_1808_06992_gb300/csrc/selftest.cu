@@ -9,6 +9,9 @@
 // initialises an mbarrier that expects one arrival and waits for phase 0 with the
 // caller's limit.  With arrive = 0 nothing arrives, so the wait must run out;
 // with arrive = 1 the thread arrives first, so the wait must succeed at once.
+//
+// uoi_selftest_alloc_limit makes device allocations of the calling thread above a size fail
+// as they do on a full device, so that what a call does then can be seen without filling one.
 #include <cuda_runtime.h>
 
 #include "kernels.h"
@@ -47,6 +50,14 @@ __global__ void k_selftest_index(int64_t index, int64_t extent, float* buf, DevS
 }  // namespace uoi
 
 using namespace uoi;
+
+namespace uoi { extern thread_local uint64_t g_alloc_limit; }
+
+extern "C" int uoi_selftest_alloc_limit(uint64_t bytes)
+{
+    g_alloc_limit = bytes;
+    return UOI_OK;
+}
 
 extern "C" int uoi_selftest_index_check(int64_t index, int64_t extent, void* stream)
 {
