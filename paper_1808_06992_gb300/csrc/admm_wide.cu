@@ -454,7 +454,7 @@ k_admm_wide(const __grid_constant__ CUtensorMap tmM, WideArgs a)
                             nv[kk] = v;
                             const float d = x - zn, dz = zn - zp;
                             n5[0] += d * d; n5[1] += dz * dz; n5[2] += x * x; n5[3] += zn * zn; n5[4] += un * un;
-                            vs[k2] = sw != 0.f ? (zn - un) * sw : 0.f;   // an ended chain's NaN or Inf stays its own
+                            vs[k2] = (zn - un) * sw;
                         }
                         const __half2 h = __floats2half2_rn(vs[0], vs[1]);
                         const float2 hf = __half22float2(h);
@@ -481,6 +481,19 @@ k_admm_wide(const __grid_constant__ CUtensorMap tmM, WideArgs a)
                 float* nw = nrm + ((int64_t)(t & 1u) * (2 * cs) + 2 * rank + half) * 5 * WD_CHAINS + ch;
 #pragma unroll
                 for (int w = 0; w < 5; ++w) __stcg(nw + w * WD_CHAINS, n5[w]);
+                // V' of a chain that has ended is the first operand of the one that takes its lane.  NaN
+                // and Inf survive the product with sw = 0: zeros over what was stored (a select
+                // per feature in the loop above cost 2.5 % of a fit at p = 192)
+                if (__builtin_expect(sw == 0.f && !(n5[2] + n5[3] + n5[4] < 3.0e38f), 0)) {
+                    unsigned char* v = reinterpret_cast<unsigned char*>(gv + (int64_t)((t + 1) & 1u) * v_buf) + ch * 64;
+#pragma unroll 1
+                    for (int x = 0; x < FH / 4; ++x) {       // 16 bytes each: two per piece of 16 features
+                        const int k = rank * F + f0 + (x >> 2) * 16;
+                        *reinterpret_cast<uint4*>(v + (size_t)((k >> 5) * 2 + ((x >> 1) & 1)) * WD_BLOCK +
+                                                  (((k >> 4) ^ (ch >> 2)) & 1) * 32 + (x & 1) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                }
+                __syncwarp();
                 asm volatile("fence.proxy.async.global;" ::: "memory");    // the bulk copies read V'
             } else if (!go && lane == 0) {
                 *(volatile int*)&s_stop = 1;
