@@ -245,13 +245,13 @@ struct StageTimer {
     }
 };
 
-void check_status(DevStatus* st, cudaStream_t s, const char* what)
+void check_status(DevStatus* st, cudaStream_t s, const char* what, int32_t first = 0)
 {
     DevStatus h{};
     UOI_CUDA(cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s));
     UOI_CUDA(cudaStreamSynchronize(s));
     if (h.code != 0)
-        throw Error(h.code, std::string(what) + " failed on batch item " + std::to_string(h.where));
+        throw Error(h.code, std::string(what) + " failed on batch item " + std::to_string(first + h.where));
 }
 
 // prm->intercept, or 0 for a caller whose struct ends before that field.
@@ -312,6 +312,31 @@ void moments(int precision, const double* X, int64_t ldx, const double* Y, int64
         moments_f64(X, ldx, Y, ldy, m, p, r, w, mask, B, G, Bm, 0, s);
 }
 
+// M_k from the factor of G_k/n_k + rho I for the systems k with done[k] = 0, run by run.
+template <typename T>
+void factor_the_rest(const std::vector<uint8_t>& done, const double* G, bool lower_only, const double* nk, double rho,
+                     int64_t p, T* A, T* M, cudaStream_t s)
+{
+    const int32_t B = (int32_t)done.size();
+    DevBuf st(sizeof(DevStatus), s);
+    UOI_CUDA(cudaMemsetAsync(st.ptr, 0, st.bytes, s));
+    for (int32_t k = 0, n; k < B; k += n) {
+        for (n = 1; k + n < B && done[(size_t)(k + n)] == done[(size_t)k]; ++n) { }
+        if (done[(size_t)k]) continue;
+        const int64_t o = (int64_t)k * p * p;
+        if constexpr (sizeof(T) == 4) {
+            if (lower_only) build_system_lower(G + o, nk + k, rho, p, n, A + o, s);
+            else build_system<float>(G + o, nk + k, rho, p, n, A + o, s);
+            cholesky_inplace<float>(A + o, p, n, st.as<DevStatus>(), s);
+        } else {
+            build_and_factor<double>(G + o, nk + k, rho, p, n, A + o, st.as<DevStatus>(), s);
+        }
+        check_status(st.as<DevStatus>(), s, "Cholesky of G/n + rho I", k);
+        DevBuf Linv(sizeof(T) * (size_t)(n * p * p), s);
+        spd_inverse_from_factor<T>(A + o, p, n, Linv.as<T>(), M + o, s);
+    }
+}
+
 template <typename T>
 void selection_admm(int precision, const double* Xd, int64_t ldx, const double* Yd, int64_t ldy,
                     int64_t m, int64_t p, int64_t r, const uint32_t* w, int32_t B,
@@ -367,25 +392,24 @@ void selection_admm(int precision, const double* Xd, int64_t ldx, const double* 
     if constexpr (sizeof(T) == 4) {
         // mixed form: block inverse with tensor-core GEMMs
         if (tc_inverse) {
-            auto build = [&] {
-                if (lower_only)
-                    build_system_lower(G.as<double>(), nk.as<double>(), rho, p, B, A.as<float>(), s);
-                else
-                    build_system<float>(G.as<double>(), nk.as<double>(), rho, p, B, A.as<float>(), s);
-            };
-            build();
-            spd_inverse_tc(A.as<float>(), p, B, M.as<float>(), st.as<DevStatus>(), s);
+            if (lower_only)
+                build_system_lower(G.as<double>(), nk.as<double>(), rho, p, B, A.as<float>(), s);
+            else
+                build_system<float>(G.as<double>(), nk.as<double>(), rho, p, B, A.as<float>(), s);
+            DevBuf bad(sizeof(int32_t) * (size_t)B, s);
+            UOI_CUDA(cudaMemsetAsync(bad.ptr, 0, bad.bytes, s));
+            spd_inverse_tc(A.as<float>(), p, B, M.as<float>(), st.as<DevStatus>(), s, bad.as<int32_t>());
             DevStatus h{};
             UOI_CUDA(cudaMemcpyAsync(&h, st.ptr, sizeof(h), cudaMemcpyDeviceToHost, s));
             UOI_CUDA(cudaStreamSynchronize(s));
             if (h.code != 0 && p < 512) {
-                // a system at the edge of FP32: the Cholesky factor decides
-                UOI_CUDA(cudaMemsetAsync(st.ptr, 0, st.bytes, s));
-                build();
-                cholesky_inplace<float>(A.as<float>(), p, B, st.as<DevStatus>(), s);
-                check_status(st.as<DevStatus>(), s, "Cholesky of G/n + rho I");
-                DevBuf Linv(sizeof(float) * (size_t)(B * p * p), s);
-                spd_inverse_from_factor<float>(A.as<float>(), p, B, Linv.as<float>(), M.as<float>(), s);
+                // a system at the edge of FP32: its Cholesky factor decides
+                std::vector<int32_t> hb((size_t)B);
+                UOI_CUDA(cudaMemcpyAsync(hb.data(), bad.ptr, bad.bytes, cudaMemcpyDeviceToHost, s));
+                UOI_CUDA(cudaStreamSynchronize(s));
+                std::vector<uint8_t> done((size_t)B);
+                for (int32_t k = 0; k < B; ++k) done[(size_t)k] = hb[(size_t)k] ? 0 : 1;
+                factor_the_rest<float>(done, G.as<double>(), lower_only, nk.as<double>(), rho, p, A.as<float>(), M.as<float>(), s);
             } else if (h.code != 0) {
                 check_status(st.as<DevStatus>(), s, "inverse of G/n + rho I");
             }
@@ -395,9 +419,12 @@ void selection_admm(int precision, const double* Xd, int64_t ldx, const double* 
         }
     }
     if constexpr (sizeof(T) == 8) {
-        if (inverse_newton(G.as<double>(), nk.as<double>(), rho, p, B, A.as<double>(), M.as<double>(), s)) {
-            rhs_from_inverse<double>(M.as<double>(), Bm.as<double>(), nk.as<double>(), p, r, B, c.as<double>(), s);
+        const std::vector<uint8_t> done =
+            inverse_newton(G.as<double>(), nk.as<double>(), rho, p, B, A.as<double>(), M.as<double>(), s);
+        if (std::count(done.begin(), done.end(), 1) > 0) {
+            factor_the_rest<double>(done, G.as<double>(), false, nk.as<double>(), rho, p, A.as<double>(), M.as<double>(), s);
             if (!ws) G.release();
+            rhs_from_inverse<double>(M.as<double>(), Bm.as<double>(), nk.as<double>(), p, r, B, c.as<double>(), s);
             inverted = true;
         }
     }
@@ -1190,19 +1217,11 @@ int uoi_ws_dataset(const double* X, const double* Y, int64_t n, int64_t p, int64
         DevBuf nk(sizeof(double) * B, s), A(sizeof(double) * (size_t)(B * p * p), s);
         moments_f64(Xd, p, Yd, r, n, p, r, wd, nullptr, B, G.as<double>(), Bm.as<double>(), 0, s);
         weight_sums(wd, nullptr, n, B, nk.as<double>(), s);
-        DevBuf st(sizeof(DevStatus), s);
-        UOI_CUDA(cudaMemsetAsync(st.ptr, 0, st.bytes, s));
         DevBuf M(sizeof(double) * (size_t)(B * p * p), s), c(sizeof(double) * (size_t)(B * p * r), s);
-        if (inverse_newton(G.as<double>(), nk.as<double>(), rho, p, B, A.as<double>(), M.as<double>(), s)) {
-            rhs_from_inverse<double>(M.as<double>(), Bm.as<double>(), nk.as<double>(), p, r, B, c.as<double>(), s);
-        } else {
-            build_and_factor<double>(G.as<double>(), nk.as<double>(), rho, p, B, A.as<double>(),
-                                     st.as<DevStatus>(), s);
-            check_status(st.as<DevStatus>(), s, "Cholesky of G/n + rho I");
-            DevBuf Linv(sizeof(double) * (size_t)(B * p * p), s);
-            inverse_and_rhs<double>(A.as<double>(), Bm.as<double>(), nk.as<double>(), p, r, B,
-                                    Linv.as<double>(), M.as<double>(), c.as<double>(), s);
-        }
+        const std::vector<uint8_t> done =
+            inverse_newton(G.as<double>(), nk.as<double>(), rho, p, B, A.as<double>(), M.as<double>(), s);
+        factor_the_rest<double>(done, G.as<double>(), false, nk.as<double>(), rho, p, A.as<double>(), M.as<double>(), s);
+        rhs_from_inverse<double>(M.as<double>(), Bm.as<double>(), nk.as<double>(), p, r, B, c.as<double>(), s);
         DevBuf zs(sizeof(double) * (size_t)rows, s), us(sizeof(double) * (size_t)rows, s);
         AdmmProblem<double> P;
         P.G = B; P.p = p; P.r = r; P.q = q;

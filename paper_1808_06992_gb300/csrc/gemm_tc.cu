@@ -514,11 +514,16 @@ void gemm3(const Pieces& A, const Pieces& B, int32_t m, int32_t n, int32_t G, fl
 // few 16-byte reads.  Against blocked elimination in steps of 32 pivots with 1024 threads
 // (one warp inverts the diagonal block while 31 wait), 24 blocks: n = 128 88 -> 42 us, n = 192
 // 262 -> 94 us; factor stage of 24 systems p = 128 0.14 -> 0.10 ms, p = 192 0.33 -> 0.16 ms.
+struct InvStatus {
+    DevStatus* st;
+    int32_t* bad;                        // per system, 1 where a pivot was not positive (nullable)
+};
+
 __device__ __forceinline__ int sweep_index(int t, int u) { return (u >> 2) * 64 + t * 4 + (u & 3); }
 
 template <int T>
 __global__ void __launch_bounds__(256) k_spd_inverse_sweep(const float* A, int64_t lda, int64_t gsa, float* M,
-                                                           int64_t ldm, int64_t gsm, int n, int g0, DevStatus* st)
+                                                           int64_t ldm, int64_t gsm, int n, int g0, InvStatus st)
 {
     __shared__ __align__(16) float buf[2][16 * T];
     const int gi = blockIdx.x, tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -550,7 +555,10 @@ __global__ void __launch_bounds__(256) k_spd_inverse_sweep(const float* A, int64
                 __syncthreads();
                 const float d = col[c];
                 if (!(d > 0.f)) {                                      // the same in every thread
-                    if (threadIdx.x == 0) dev_fail(st, UOI_ERR_NOT_PD, g0 + gi);
+                    if (threadIdx.x == 0) {
+                        dev_fail(st.st, UOI_ERR_NOT_PD, g0 + gi);
+                        if (st.bad) st.bad[g0 + gi] = 1;
+                    }
                     return;
                 }
                 const float inv = 1.f / d;
@@ -588,7 +596,7 @@ __global__ void __launch_bounds__(256) k_spd_inverse_sweep(const float* A, int64
 }
 
 void inv_base(const float* A, int64_t ldA, int64_t gsA, float* Mout, int64_t ldM, int64_t gsM,
-              int64_t n, int32_t G, int32_t g0, DevStatus* st, cudaStream_t s)
+              int64_t n, int32_t G, int32_t g0, InvStatus st, cudaStream_t s)
 {
     const auto kern = n <= 64 ? k_spd_inverse_sweep<4> : n <= 128 ? k_spd_inverse_sweep<8> : k_spd_inverse_sweep<12>;
     kern<<<(unsigned)G, 256, 0, s>>>(A, ldA, gsA, Mout, ldM, gsM, (int)n, g0, st);
@@ -626,7 +634,7 @@ size_t inv_scratch_bytes(int64_t n, int32_t G)
 
 // g0: index of the first of the G systems in the caller's batch (for error reports).
 void inv_rec(const float* A, int64_t ldA, int64_t gsA, float* M, int64_t ldM, int64_t gsM, int64_t n,
-             int32_t G, int32_t g0, DevStatus* st, int32_t* err, InvScratch& W, cudaStream_t s)
+             int32_t G, int32_t g0, InvStatus st, int32_t* err, InvScratch& W, cudaStream_t s)
 {
     if (n <= INV_BASE) {
         inv_base(A, ldA, gsA, M, ldM, gsM, n, G, g0, st, s);
@@ -705,7 +713,7 @@ void inv_rec(const float* A, int64_t ldA, int64_t gsA, float* M, int64_t ldM, in
 
 // The recursion for G systems on stream s, with its scratch taken from one
 // allocation on s.
-void inv_chain(const float* A, int64_t p, int32_t G, int32_t g0, float* M, DevStatus* st, int32_t* err,
+void inv_chain(const float* A, int64_t p, int32_t G, int32_t g0, float* M, InvStatus st, int32_t* err,
                cudaStream_t s)
 {
     InvScratch W;
@@ -719,8 +727,9 @@ void inv_chain(const float* A, int64_t p, int32_t G, int32_t g0, float* M, DevSt
 
 bool inverse_tc_available() { return gram_tc_available(); }
 
-void spd_inverse_tc(const float* A, int64_t p, int32_t G, float* M, DevStatus* st, cudaStream_t s)
+void spd_inverse_tc(const float* A, int64_t p, int32_t G, float* M, DevStatus* status, cudaStream_t s, int32_t* bad)
 {
+    const InvStatus st{ status, bad };
     DevBuf err(sizeof(int32_t), s);
     UOI_CUDA(cudaMemsetAsync(err.ptr, 0, sizeof(int32_t), s));
     // Below the top levels the recursion is a chain of short launches (leaves of one

@@ -118,6 +118,7 @@ k_gram_f64tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int item = blockIdx.y;
     const int ti = a.tiles[2 * blockIdx.x], tj = a.tiles[2 * blockIdx.x + 1];
+    if (a.items[item].entries == 0 && NA == 8) return;   // a residual that nobody asked for
     const int chunks = min(max(a.items[item].entries / OZ_CHUNK - a.chunk0, 0), a.range);
     const int c0 = (int)((int64_t)chunks * blockIdx.z / gridDim.z);
     const int nc = (int)((int64_t)chunks * (blockIdx.z + 1) / gridDim.z) - c0;
@@ -508,24 +509,25 @@ k_oz_finish(const long long* T, int32_t ntiles, const int32_t* tiles, const uint
 // are the largest error of a sum whose terms cancel, and a Newton step cannot go below it
 // (without it c = M b came out at 1.4e-14 for p = 400, with it at the level of b).
 
-// One list of the rows 0 .. n - 1 for every item, and the items' entry counts.
-__global__ void k_oz_all_rows(int32_t n, int32_t n_pad, int32_t B, int32_t* rows, OzItem* items)
+// One list of the rows 0 .. n - 1 for every item, and the items' entry counts (none where it is
+// not active: the kernels below then leave it out).
+__global__ void k_oz_all_rows(int32_t n, int32_t n_pad, int32_t B, const int32_t* active, int32_t* rows, OzItem* items)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n_pad) rows[t] = t < n ? t : -1;
     if (t < B) {
         items[t].weight = (unsigned long long)n;
-        items[t].entries = n_pad;
+        items[t].entries = active[t] > 0 ? n_pad : 0;
     }
 }
 
 // Largest high words of the columns of A_k and of M_k (a slice of the rows per block z).
 __global__ void __launch_bounds__(128)
-k_oz_colmax_pair(const double* __restrict__ A, const double* __restrict__ M, int32_t p, uint32_t* cmax,
-                 int32_t* nonfinite)
+k_oz_colmax_pair(const double* __restrict__ A, const double* __restrict__ M, int32_t p, const OzItem* items,
+                 uint32_t* cmax)
 {
     const int item = blockIdx.y, c = blockIdx.x * 128 + threadIdx.x;
-    if (c >= 2 * p) return;
+    if (c >= 2 * p || items[item].entries == 0) return;
     const int r0 = (int)((int64_t)p * blockIdx.z / gridDim.z), r1 = (int)((int64_t)p * (blockIdx.z + 1) / gridDim.z);
     const double* src = (c < p ? A + c : M + (c - p)) + (int64_t)item * p * p;
     uint32_t h = 0;
@@ -535,22 +537,24 @@ k_oz_colmax_pair(const double* __restrict__ A, const double* __restrict__ M, int
         const uint32_t w = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
         h = max(h, w == 0 && __double2loint(x) != 0 ? 1u : w);
     }
-    if (h >= 0x7FF00000u) atomicExch(nonfinite, 1);
     if (h) atomicMax(&cmax[(int64_t)item * 2 * p + c], h);
 }
 
-// R = I - A M in FP32 and the sums of |R| over each row, 64 x 64 at a time (rows of the
-// sums are M's columns).
+// R = I - A M in FP32, 64 x 64 at a time (rows of the sums are M's columns), and the sums of |R|
+// over 32 columns of each row: part[(item * nseg + segment) * p + row], segments counted from
+// column 128 (p / 128) of Z.
 __global__ void __launch_bounds__(256)
-k_oz_residual(const long long* T, int32_t ntiles, const int32_t* tiles, const uint32_t* cmax, int32_t p, float* R,
-              float* rowsum)
+k_oz_residual(const long long* T, int32_t ntiles, const int32_t* tiles, const OzItem* items, const uint32_t* cmax, int32_t p,
+              int32_t nseg, float* R, float* part)
 {
     const int item = blockIdx.y;
+    if (items[item].entries == 0) return;
     const int ti = tiles[2 * blockIdx.x], tj = tiles[2 * blockIdx.x + 1];
     const long long* t = T + ((int64_t)item * ntiles + blockIdx.x) * (2 * OZ_TILE) + blockIdx.z * 64;
     const uint32_t* cm = cmax + (int64_t)item * 2 * p;
     const int i0 = ti * OZ_TM + blockIdx.z * 64 - p, j0 = tj * OZ_TN;      // column of M, row of A
     if (i0 + 63 < 0 || i0 >= p) return;
+    const int seg = (i0 + p - p / OZ_TM * OZ_TM) / 32;
     for (int x = threadIdx.x; x < 64 * 64; x += 256) {
         const int i = i0 + (x & 63), j = j0 + (x >> 6);
         float v = 0.f;
@@ -562,7 +566,35 @@ k_oz_residual(const long long* T, int32_t ntiles, const int32_t* tiles, const ui
             R[((int64_t)item * p + j) * p + i] = v;
         }
         const float sum = warp_sum(fabsf(v));            // a warp lies within one row
-        if ((threadIdx.x & 31) == 0 && j < p) atomicAdd(&rowsum[(int64_t)item * p + j], sum);
+        if ((threadIdx.x & 31) == 0 && j < p) part[((int64_t)item * nseg + seg + ((x >> 5) & 1)) * p + j] = sum;
+    }
+}
+
+// norm[item]: the largest row sum of |R|, each summed in the order of its segments.
+__global__ void __launch_bounds__(256)
+k_oz_norm(const float* part, const OzItem* items, const uint32_t* cmax, int32_t p, int32_t nseg, float* norm)
+{
+    __shared__ uint32_t red[8];
+    const int item = blockIdx.x;
+    if (items[item].entries == 0) return;
+    const int first = -p + p / OZ_TM * OZ_TM;            // M's column at segment 0
+    uint32_t top = 0;                                    // floats >= 0 order as their bits, NaN above all
+    for (int j = threadIdx.x; j < p; j += 256) {
+        float sum = 0.f;
+        for (int s = 0; s < nseg; ++s) {
+            const int i0 = first + s / 2 * 64;           // k_oz_residual's blocks: others wrote nothing
+            if (i0 + 63 >= 0 && i0 < p) sum += part[((int64_t)item * nseg + s) * p + j];
+        }
+        top = max(top, __float_as_uint(sum));
+    }
+    for (int c = threadIdx.x; c < 2 * p; c += 256)
+        if (cmax[(int64_t)item * 2 * p + c] >= 0x7FF00000u) top = max(top, 0x7F800000u);
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) top = max(top, red[w]);
+        norm[item] = __uint_as_float(top);
     }
 }
 
@@ -583,10 +615,10 @@ CUtensorMap oz_map(void* base, int64_t n_pad, int64_t pz_pad, int64_t depth, int
 
 }  // namespace
 
-// R_k = I - A_k M_k (FP32, p x p each) with FP64-accurate products, and the row sums of
-// |R_k|; flags[0] becomes 1 if an entry is NaN or Inf, flags[1] a pipeline error.
-void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float* R, float* rowsum, int32_t* flags,
-                  cudaStream_t s)
+// R_k = I - A_k M_k (FP32, p x p each) with FP64-accurate products and the largest row sum of
+// |R_k|; *err becomes a pipeline error.
+void residual_f64(const double* A, const double* M, int64_t p, int32_t B, const int32_t* active, float* R, float* norm,
+                  int32_t* err, cudaStream_t s)
 {
     const int32_t pz_x = (int32_t)p, pz = 2 * pz_x;
     const int32_t pz_pad = (int32_t)ceil_div(pz, OZ_TM) * OZ_TM;
@@ -597,17 +629,17 @@ void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float*
     const int ntiles = (int)tiles.size() / 2;
     const size_t per_item = (size_t)OZ_S * pz_pad * n_pad * sizeof(__nv_bfloat16);
     const size_t t_item = sizeof(long long) * 2 * OZ_TILE * (size_t)ntiles;
+    const int32_t nseg = (pz_pad - pz_x / OZ_TM * OZ_TM) / 32;
     const int group = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, scratch_share(8ull << 30) / (per_item + t_item)));
     DevBuf tl(sizeof(int32_t) * tiles.size(), s), rows(sizeof(int32_t) * (size_t)n_pad, s);
     DevBuf items(sizeof(OzItem) * (size_t)B, s), cmax(sizeof(uint32_t) * (size_t)B * pz, s);
     DevBuf cshift(sizeof(int32_t) * (size_t)group * max_chunks, s);
-    DevBuf zt(per_item * group, s), T(t_item * group, s);
+    DevBuf zt(per_item * group, s), T(t_item * group, s), part(sizeof(float) * (size_t)group * nseg * p, s);
     UOI_CUDA(cudaMemcpyAsync(tl.ptr, tiles.data(), sizeof(int32_t) * tiles.size(), cudaMemcpyHostToDevice, s));
     UOI_CUDA(cudaMemsetAsync(cmax.ptr, 0, cmax.bytes, s));
     UOI_CUDA(cudaMemsetAsync(cshift.ptr, 0, cshift.bytes, s));
-    UOI_CUDA(cudaMemsetAsync(rowsum, 0, sizeof(float) * (size_t)(B * p), s));
-    k_oz_all_rows<<<(unsigned)ceil_div(std::max<int64_t>(n_pad, B), 256), 256, 0, s>>>(pz_x, n_pad, B, rows.as<int32_t>(),
-                                                                                      items.as<OzItem>());
+    k_oz_all_rows<<<(unsigned)ceil_div(std::max<int64_t>(n_pad, B), 256), 256, 0, s>>>(
+        pz_x, n_pad, B, active, rows.as<int32_t>(), items.as<OzItem>());
     UOI_CHECK_LAUNCH();
     UOI_CUDA(cudaFuncSetAttribute(k_gram_f64tc<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
     for (int b0 = 0; b0 < B; b0 += group) {
@@ -616,10 +648,10 @@ void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float*
         uint32_t* cm = cmax.as<uint32_t>() + (int64_t)b0 * pz;
         const unsigned cb = (unsigned)ceil_div(pz, 128);
         k_oz_colmax_pair<<<dim3(cb, (unsigned)nb, (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(p, 32), 1216 / (cb * nb)))),
-                           128, 0, s>>>(A + o, M + o, pz_x, cm, flags);
+                           128, 0, s>>>(A + o, M + o, pz_x, items.as<OzItem>() + b0, cm);
         UOI_CHECK_LAUNCH();
         k_oz_split<<<dim3((unsigned)nb, (unsigned)max_chunks, (unsigned)(pz_pad / 32)), 256, 0, s>>>(
-            A + o, p, p * p, M + o, p, p * p, pz_x, pz, rows.as<int32_t>(), 0, items.as<OzItem>(), cm, n_pad, pz_pad, 0,
+            A + o, p, p * p, M + o, p, p * p, pz_x, pz, rows.as<int32_t>(), 0, items.as<OzItem>() + b0, cm, n_pad, pz_pad, 0,
             zt.as<__nv_bfloat16>());
         UOI_CHECK_LAUNCH();
         const int splits = (int)std::max<int64_t>(
@@ -627,18 +659,21 @@ void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float*
         if (splits > 1) UOI_CUDA(cudaMemsetAsync(T.ptr, 0, t_item * nb, s));
         OzArgs a;
         a.pz = pz; a.pz_x = pz_x; a.ntiles = ntiles;
-        a.tiles = tl.as<int32_t>(); a.items = items.as<OzItem>();
+        a.tiles = tl.as<int32_t>(); a.items = items.as<OzItem>() + b0;
         a.cshift = cshift.as<int32_t>(); a.max_chunks = a.range = max_chunks;
         a.chunk0 = 0; a.add = splits > 1;
-        a.T = T.as<long long>(); a.err = flags + 1;
+        a.T = T.as<long long>(); a.err = err;
         k_gram_f64tc<8><<<dim3((unsigned)ntiles, (unsigned)nb, (unsigned)splits), OZ_THREADS, OZ_SMEM, s>>>(
             oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TM),
             oz_map(zt.ptr, n_pad, pz_pad, (int64_t)OZ_S * nb, OZ_TN), a);
         UOI_CHECK_LAUNCH();
         k_oz_residual<<<dim3((unsigned)ntiles, (unsigned)nb, 2), 256, 0, s>>>(T.as<long long>(), ntiles, tl.as<int32_t>(),
-                                                                             cm, pz_x, R + o, rowsum + (int64_t)b0 * p);
+                                                                             items.as<OzItem>() + b0, cm, pz_x, nseg, R + o,
+                                                                             part.as<float>());
         UOI_CHECK_LAUNCH();
-        count_launch(4);
+        k_oz_norm<<<(unsigned)nb, 256, 0, s>>>(part.as<float>(), items.as<OzItem>() + b0, cm, pz_x, nseg, norm + b0);
+        UOI_CHECK_LAUNCH();
+        count_launch(5);
     }
     count_launch();
 }

@@ -7,9 +7,10 @@
 // products (exact integer slices on the tensor cores, gram_f64tc.cu) and adds M R: as R is
 // small, an FP32 product is enough, and the error of M falls from e to e (e + c 2^-24).  A step
 // whose residual is at most 2^-30 (largest row sum) is the last: what it leaves is below
-// 2^-52 of M.  Two steps do for condition numbers of a few hundred, three or four for 10^5.
-// A residual that starts at 1 or more, or stops shrinking, returns false and the caller takes
-// the FP64 Cholesky factor.
+// 2^-52 of M.  Each system stops on its own residual, summed in a fixed order: its bits are those
+// it has alone.  Two steps do for condition numbers of a few hundred, three or four for 10^5.
+// A system whose residual starts at 1 or more, or stops shrinking, is left to the FP64 Cholesky
+// factor.
 //
 // Why: this part's FP64 pipe takes 19 clocks per warp multiply-add, and factor, triangular
 // inverse and product need p^3 / 2 of them per system; here FP64 work is p^2 per step.
@@ -20,6 +21,7 @@
 // less (tests/test_gpu_inverse_newton.py).
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "kernels.h"
@@ -68,9 +70,14 @@ __global__ void k_widen(const float* __restrict__ src, double* __restrict__ dst,
         dst[t] = (double)src[t];
 }
 
+// What a system does with its residual.
+enum NewtonAction : int32_t { NEWTON_NONE = 0, NEWTON_STEP = 1, NEWTON_FINISH = -1 };
+
 // M += M32 R (FP32 product), M32out = M rounded.
-__global__ void __launch_bounds__(256) k_newton_step(double* M, const float* M32, const float* R, float* M32out, int64_t p)
+__global__ void __launch_bounds__(256) k_newton_step(const int32_t* action, double* M, const float* M32, const float* R,
+                                                     float* M32out, int64_t p)
 {
+    if (action[blockIdx.y] != NEWTON_STEP) return;
     const int64_t base = blockIdx.y * p * p, tt = (p + 63) / 64;
     const int64_t i0 = (blockIdx.x / tt) * 64, j0 = (blockIdx.x % tt) * 64;
     float acc[4][4] = {};
@@ -91,9 +98,10 @@ __global__ void __launch_bounds__(256) k_newton_step(double* M, const float* M32
 }
 
 // The last step: lower tiles, back to the scale of A, and their mirror.
-__global__ void __launch_bounds__(256) k_newton_last(double* M, const float* M32, const float* R, const int32_t* ex,
-                                                     int64_t p)
+__global__ void __launch_bounds__(256) k_newton_last(const int32_t* action, double* M, const float* M32, const float* R,
+                                                     const int32_t* ex, int64_t p)
 {
+    if (action[blockIdx.y] != NEWTON_FINISH) return;
     const int64_t base = blockIdx.y * p * p;
     const int32_t* e = ex + blockIdx.y * p;
     int64_t ti, tj;
@@ -120,80 +128,94 @@ constexpr int NEWTON_MAX = 8;
 constexpr float NEWTON_LAST = 0x1p-30f;
 constexpr size_t NEWTON_SCRATCH = 2ull << 30;   // FP32 copies of the systems in flight
 
-bool newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A, double* M, cudaStream_t s)
+void newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A, double* M, uint8_t* settled,
+            cudaStream_t s)
 {
     const size_t per = 3 * sizeof(float) * (size_t)(p * p);
     const int32_t group = (int32_t)std::max<size_t>(1, std::min<size_t>((size_t)B, scratch_share(NEWTON_SCRATCH) / per));
     const size_t words = (size_t)group * p * p;
-    DevBuf ex(sizeof(int32_t) * (size_t)(group * p), s), rowsum(sizeof(float) * (size_t)(group * p), s);
+    DevBuf ex(sizeof(int32_t) * (size_t)(group * p), s);
     DevBuf a32(sizeof(float) * words, s), m32(sizeof(float) * words, s), r32(sizeof(float) * words, s);
-    DevBuf st(sizeof(DevStatus) + 2 * sizeof(int32_t), s);
-    int32_t* flags = reinterpret_cast<int32_t*>(st.as<DevStatus>() + 1);
-    std::vector<float> sums((size_t)(group * p));
+    // status of the FP32 inverse and, read together: pipeline error, then per system the norm, whether
+    // its FP32 inverse failed, and its action (the residual is taken where it is to step)
+    DevBuf st(sizeof(DevStatus), s), info(sizeof(int32_t) * (size_t)(1 + 3 * group), s);
+    int32_t* err = info.as<int32_t>();
+    float* norm = reinterpret_cast<float*>(err + 1);
+    int32_t* bad = err + 1 + group;
+    int32_t* action = bad + group;
+    std::vector<int32_t> h((size_t)(1 + 2 * group)), act((size_t)group);
+    std::vector<float> prev((size_t)group);
     for (int32_t b0 = 0; b0 < B; b0 += group) {
         const int32_t nb = std::min(group, B - b0);
         const int64_t o = (int64_t)b0 * p * p, count = (int64_t)nb * p * p;
         const dim3 rows((unsigned)std::min<int64_t>(p, 1024), (unsigned)nb);
         UOI_CUDA(cudaMemsetAsync(st.ptr, 0, st.bytes, s));
+        UOI_CUDA(cudaMemsetAsync(info.ptr, 0, sizeof(int32_t) * (size_t)(1 + 2 * group), s));
         k_equil_exponents<<<(unsigned)std::min<int64_t>(ceil_div(nb * p, 256), 1024), 256, 0, s>>>(
             G + o, nk + b0, rho, p, nb, ex.as<int32_t>());
         UOI_CHECK_LAUNCH();
         k_build_equil<<<rows, 256, 0, s>>>(G + o, nk + b0, rho, p, ex.as<int32_t>(), A + o, a32.as<float>());
         UOI_CHECK_LAUNCH();
-        spd_inverse_tc(a32.as<float>(), p, nb, m32.as<float>(), st.as<DevStatus>(), s);
+        spd_inverse_tc(a32.as<float>(), p, nb, m32.as<float>(), st.as<DevStatus>(), s, bad);
         k_widen<<<(unsigned)std::min<int64_t>(ceil_div(count, 1024), 152 * 16), 256, 0, s>>>(m32.as<float>(), M + o, count);
         UOI_CHECK_LAUNCH();
         count_launch(3);
         float* cur = m32.as<float>();
         float* other = a32.as<float>();                  // A32 is read by the FP32 inverse alone
-        float prev = 1.f;
-        bool done = false;
-        for (int it = 0; it < NEWTON_MAX && !done; ++it) {
-            residual_f64(A + o, M + o, p, nb, r32.as<float>(), rowsum.as<float>(), flags, s);
-            struct { DevStatus st; int32_t flags[2]; } h;
-            static_assert(sizeof(h) == sizeof(DevStatus) + 2 * sizeof(int32_t), "read in one copy");
-            UOI_CUDA(cudaMemcpyAsync(&h, st.ptr, sizeof(h), cudaMemcpyDeviceToHost, s));
-            UOI_CUDA(cudaMemcpyAsync(sums.data(), rowsum.ptr, sizeof(float) * (size_t)(nb * p), cudaMemcpyDeviceToHost, s));
+        std::fill(prev.begin(), prev.end(), 1.f);
+        int32_t at_work = nb;
+        std::fill(act.begin(), act.begin() + nb, (int32_t)NEWTON_STEP);
+        UOI_CUDA(cudaMemcpyAsync(action, act.data(), sizeof(int32_t) * (size_t)nb, cudaMemcpyHostToDevice, s));
+        for (int it = 0; it < NEWTON_MAX && at_work > 0; ++it) {
+            residual_f64(A + o, M + o, p, nb, action, r32.as<float>(), norm, err, s);
+            UOI_CUDA(cudaMemcpyAsync(h.data(), err, sizeof(int32_t) * (size_t)(1 + 2 * group), cudaMemcpyDeviceToHost, s));
             UOI_CUDA(cudaStreamSynchronize(s));
-            if (h.flags[1]) throw Error(h.flags[1], "tensor-core FP64 residual: a bounded pipeline wait expired");
-            float norm = 0.f;
-            bool finite = h.st.code == 0 && h.flags[0] == 0;
-            for (int64_t i = 0; i < nb * p; ++i) {
-                finite = finite && std::isfinite(sums[(size_t)i]);
-                norm = std::max(norm, sums[(size_t)i]);
+            if (h[0]) throw Error(h[0], "tensor-core FP64 residual: a bounded pipeline wait expired");
+            int32_t steps = 0, last = 0;
+            for (int32_t k = 0; k < nb; ++k) {
+                int32_t& a = act[(size_t)k];
+                if (a != NEWTON_STEP) { a = NEWTON_NONE; continue; }
+                float n;
+                std::memcpy(&n, &h[(size_t)(1 + k)], sizeof(n));
+                if (h[(size_t)(1 + group + k)] || !(n < prev[(size_t)k])) a = NEWTON_NONE;     // left to the factor
+                else if (n <= NEWTON_LAST) { a = NEWTON_FINISH; settled[b0 + k] = 1; ++last; }
+                else ++steps;
+                prev[(size_t)k] = 0.5f * n;
             }
-            if (!finite || !(norm < prev)) return false;
-            done = norm <= NEWTON_LAST;
-            prev = 0.5f * norm;
+            UOI_CUDA(cudaMemcpyAsync(action, act.data(), sizeof(int32_t) * (size_t)nb, cudaMemcpyHostToDevice, s));
             const unsigned tt = (unsigned)ceil_div(p, 64);
-            if (done) {
-                k_newton_last<<<dim3(tt * (tt + 1) / 2, (unsigned)nb), 256, 0, s>>>(M + o, cur, r32.as<float>(),
+            if (last) {
+                k_newton_last<<<dim3(tt * (tt + 1) / 2, (unsigned)nb), 256, 0, s>>>(action, M + o, cur, r32.as<float>(),
                                                                                    ex.as<int32_t>(), p);
-            } else {
-                k_newton_step<<<dim3(tt * tt, (unsigned)nb), 256, 0, s>>>(M + o, cur, r32.as<float>(), other, p);
+                UOI_CHECK_LAUNCH();
+                count_launch();
+            }
+            if (steps) {
+                k_newton_step<<<dim3(tt * tt, (unsigned)nb), 256, 0, s>>>(action, M + o, cur, r32.as<float>(), other, p);
+                UOI_CHECK_LAUNCH();
+                count_launch();
                 std::swap(cur, other);
             }
-            UOI_CHECK_LAUNCH();
-            count_launch();
+            at_work = steps;
         }
-        if (!done) return false;
     }
-    return true;
 }
 
 }  // namespace
 
-bool inverse_newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A, double* M,
-                    cudaStream_t s)
+std::vector<uint8_t> inverse_newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A,
+                                    double* M, cudaStream_t s)
 {
-    if (p < INVERSE_NEWTON_MIN || 3 * sizeof(float) * (size_t)(p * p) > NEWTON_SCRATCH || !inverse_tc_available()) return false;
+    std::vector<uint8_t> settled((size_t)B, 0);
+    if (p < INVERSE_NEWTON_MIN || 3 * sizeof(float) * (size_t)(p * p) > NEWTON_SCRATCH || !inverse_tc_available())
+        return settled;
     try {
-        return newton(G, nk, rho, p, B, A, M, s);
+        newton(G, nk, rho, p, B, A, M, settled.data(), s);
     } catch (const Error& e) {
         if (e.status != UOI_ERR_OOM) throw;                  // the factor needs none of the scratch
         cudaGetLastError();
-        return false;
     }
+    return settled;
 }
 
 }  // namespace uoi

@@ -12,6 +12,7 @@
 #include <optional>
 
 #include <string>
+#include <vector>
 
 namespace uoi {
 
@@ -178,18 +179,21 @@ void rhs_from_inverse(const T* M, const double* Bm, const double* nk, int64_t p,
 // side stream (the second half enqueued by a helper thread; not on the workers of
 // a batch of fits); s waits for both.
 bool inverse_tc_available();
-void spd_inverse_tc(const float* A, int64_t p, int32_t G, float* M, DevStatus* status, cudaStream_t s);
+void spd_inverse_tc(const float* A, int64_t p, int32_t G, float* M, DevStatus* status, cudaStream_t s,
+                    int32_t* bad = nullptr);   // bad[k] = 1 where a pivot was not positive (zero before)
 // The calling host thread's second stream (estimate.cu).
 cudaStream_t side_stream();
 // M_k = (G_k/n_k + rho I)^{-1} in FP64 accuracy by Newton's iteration from the FP32 inverse
-// (inverse_f64.cu); A: B x p x p scratch.  false (nothing usable in M) when the size is not
-// its own or the iteration does not settle: the caller then takes the FP64 factor.
+// (inverse_f64.cu); A: B x p x p scratch.  Per system, 1 if it is done and 0 (nothing usable in
+// M_k) where the size is not its own or the iteration does not settle: the caller then takes the
+// FP64 factor.  A system's bits do not depend on the others.
 constexpr int64_t INVERSE_NEWTON_MIN = 64;
-bool inverse_newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A, double* M,
-                    cudaStream_t s);
-// R_k = I - A_k M_k with FP64-accurate products (gram_f64tc.cu); flags: non-finite entry, error.
-void residual_f64(const double* A, const double* M, int64_t p, int32_t B, float* R, float* rowsum, int32_t* flags,
-                  cudaStream_t s);
+std::vector<uint8_t> inverse_newton(const double* G, const double* nk, double rho, int64_t p, int32_t B, double* A,
+                                    double* M, cudaStream_t s);
+// R_k = I - A_k M_k with FP64-accurate products (gram_f64tc.cu) for the systems with active[k] > 0,
+// and norm[k], the largest row sum of |R_k| (Inf or NaN if an entry of A_k or M_k is).
+void residual_f64(const double* A, const double* M, int64_t p, int32_t B, const int32_t* active, float* R, float* norm,
+                  int32_t* err, cudaStream_t s);
 
 // M_k = A_k^{-1} from the factor L (lower triangle of A), then
 // c_k[e][i] = (M_k Bm_k)[i][e] / nk[k].
