@@ -23,7 +23,7 @@
  *  - Work is issued on prm->stream / the stream argument (NULL = the legacy
  *    default stream); every entry point returns after the results are in the
  *    output buffers (it synchronises that stream).  Some independent work also
- *    runs on a second stream the library keeps per calling thread, ordered
+ *    runs on a second stream the library keeps per calling thread and device, ordered
  *    against the caller's stream by events (the smaller supports of the
  *    estimation's loss pass; half of the selection's systems in the tensor-core
  *    inverse, enqueued by a helper thread that ends before the inverse returns;

@@ -1362,14 +1362,26 @@ __global__ void __launch_bounds__(UNION_WORDS) k_union_cols(const uint64_t* fam,
 
 }  // namespace
 
-// A second stream per host thread, for work that runs beside the thread's main
-// stream (the small-support class of the loss pass, half of the batch of the
-// tensor-core inverse); created once and kept for the thread's life.
+// A second stream per host thread and device, for work that runs beside the thread's main
+// stream (the smaller classes of the loss pass, half of the batch of the tensor-core
+// inverse, sums of the warm-start gradient); made on first use, given back when the thread ends.
 cudaStream_t side_stream()
 {
-    thread_local cudaStream_t side = nullptr;
-    if (!side) UOI_CUDA(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
-    return side;
+    struct Streams {
+        std::vector<cudaStream_t> of;                        // by device
+        ~Streams()
+        {
+            for (cudaStream_t q : of)
+                if (q) cudaStreamDestroy(q);
+        }
+    };
+    thread_local Streams streams;
+    int dev = 0;
+    UOI_CUDA(cudaGetDevice(&dev));
+    if ((size_t)dev >= streams.of.size()) streams.of.resize((size_t)dev + 1, nullptr);
+    cudaStream_t& q = streams.of[(size_t)dev];
+    if (!q) UOI_CUDA(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
+    return q;
 }
 
 int32_t union_columns(const uint64_t* family, int64_t count, int64_t p, int32_t* cols,
