@@ -567,8 +567,12 @@ double loss_grad(WsModel* M, const float* X, const float* T, int64_t N, float* g
     UOI_CHECK_LAUNCH();
     const size_t hb = sizeof(__nv_bfloat16) * (size_t)N * WS_H;
     const size_t tb = sizeof(__nv_bfloat16) * (size_t)WS_H * A.ldt;
-    DevBuf da3(hb, s), da2(hb, s), da3t(tb, s), da2t(tb, s), da1t(tb, s);
-    UOI_CUDA(cudaMemsetAsync(da1t.ptr, 0, tb, s));
+    // buffers whose last reader on s comes before their next writer there serve twice: the
+    // head has read h3 when da2 is made, the third layer's gradient h2t (its padding rows stay
+    // zero) when da1t is; 15 KB per row in all
+    DevBuf da3(hb, s), da3t(tb, s), da2t(tb, s);
+    DevBuf& da2 = A.h3;
+    DevBuf& da1t = A.h2t;
     UOI_CUDA(cudaMemsetAsync(da3t.ptr, 0, tb, s));
     UOI_CUDA(cudaMemsetAsync(da2t.ptr, 0, tb, s));
     // The row sums occupy a few SMs for the length of their chains: they run on the
