@@ -14,9 +14,11 @@
 // and G_ij = (T_hi 2^-38 + T_lo 2^-62) 2^(e_i + e_j) is rounded once at the end.
 // Errors: the rounding of z (2^-56 of the column's largest value) and the products of
 // orders 7 and up (the same size, zero-mean).  An FP64 dot product of n terms rounds
-// n partial sums; on 200..20000 standard normal rows this form's error is the smaller
-// one (tests/test_gpu_gram.py).  Sums are integers, so the split of the rows over CTAs
-// changes no bit.
+// n partial sums; on 200 and 5000 standard normal rows and 700 with columns 2^60 apart this
+// form's error is the smaller one (tests/test_gpu_gram_f64.py).  Entries too far above their
+// column's others for that (oz_spread) are zero to the slicing and their products are summed in
+// FP64 beside it.  Sums are integers, so the split of the rows over CTAs and launches changes
+// no bit.
 //
 // Weights are handled exactly too: w = sum of its bits, rows are listed once for every
 // set bit b, the lists of one bit padded to 128 rows, and a drained sum counts 2^b times.
@@ -28,7 +30,8 @@
 // Measured against the CUDA-core form (k_moments_fp64, selection moments of 20
 // bootstraps): 20000 x 1000 414 -> 10.9 ms, 5000 x 400 26.0 -> 1.05 ms, 200 x 50 0.23 ->
 // 0.13 ms; X^T Y of 192 responses x 5000 rows (the lambda grid of a VAR) 5.9 -> 0.3 ms.
-// No size was found where the CUDA-core form is the faster one.
+// No size was found where the CUDA-core form is the faster one.  Far entries: 20000 x 1000
+// exp(2 N(0,1)) 11.7 ms, exp(3 N(0,1)), 1 % of the entries, 26.4 ms (normal columns 10.9).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -265,10 +268,32 @@ __device__ __forceinline__ uint32_t oz_weight(const uint32_t* w, const uint8_t* 
     return w ? w[i] : (mask ? (mask[i] ? 1u : 0u) : 1u);
 }
 
+// A column's largest entry may lie 2^oz_spread above its typical one (the mean exponent of its
+// entries that are not zero).  Rounded against the largest value, sums of n products of
+// typical entries are off by n^(1/2) 2^-57 of that value; FP64 sums by about n 2^-54 of the
+// typical one: the slicing is the less accurate one from 2^(2.5) n^(1/2) on.  It never matters
+// to the fit (the error stays 2^-56 of the product of the columns' norms), but it does to an
+// entry of G whose other column is zero where the large values are.
+__host__ __device__ __forceinline__ int oz_spread(unsigned long long weight)
+{
+    int bits = 0;
+    while (weight) { weight >>= 1; ++bits; }
+    return 3 + bits / 2;
+}
+
+// Sum of biased exponents << 24 | number, of a column's entries that are not zero (m < 2^23).
+__device__ __forceinline__ int oz_mean_exponent(unsigned long long stat)
+{
+    const unsigned long long n = stat & 0xFFFFFFu;
+    return n ? (int)((stat >> 24) / n) : 0;
+}
+
 // Per item: the sum of the weights and the number of listed rows (the rows of each set
-// bit padded to a chunk).  One block per item.
+// bit padded to a chunk).  One block per item.  After k_oz_colmax: *spread = 1 if a column of
+// the item has entries too far above its typical ones (stat nullable).
 __global__ void __launch_bounds__(1024)
-k_oz_count(const uint32_t* w, const uint8_t* mask, int64_t m, OzItem* items)
+k_oz_count(const uint32_t* w, const uint8_t* mask, int64_t m, OzItem* items, const uint32_t* cmax, const unsigned long long* stat, int32_t pz,
+           int32_t* spread)
 {
     __shared__ unsigned s_cnt[32];
     __shared__ unsigned long long s_sum;
@@ -298,6 +323,10 @@ k_oz_count(const uint32_t* w, const uint8_t* mask, int64_t m, OzItem* items)
         items[blockIdx.x].weight = s_sum;
         items[blockIdx.x].entries = (int32_t)min(e, 0x7fffff80ull);
     }
+    if (!stat) return;
+    const int far = oz_spread(s_sum);
+    for (int c = threadIdx.x; c < pz; c += blockDim.x)
+        if ((int)(cmax[(int64_t)blockIdx.x * pz + c] >> 20) - oz_mean_exponent(stat[c]) > far) *spread = 1;
 }
 
 // The listed rows of each item, increasing within a bit, -1 as padding, and each
@@ -347,18 +376,19 @@ k_oz_lists(const uint32_t* w, const uint8_t* mask, int64_t m, int64_t cap, int32
 
 // cmax[item * pz + c] = largest high word of |z| over the rows of the item with positive
 // weight (the exponent of the column's largest value); *nonfinite = 1 if any entry is
-// NaN or Inf, whatever its weight.  A block reads 64 rows x 128 columns once and keeps
-// their high words in registers while it goes through the items.
+// NaN or Inf, whatever its weight; stat[c] as above over all rows (nullable); entries past lim
+// (nullable) count as zero.  A block reads 64
+// rows x 128 columns once and keeps their high words in registers while it goes through the items.
 constexpr int OZ_MAX_ROWS = 64;
 __global__ void __launch_bounds__(128)
 k_oz_colmax(const double* __restrict__ X, int64_t ldx, const double* __restrict__ Y, int64_t ldy, int64_t m,
             int32_t pz_x, int32_t pz, int32_t B, const uint32_t* w, const uint8_t* mask, uint32_t* cmax,
-            int32_t* nonfinite)
+            unsigned long long* stat, const int32_t* lim, int32_t* nonfinite)
 {
     const int c = blockIdx.x * 128 + threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.y * OZ_MAX_ROWS;
     const int lane = threadIdx.x & 31;
-    uint32_t h[OZ_MAX_ROWS], all = 0;
+    uint32_t h[OZ_MAX_ROWS], all = 0, exps = 0, used = 0;
 #pragma unroll
     for (int u = 0; u < OZ_MAX_ROWS; ++u) {
         const int64_t t = r0 + u;
@@ -367,8 +397,12 @@ k_oz_colmax(const double* __restrict__ X, int64_t ldx, const double* __restrict_
         h[u] = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
         // a subnormal below the high word still counts as the smallest exponent
         if (h[u] == 0 && __double2loint(x) != 0) h[u] = 1;
+        if (lim && c < pz && (int)(h[u] >> 20) > lim[c]) h[u] = 0;
         all = max(all, h[u]);
+        exps += h[u] >> 20;
+        used += h[u] ? 1u : 0u;
     }
+    if (stat && used) atomicAdd(&stat[c], (unsigned long long)exps << 24 | used);
     if (__any_sync(0xffffffffu, all >= 0x7FF00000u) && lane == 0) atomicExch(nonfinite, 1);
     for (int k = 0; k < B; ++k) {
         const int64_t o = (int64_t)k * m + r0;
@@ -381,6 +415,109 @@ k_oz_colmax(const double* __restrict__ X, int64_t ldx, const double* __restrict_
             if ((mb >> u) & 1u) mx = max(mx, h[32 + u]);
         }
         if (c < pz && mx) atomicMax(&cmax[(int64_t)k * pz + c], mx);
+    }
+}
+
+// Entries far above the typical one of their column (oz_spread) are zero to the slicing; their
+// products are summed in FP64 beside it.  lim[c]: the largest biased exponent of an ordinary entry.
+__global__ void k_oz_limits(const unsigned long long* stat, int32_t pz, int far, int32_t* lim)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < pz) lim[c] = oz_mean_exponent(stat[c]) + far;
+}
+
+__device__ __forceinline__ double oz_entry(const double* __restrict__ X, int64_t ldx, const double* __restrict__ Y, int64_t ldy,
+                                           int32_t pz_x, int64_t t, int32_t c)
+{
+    return c < pz_x ? __ldg(X + t * ldx + c) : __ldg(Y + t * ldy + (c - pz_x));
+}
+__device__ __forceinline__ bool oz_far(double x, int lim) { return (int)((__double2hiint(x) >> 20) & 0x7FF) > lim; }
+
+// The rows of each column's far entries, increasing: a warp takes 32 columns of one of OZ_SEGS runs of
+// rows.  Without `rows` it counts them into cnt[segment * pz + column], with it it lists them from
+// the place that cnt gives then (k_oz_far_places).
+constexpr int OZ_SEGS = 256;
+__global__ void __launch_bounds__(256)
+k_oz_far_entries(const double* __restrict__ X, int64_t ldx, const double* __restrict__ Y, int64_t ldy, int64_t m, int32_t pz_x,
+                 int32_t pz, const int32_t* lim, int64_t* cnt, int32_t* rows)
+{
+    const int seg = blockIdx.y * 8 + (threadIdx.x >> 5), c = blockIdx.x * 32 + (threadIdx.x & 31);
+    if (c >= pz) return;
+    const int64_t t0 = m * seg / OZ_SEGS, t1 = m * (seg + 1) / OZ_SEGS;
+    const int l = lim[c];
+    int64_t at = rows ? cnt[(int64_t)seg * pz + c] : 0;
+#pragma unroll 4
+    for (int64_t t = t0; t < t1; ++t)
+        if (oz_far(oz_entry(X, ldx, Y, ldy, pz_x, t, c), l)) {
+            if (rows) rows[at] = (int32_t)t;
+            ++at;
+        }
+    if (!rows) cnt[(int64_t)seg * pz + c] = at;
+}
+
+// Counts -> places: column after column, segment after segment; first[c] .. first[c + 1] - 1 are
+// column c's.  One block.
+__global__ void __launch_bounds__(1024) k_oz_far_places(int64_t* cnt, int32_t pz, int64_t* first)
+{
+    __shared__ int64_t tot[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int64_t base = 0;                                    // the same in every thread
+    for (int c0 = 0; c0 < pz; c0 += 1024) {
+        const int c = c0 + threadIdx.x;
+        int64_t n = 0;
+        if (c < pz)
+            for (int s = 0; s < OZ_SEGS; ++s) n += cnt[(int64_t)s * pz + c];
+        int64_t inc = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        __syncthreads();                                 // the previous totals have been read
+        if (lane == 31) tot[wid] = inc;
+        __syncthreads();
+        int64_t at = base + inc - n;
+        for (int k = 0; k < 32; ++k) {
+            if (k < wid) at += tot[k];
+            base += tot[k];
+        }
+        if (c < pz) {
+            first[c] = at;
+            for (int s = 0; s < OZ_SEGS; ++s) {
+                const int64_t v = cnt[(int64_t)s * pz + c];
+                cnt[(int64_t)s * pz + c] = at;
+                at += v;
+            }
+        }
+    }
+    if (threadIdx.x == 0) first[pz] = base;
+}
+
+// S[item][i][j] = sum over the far entries f of column i, in row order, of w f z_j: z_j whole for
+// j <= i, without column j's own far entries for j > i, so that every product with a far entry
+// stands in one of S[i][j] and S[j][i].  A block per column i and item; b_only: the pairs with a
+// column of Y.  Columns without far entries are not written.
+__global__ void __launch_bounds__(256)
+k_oz_far_sums(const double* __restrict__ X, int64_t ldx, const double* __restrict__ Y, int64_t ldy, int64_t m, int32_t pz_x,
+              int32_t pz, const uint32_t* w, const uint8_t* mask, const int32_t* lim, const int64_t* first, const int32_t* rows,
+              int b_only, double* S)
+{
+    const int i = blockIdx.x, item = blockIdx.y;
+    const int64_t n0 = first[i], n1 = first[i + 1];
+    if (n0 == n1) return;
+    double* out = S + ((int64_t)item * pz + i) * pz;
+    for (int j = threadIdx.x; j < pz; j += 256) {
+        if (i >= pz_x ? j >= pz_x : (b_only && j < pz_x)) continue;
+        double sum = 0.0;
+        for (int64_t e = n0; e < n1; ++e) {
+            const int64_t t = rows[e];
+            const uint32_t wt = oz_weight(w, mask, (int64_t)item * m + t);
+            if (wt == 0) continue;
+            const double z = oz_entry(X, ldx, Y, ldy, pz_x, t, j);
+            if (j > i && oz_far(z, lim[j])) continue;
+            sum += (double)wt * oz_entry(X, ldx, Y, ldy, pz_x, t, i) * z;
+        }
+        out[j] = sum;
     }
 }
 
@@ -417,7 +554,7 @@ constexpr int OZ_LD = OZ_CHUNK + 2;
 __global__ void __launch_bounds__(256)
 k_oz_split(const double* __restrict__ X, int64_t ldx, int64_t gsx, const double* __restrict__ Y, int64_t ldy,
            int64_t gsy, int32_t pz_x, int32_t pz, const int32_t* __restrict__ rows, int64_t cap, const OzItem* items, const uint32_t* cmax,
-           int64_t n_pad, int32_t pz_pad, int32_t chunk0, __nv_bfloat16* out)
+           int64_t n_pad, int32_t pz_pad, int32_t chunk0, const int32_t* lim, __nv_bfloat16* out)
 {
     __shared__ long long tile[32][OZ_LD];
     const int item = blockIdx.x;
@@ -436,6 +573,12 @@ k_oz_split(const double* __restrict__ X, int64_t ldx, int64_t gsx, const double*
         const int64_t row = rl[warp * 16 + i];
         x[i] = 0.0;
         if (row >= 0 && c < pz) x[i] = c < pz_x ? __ldg(X + row * ldx + c) : __ldg(Y + row * ldy + (c - pz_x));
+    }
+    if (lim && c < pz) {
+        const int l = lim[c];
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (oz_far(x[i], l)) x[i] = 0.0;
     }
 #pragma unroll
     for (int i = 0; i < 16; ++i) tile[lane][warp * 16 + i] = oz_fixed(x[i], e);
@@ -467,11 +610,12 @@ k_oz_split(const double* __restrict__ X, int64_t ldx, int64_t gsx, const double*
     }
 }
 
-// Integer sums -> FP64 outputs, 64 x 64 at a time: the lower triangle of G along its
-// rows (turned over in shared memory), its mirror along the sums' own order, and Bm.
+// Integer sums (and the far entries' sums S, nullable) -> FP64 outputs, 64 x 64 at a time: the
+// lower triangle of G along its rows (turned over in shared memory), its mirror along the sums'
+// own order, and Bm.
 __global__ void __launch_bounds__(256)
 k_oz_finish(const long long* T, int32_t ntiles, const int32_t* tiles, const uint32_t* cmax, int32_t pz, int32_t pz_x,
-            int32_t r, double* G, double* Bm)
+            int32_t r, const double* S, const int64_t* first, double* G, double* Bm)
 {
     __shared__ double v[64][65];
     const int item = blockIdx.y;
@@ -488,6 +632,12 @@ k_oz_finish(const long long* T, int32_t ntiles, const int32_t* tiles, const uint
             const long long lo = t[OZ_TILE + (int64_t)(x >> 6) * OZ_TM + (x & 63)];
             const int e = oz_exponent(cm[i]) + oz_exponent(cm[j]);
             val = scalbn(fma((double)lo, 0x1p-24, (double)hi), e - 38);
+            if (S && j <= i) {
+                const double* sk = S + (int64_t)item * pz * pz;
+                const double a = first[i] < first[i + 1] ? sk[(int64_t)i * pz + j] : 0.0;
+                const double b = j < i && first[j] < first[j + 1] ? sk[(int64_t)j * pz + i] : 0.0;
+                val += a + b;
+            }
             if (G && i < pz_x && j < i) G[((int64_t)item * pz_x + j) * pz_x + i] = val;
         }
         v[x & 63][x >> 6] = val;
@@ -652,7 +802,7 @@ void residual_f64(const double* A, const double* M, int64_t p, int32_t B, const 
         UOI_CHECK_LAUNCH();
         k_oz_split<<<dim3((unsigned)nb, (unsigned)max_chunks, (unsigned)(pz_pad / 32)), 256, 0, s>>>(
             A + o, p, p * p, M + o, p, p * p, pz_x, pz, rows.as<int32_t>(), 0, items.as<OzItem>() + b0, cm, n_pad, pz_pad, 0,
-            zt.as<__nv_bfloat16>());
+            nullptr, zt.as<__nv_bfloat16>());
         UOI_CHECK_LAUNCH();
         const int splits = (int)std::max<int64_t>(
             1, std::min<int64_t>(max_chunks, 152 / std::max<int64_t>(1, (int64_t)ntiles * nb)));
@@ -682,6 +832,9 @@ namespace {
 
 constexpr size_t OZ_SCRATCH = 16ull << 30;      // slices and sums in flight
 constexpr size_t OZ_SCRATCH_MIN = 16ull << 20;
+// One entry in so many may be far above its column's others (each costs p FP64 products per
+// item); past that all sums are plain.
+constexpr int64_t OZ_FAR_SHARE = 32;
 
 // The sliced moments with at most `budget` bytes of slices and sums (one chunk of rows of one item
 // at least); false (nothing usable written) for inputs that it does not take.
@@ -692,27 +845,59 @@ bool moments_sliced(const double* X, int64_t ldx, const double* Y, int64_t ldy, 
     const int32_t pz_x = (int32_t)p, pz = (int32_t)(p + r);
     const int32_t pz_pad = (int32_t)ceil_div(pz, OZ_TM) * OZ_TM;
     DevBuf items(sizeof(OzItem) * (size_t)B, s), cmax(sizeof(uint32_t) * (size_t)B * pz, s);
-    DevBuf flags(2 * sizeof(int32_t), s);                // non-finite input, pipeline error
-    UOI_CUDA(cudaMemsetAsync(cmax.ptr, 0, cmax.bytes, s));
-    UOI_CUDA(cudaMemsetAsync(flags.ptr, 0, flags.bytes, s));
-    k_oz_count<<<B, 1024, 0, s>>>(w, mask, m, items.as<OzItem>());
-    UOI_CHECK_LAUNCH();
-    k_oz_colmax<<<dim3((unsigned)ceil_div(pz, 128), (unsigned)ceil_div(m, OZ_MAX_ROWS)), 128, 0, s>>>(
-        X, ldx, Y, ldy, m, pz_x, pz, B, w, mask, cmax.as<uint32_t>(), flags.as<int32_t>());
-    UOI_CHECK_LAUNCH();
-    count_launch(2);
+    DevBuf flags(3 * sizeof(int32_t), s);                // non-finite input, pipeline error, wide columns
+    DevBuf stat(sizeof(unsigned long long) * (size_t)pz, s), lim, first, far_rows;
     std::vector<OzItem> hi((size_t)B);
-    int32_t nonfinite = 0;
-    UOI_CUDA(cudaMemcpyAsync(hi.data(), items.ptr, sizeof(OzItem) * (size_t)B, cudaMemcpyDeviceToHost, s));
-    UOI_CUDA(cudaMemcpyAsync(&nonfinite, flags.ptr, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    UOI_CUDA(cudaStreamSynchronize(s));
-    int32_t entries = OZ_CHUNK;
-    unsigned long long weight = 0;
-    for (const OzItem& it : hi) { entries = std::max(entries, it.entries); weight = std::max(weight, it.weight); }
-    if (nonfinite || weight > OZ_MAX_WEIGHT || entries / OZ_CHUNK > 65535) {
-        // Inf and NaN propagate through the plain sums; heavier weights could pass 2^63
-        return false;
+    int32_t entries = OZ_CHUNK, hf[3] = {};
+    unsigned long long weight = 0, least = ~0ull;
+    auto look = [&](unsigned long long* st, const int32_t* limits) {
+        UOI_CUDA(cudaMemsetAsync(cmax.ptr, 0, cmax.bytes, s));
+        UOI_CUDA(cudaMemsetAsync(flags.ptr, 0, flags.bytes, s));
+        if (st) UOI_CUDA(cudaMemsetAsync(st, 0, stat.bytes, s));
+        k_oz_colmax<<<dim3((unsigned)ceil_div(pz, 128), (unsigned)ceil_div(m, OZ_MAX_ROWS)), 128, 0, s>>>(
+            X, ldx, Y, ldy, m, pz_x, pz, B, w, mask, cmax.as<uint32_t>(), st, limits, flags.as<int32_t>());
+        UOI_CHECK_LAUNCH();
+        k_oz_count<<<B, 1024, 0, s>>>(w, mask, m, items.as<OzItem>(), cmax.as<uint32_t>(), st, pz, flags.as<int32_t>() + 2);
+        UOI_CHECK_LAUNCH();
+        count_launch(2);
+        UOI_CUDA(cudaMemcpyAsync(hi.data(), items.ptr, sizeof(OzItem) * (size_t)B, cudaMemcpyDeviceToHost, s));
+        UOI_CUDA(cudaMemcpyAsync(hf, flags.ptr, sizeof(hf), cudaMemcpyDeviceToHost, s));
+        UOI_CUDA(cudaStreamSynchronize(s));
+        entries = OZ_CHUNK;
+        for (const OzItem& it : hi) {
+            entries = std::max(entries, it.entries);
+            weight = std::max(weight, it.weight);
+            if (it.weight) least = std::min(least, it.weight);
+        }
+    };
+    look(stat.as<unsigned long long>(), nullptr);
+    // Inf and NaN propagate through the plain sums; heavier weights could pass 2^63
+    if (hf[0] || weight > OZ_MAX_WEIGHT) return false;
+    const bool far = hf[2] != 0;
+    if (far) {
+        lim.alloc(sizeof(int32_t) * (size_t)pz, s);
+        first.alloc(sizeof(int64_t) * (size_t)(pz + 1), s);
+        DevBuf cnt(sizeof(int64_t) * (size_t)OZ_SEGS * pz, s);
+        const dim3 grid((unsigned)ceil_div(pz, 32), OZ_SEGS / 8);
+        k_oz_limits<<<(unsigned)ceil_div(pz, 256), 256, 0, s>>>(stat.as<unsigned long long>(), pz, oz_spread(least), lim.as<int32_t>());
+        UOI_CHECK_LAUNCH();
+        k_oz_far_entries<<<grid, 256, 0, s>>>(X, ldx, Y, ldy, m, pz_x, pz, lim.as<int32_t>(), cnt.as<int64_t>(), nullptr);
+        UOI_CHECK_LAUNCH();
+        k_oz_far_places<<<1, 1024, 0, s>>>(cnt.as<int64_t>(), pz, first.as<int64_t>());
+        UOI_CHECK_LAUNCH();
+        int64_t n = 0;
+        UOI_CUDA(cudaMemcpyAsync(&n, first.as<int64_t>() + pz, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        UOI_CUDA(cudaStreamSynchronize(s));
+        count_launch(3);
+        if (n > m * (int64_t)pz / OZ_FAR_SHARE) return false;
+        far_rows.alloc(sizeof(int32_t) * (size_t)std::max<int64_t>(n, 1), s);
+        k_oz_far_entries<<<grid, 256, 0, s>>>(X, ldx, Y, ldy, m, pz_x, pz, lim.as<int32_t>(), cnt.as<int64_t>(),
+                                              far_rows.as<int32_t>());
+        UOI_CHECK_LAUNCH();
+        count_launch();
+        look(nullptr, lim.as<int32_t>());
     }
+    if (entries / OZ_CHUNK > 65535) return false;
     const int32_t max_chunks = entries / OZ_CHUNK;
     // tiles of the lower triangle of G and of the B block (b_only: those with a row of Y)
     std::vector<int32_t> tiles;
@@ -730,12 +915,14 @@ bool moments_sliced(const double* X, int64_t ldx, const double* Y, int64_t ldy, 
     // as many items at a time as the budget holds; an item that is larger alone in ranges of its
     // rows (integer sums: any split gives the same bits)
     const size_t per_chunk = (size_t)OZ_S * pz_pad * OZ_CHUNK * sizeof(__nv_bfloat16);
-    const size_t t_item = sizeof(long long) * 2 * OZ_TILE * (size_t)ntiles;
+    const size_t s_item = far ? sizeof(double) * (size_t)pz * pz : 0;
+    const size_t t_item = sizeof(long long) * 2 * OZ_TILE * (size_t)ntiles + s_item;
     const int group = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, budget / (per_chunk * max_chunks + t_item)));
     const int32_t range = (int32_t)std::max<int64_t>(
         1, std::min<int64_t>(max_chunks, ((int64_t)(budget / group) - (int64_t)t_item) / (int64_t)per_chunk));
     const int64_t n_pad = (int64_t)range * OZ_CHUNK;
-    DevBuf zt(per_chunk * range * group, s), T(t_item * group, s);
+    DevBuf zt(per_chunk * range * group, s), T((t_item - s_item) * group, s), S;
+    if (far) S.alloc(s_item * group, s);
     UOI_CUDA(cudaFuncSetAttribute(k_gram_f64tc<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
     for (int b0 = 0; b0 < B; b0 += group) {
         const int nb = std::min(group, B - b0);
@@ -744,7 +931,7 @@ bool moments_sliced(const double* X, int64_t ldx, const double* Y, int64_t ldy, 
         const int splits = (int)std::max<int64_t>(
             1, std::min<int64_t>(range, 152 / std::max<int64_t>(1, (int64_t)ntiles * nb)));
         const bool add = splits > 1 || range < max_chunks;
-        if (add) UOI_CUDA(cudaMemsetAsync(T.ptr, 0, t_item * nb, s));
+        if (add) UOI_CUDA(cudaMemsetAsync(T.ptr, 0, (t_item - s_item) * nb, s));
         OzArgs a;
         a.pz = pz; a.pz_x = pz_x; a.ntiles = ntiles;
         a.tiles = tl.as<int32_t>(); a.items = items.as<OzItem>() + b0;
@@ -756,15 +943,23 @@ bool moments_sliced(const double* X, int64_t ldx, const double* Y, int64_t ldy, 
         for (a.chunk0 = 0; a.chunk0 < max_chunks; a.chunk0 += range) {
             k_oz_split<<<dim3((unsigned)nb, (unsigned)std::min(range, max_chunks - a.chunk0), (unsigned)(pz_pad / 32)), 256, 0, s>>>(
                 X, ldx, 0, Y, ldy, 0, pz_x, pz, rows.as<int32_t>() + (int64_t)b0 * entries, entries, items.as<OzItem>() + b0,
-                cmax.as<uint32_t>() + (int64_t)b0 * pz, n_pad, pz_pad, a.chunk0, zt.as<__nv_bfloat16>());
+                cmax.as<uint32_t>() + (int64_t)b0 * pz, n_pad, pz_pad, a.chunk0, lim.as<int32_t>(),
+                zt.as<__nv_bfloat16>());
             UOI_CHECK_LAUNCH();
             k_gram_f64tc<7><<<dim3((unsigned)ntiles, (unsigned)nb, (unsigned)splits), OZ_THREADS, OZ_SMEM, s>>>(mA, mB, a);
             UOI_CHECK_LAUNCH();
             count_launch(2);
         }
+        if (far) {
+            k_oz_far_sums<<<dim3((unsigned)pz, (unsigned)nb), 256, 0, s>>>(
+                X, ldx, Y, ldy, m, pz_x, pz, w ? w + (int64_t)b0 * m : nullptr, mask ? mask + (int64_t)b0 * m : nullptr,
+                lim.as<int32_t>(), first.as<int64_t>(), far_rows.as<int32_t>(), b_only, S.as<double>());
+            UOI_CHECK_LAUNCH();
+            count_launch();
+        }
         k_oz_finish<<<dim3((unsigned)ntiles, (unsigned)nb, 2), 256, 0, s>>>(
             T.as<long long>(), ntiles, tl.as<int32_t>(), cmax.as<uint32_t>() + (int64_t)b0 * pz, pz, pz_x, (int32_t)r,
-            b_only ? nullptr : G + (size_t)b0 * p * p, Bm + (size_t)b0 * p * r);
+            S.as<double>(), first.as<int64_t>(), b_only ? nullptr : G + (size_t)b0 * p * p, Bm + (size_t)b0 * p * r);
         UOI_CHECK_LAUNCH();
         count_launch();
     }
