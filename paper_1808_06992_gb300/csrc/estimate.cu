@@ -409,8 +409,9 @@ struct OlsWarpSmem {
     float buf[2][32];
     int idx[32], ex[32];
 };
-__global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits)
+__global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a)
 {
+    constexpr int BITS = 57, LOB = 29;                      // sums of 32 products fit 62 bits
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     OlsWarpSmem& m = reinterpret_cast<OlsWarpSmem*>(smem_raw)[warp];
@@ -443,7 +444,7 @@ __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits
         __syncwarp();
         bool bad = hb == OLS_EXP_NONFINITE;                  // scaled entries of G at 1 or above: below
         float g[32];
-        const float unit = __uint_as_float((uint32_t)(127 + 28 - bits) << 23);
+        constexpr float unit = 1.f / (float)(1 << (BITS - LOB));
 #pragma unroll
         for (int c0 = 0; c0 < 32; c0 += 8) {
             if (c0 < s) {
@@ -454,7 +455,7 @@ __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int ev = e + m.ex[c0 + i];
-                    const int2 d = fx_digits(v[i], ev, bits);
+                    const int2 d = fx_digits(v[i], ev, BITS, LOB);
                     bad |= ols_exceeds(v[i], ev);
                     if (in && c0 + i < s) Gd[(c0 + i) * s + lane] = d;
                     g[c0 + i] = (float)d.x * unit;
@@ -516,13 +517,13 @@ __global__ void __launch_bounds__(32 * OLS_WARPS) k_ols_warp(OlsArgs a, int bits
                 if (st) { done = st > 0; break; }
                 prev = dmx;
                 const int ev = hx ? fx_exponent(hx) : 0;
-                m.xd[lane] = fx_digits(x, ev, bits);
+                m.xd[lane] = fx_digits(x, ev, BITS, LOB);
                 __syncwarp();
-                FxSum sum;
+                FxFull sum;
                 if (in)
 #pragma unroll 4
                     for (int c = 0; c < s; ++c) sum.add(Gd[c * s + lane], m.xd[c]);
-                w = f64_to_f32_int(fma(-fx_pow2(ev - 2 * bits + 56), (double)sum.value(), bs));
+                w = f64_to_f32_int(fx_residual(bs, sum.hh, sum.low(LOB), ev - 2 * BITS, LOB));
             }
         }
         if (s > 0 && !done) {
@@ -560,6 +561,7 @@ template <int T>
 struct OlsBlockSmem {
     double bs[16 * T], x[16 * T];
     long long part[256];
+    double part_low[256];
     int2 xd[16 * T];
     float buf[2][16 * T], w[16 * T], y[16 * T], thr[16 * T];
     int idx[16 * T], ex[16 * T];
@@ -576,8 +578,9 @@ __global__ void __launch_bounds__(256, T == 4 ? 4 : 2) k_ols_block(OlsArgs a)
     OlsBlockSmem<T>& m = *reinterpret_cast<OlsBlockSmem<T>*>(smem_raw);
     int2* Gd = reinterpret_cast<int2*>(smem_raw + sizeof(OlsBlockSmem<T>));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tx = tid & 15, ty = tid >> 4;
-    constexpr int bits = 55;                                 // sums of 128 products fit
-    constexpr float unit = 1.f / (float)(1 << (bits - 28));
+    // upper digits: sums of all 16 T products fit 62 bits; the others: sums of one part's
+    constexpr int BITS = T == 4 ? 58 : 56, LOB = T == 4 ? 30 : 29;
+    constexpr float unit = 1.f / (float)(1 << (BITS - LOB));
     auto fetch = [&](int64_t t) -> int64_t {
         if (!a.next) return t < 0 ? (int64_t)blockIdx.x : t + gridDim.x;
         __syncthreads();
@@ -632,7 +635,7 @@ __global__ void __launch_bounds__(256, T == 4 ? 4 : 2) k_ols_block(OlsArgs a)
             for (int i = 0; i < R / 32; ++i) {
                 const int ev = m.ex[c] + m.ex[lane + 32 * i];
                 bad |= ols_exceeds(v[i], ev);
-                if (lane + 32 * i < s) Gd[c * s + lane + 32 * i] = fx_digits(v[i], ev, bits);
+                if (lane + 32 * i < s) Gd[c * s + lane + 32 * i] = fx_digits(v[i], ev, BITS, LOB);
             }
         }
         const double bs = scalbn(b, -e - eb);
@@ -712,21 +715,26 @@ __global__ void __launch_bounds__(256, T == 4 ? 4 : 2) k_ols_block(OlsArgs a)
                 if (st) { done = st > 0; break; }
                 prev = dmx;
                 const int ev = hx ? fx_exponent(hx) : 0;
-                if (tid < s) m.xd[tid] = fx_digits(x, ev, bits);
+                if (tid < s) m.xd[tid] = fx_digits(x, ev, BITS, LOB);
                 __syncthreads();
                 const int row = tid % R, part = tid / R;
                 if (row < s) {
-                    FxSum sum;
+                    FxFull sum;
 #pragma unroll 4
                     for (int c = part; c < s; c += PARTS) sum.add(Gd[c * s + row], m.xd[c]);
-                    m.part[tid] = sum.value();
+                    m.part[tid] = sum.hh;
+                    m.part_low[tid] = sum.low(LOB);
                 }
                 __syncthreads();
                 if (tid < s) {
                     long long q = 0;
+                    double low = 0.0;
 #pragma unroll
-                    for (int k = 0; k < PARTS; ++k) q += m.part[k * R + tid];
-                    m.w[tid] = f64_to_f32_int(fma(-fx_pow2(ev - 2 * bits + 56), (double)q, m.bs[tid]));
+                    for (int k = 0; k < PARTS; ++k) {
+                        q += m.part[k * R + tid];
+                        low += m.part_low[k * R + tid];
+                    }
+                    m.w[tid] = f64_to_f32_int(fx_residual(m.bs[tid], q, low, ev - 2 * BITS, LOB));
                 }
             }
         }
@@ -1279,7 +1287,7 @@ void launch_ols_class(OlsArgs a, int cls, DevBuf& fscratch, cudaStream_t s)
     allow_max_dynamic_smem(kern);
     UOI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem));
     const int grid = (int)std::min<int64_t>(work, (int64_t)nsm * std::max(1, per));
-    if (cls == 0) k_ols_warp<<<grid, threads, smem, s>>>(a, fx_bits(32));
+    if (cls == 0) k_ols_warp<<<grid, threads, smem, s>>>(a);
     else if (cls == 1) k_ols_block<4><<<grid, threads, smem, s>>>(a);
     else if (cls == 2) k_ols_block<8><<<grid, threads, smem, s>>>(a);
     else k_ols_mixed<<<grid, threads, smem, s>>>(a);

@@ -12,15 +12,6 @@
 
 namespace uoi {
 
-// Bits of Q and P below the sign, at most 56: `terms` products of their upper digits fit
-// 61 bits.
-inline int fx_bits(int terms)
-{
-    int lg = 0;
-    while ((1 << lg) < terms) ++lg;
-    return 28 + (61 - (lg < 5 ? 5 : lg)) / 2;
-}
-
 // rint(x 2^(bits - e)) for |x| < 2^e as two digits.
 __device__ __forceinline__ int2 fx_digits(double x, int e, int bits, int lob = 28)
 {
@@ -60,10 +51,33 @@ struct FxSum {
     __device__ __forceinline__ long long value(int lob = 28) const { return hh + ((mid + (1ll << (lob - 1))) >> lob); }
 };
 
+// All four products: the sum is hh 2^(2 lob) + low(lob), the first exact, the second rounded at
+// 2^-53 of itself.
+struct FxFull {
+    long long hh = 0, mid = 0, ll = 0;
+    __device__ __forceinline__ void add(int2 m, int2 v)
+    {
+        hh += (long long)m.x * v.x;
+        mid += (long long)m.x * v.y;
+        mid += (long long)m.y * v.x;
+        ll += (long long)m.y * v.y;
+    }
+    __device__ __forceinline__ double low(int lob) const { return fma((double)mid, (double)(1ll << lob), (double)ll); }
+};
+
 // 2^e for any e that FP64 can hold (0 or Inf past its range).
 __device__ __forceinline__ double fx_pow2(int e)
 {
     return e > -1023 && e < 1024 ? __longlong_as_double((long long)(e + 1023) << 52) : scalbn(1.0, e);
+}
+
+// b - 2^e (hh 2^(2 lob) + low): the digits of hh go in one after the other, so that nothing but
+// the result is rounded where it cancels against b.
+__device__ __forceinline__ double fx_residual(double b, long long hh, double low, int e, int lob)
+{
+    b = fma(-fx_pow2(e + 2 * lob + 32), (double)(int)(hh >> 32), b);
+    b = fma(-fx_pow2(e + 2 * lob), (double)(uint32_t)hh, b);
+    return fma(-fx_pow2(e), low, b);
 }
 
 }  // namespace uoi
