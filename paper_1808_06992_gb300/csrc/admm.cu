@@ -14,7 +14,8 @@
 // Schedules:
 //  * chain (FP64, and FP32 with few chains): one cluster of CTAs iterates one chain
 //    (or four) at a time from start to end in a single launch, see k_admm_chain.
-//  * resident (FP32, p <= 192, many chains): one CTA keeps M_g in shared
+//  * wide (FP32, many chains, 64 < p <= 512): admm_wide.cu.
+//  * resident (FP32, many chains, p <= 64; with a given start p <= 192): one CTA keeps M_g in shared
 //    memory; each warp runs its own chains to completion with no block-wide
 //    barrier (the warp only reads its own columns of V = z - u), pulling new
 //    chains from a per-group counter.  One launch solves everything.

@@ -1,5 +1,5 @@
 // admm_wide.cu -- G4 for many FP32 chains per group (the equations of a VAR, the lambdas
-// of a cold start), p <= 512: the whole ADMM of a group in one launch, x-updates on the
+// of a cold start), 64 < p <= 512: the whole ADMM of a group in one launch, x-updates on the
 // tensor cores with the chains as the products' rows.
 //
 //   x = c + rho M V,  v = x + u,  u' = clamp(v, +-kappa),  z' = v - u',  V' = z' - u'
@@ -32,10 +32,18 @@
 // p = 384 12.0k, at 500 14.2k, where the products (72 clocks each) lead.  One launch per
 // step spent 88k clocks per iteration at p = 384, half of them between launches.
 // Measured, ADMM stage of a fit (before: the CUDA-core kernel with M in shared memory for
-// p <= 192, else k_xupdate_tc once per iteration): VAR p = 192, 30 x 32 46.4 -> 17.8 ms;
-// VAR(2) p = 192 (384 regressors), 20 x 16 174 -> 37 ms; VAR p = 500, 8 x 16 174 -> 71 ms.
-// Iterates are as far from the FP64 form's as before (6e-6 after 20 iterations at every p,
-// set by the moments).
+// p <= 192, else k_xupdate_tc once per iteration): VAR p = 192, 30 x 32 46.4 -> 18.7 ms;
+// VAR(2) p = 192 (384 regressors), 20 x 16 174 -> 37 ms; VAR p = 500, 8 x 16 174 -> 72 ms.
+//
+// Precision up to p = 192, where the CUDA-core kernel multiplied in FP32: the tensor cores cut
+// off their sums and two fp16 pieces hold 23 bits, and with all of M in the products z was
+// 1.1 to 1.7 times as far from FP64 iterates on the same M and c.  M's diagonal, most of a row's
+// sum, is therefore left out of the pieces and multiplied in FP32 by the update (FINE): 0.35 to
+// 0.6 times as far (p = 65..192, 40 iterations), for 5 % of a VAR p = 192.  Above, the form that
+// was replaced had the same pieces.
+// At p <= 64 one warp per chain (k_admm_resident) is as quick or quicker: ADMM call of 20 groups,
+// r = p, 16 lambdas, here and there: p = 16 1.09 and 0.59 ms, 40 1.21 and 0.85, 64 1.34 and 1.13,
+// 72 1.49 and 1.44, 96 1.59 and 1.93; cold starts of 384 chains 0.40 and 0.42 at p = 40.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -54,6 +62,7 @@ constexpr int WD_EPI = 256;                    // threads of the epilogue
 constexpr int WD_BLOCK = WD_CHAINS * 64;       // one piece of a V block (128 chains x 32 k)
 constexpr int WD_KB_MAX = 16;                  // k blocks (p <= 512)
 constexpr int WD_CS_MAX = 8;
+constexpr int WD_MIN_P = 64;                   // up to here one warp per chain is quicker
 constexpr int WD_KAPPA = 256;                  // thresholds kept in shared memory
 constexpr int WD_SCALE_EXP = 10;               // scaled magnitudes stay below 2^10
 
@@ -64,6 +73,7 @@ struct WideArgs {
     const float* c;                 // G x r x p
     const float* cn;                // G x r: norms of c
     const float* row_inv;           // G x (cs F): 1 / scale of the row of M
+    const float* diag;              // G x (cs F): M's diagonal (FINE)
     const double* lambdas;
     __half* v;                      // clusters x 2 x kb x 2 pieces x 128 x 32, zero
     float* norms;                   // clusters x 2 x (2 cs) x 5 x 128
@@ -131,9 +141,10 @@ __device__ __forceinline__ void wd_store32(void* p, const uint32_t (&v)[8])
                  : "memory");
 }
 
-// NQ accumulators of h.H (one per 128 k), added with their rounding errors when COMP.
+// NQ accumulators of h.H (one per 128 k), added with their rounding errors when COMP.  FINE: M's
+// diagonal is not in the products; the update multiplies it in FP32.
 // TMEM columns: h.H [NQ][F], small products [F], v [F], c [F].
-template <int NQ, bool COMP>
+template <int NQ, bool COMP, bool FINE>
 __global__ void __launch_bounds__(WD_THREADS, 1)
 k_admm_wide(const __grid_constant__ CUtensorMap tmM, WideArgs a)
 {
@@ -141,7 +152,7 @@ k_admm_wide(const __grid_constant__ CUtensorMap tmM, WideArgs a)
     __shared__ uint64_t vfull[WD_KB_MAX], vempty[WD_KB_MAX], mfull, accf, cbar;
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag, s_stop, s_any[2];
-    __shared__ __align__(16) float s_rinv[128];
+    __shared__ __align__(16) float s_rinv[128], s_diag[FINE ? 128 : 4];
     __shared__ float s_kappa[WD_KAPPA];
     __shared__ float s_kst[WD_CHAINS], s_kc[WD_CHAINS], s_vrinv[WD_CHAINS], s_vw[WD_CHAINS];
     __shared__ int s_cid[WD_CHAINS];
@@ -172,6 +183,8 @@ k_admm_wide(const __grid_constant__ CUtensorMap tmM, WideArgs a)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     for (int i = threadIdx.x; i < F; i += blockDim.x) s_rinv[i] = a.row_inv[(int64_t)g * cs * F + rank * F + i];
+    if constexpr (FINE)
+        for (int i = threadIdx.x; i < F; i += blockDim.x) s_diag[i] = a.diag[(int64_t)g * cs * F + rank * F + i];
     for (int i = threadIdx.x; i < min(a.q, WD_KAPPA); i += blockDim.x) s_kappa[i] = (float)a.lambdas[i] / a.rho;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
@@ -446,10 +459,11 @@ k_admm_wide(const __grid_constant__ CUtensorMap tmM, WideArgs a)
                                 }
                                 hh = s;
                             }
-                            const float prod = (hh + lo) * (s_rinv[f0 + f + kk] * vi);
-                            const float x = __uint_as_float(rr[NQ + 2][kk]) + a.rho * prod;
                             const float vo = __uint_as_float(rr[NQ + 1][kk]);
                             const float uo = wd_clamp(vo, ks), zp = vo - uo;
+                            float prod = (hh + lo) * (s_rinv[f0 + f + kk] * vi);
+                            if constexpr (FINE) prod = fmaf(s_diag[f0 + f + kk], zp - uo, prod);
+                            const float x = __uint_as_float(rr[NQ + 2][kk]) + a.rho * prod;
                             const float v = x + uo, un = wd_clamp(v, kn), zn = v - un;
                             nv[kk] = v;
                             const float d = x - zn, dz = zn - zp;
@@ -520,8 +534,9 @@ k_admm_wide(const __grid_constant__ CUtensorMap tmM, WideArgs a)
 }
 
 // M_g -> per-row scales and fp16 pieces in blocks [g][rank][k block][piece][F][32] (zero
-// padded), one warp per row; the arithmetic is k_scale_split_m's (xupdate_tc.cu).
-__global__ void k_wide_split_m(const float* M, int32_t G, int p, int cs, int F, int kb, float* row_inv, __half* out)
+// padded), one warp per row; the arithmetic is k_scale_split_m's (xupdate_tc.cu).  diag
+// (nullable): the diagonal goes there, and zero to the pieces.
+__global__ void k_wide_split_m(const float* M, int32_t G, int p, int cs, int F, int kb, float* row_inv, float* diag, __half* out)
 {
     const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31, ppad = cs * F;
@@ -535,6 +550,10 @@ __global__ void k_wide_split_m(const float* M, int32_t G, int p, int cs, int F, 
     for (int b = 0; b < WD_KB_MAX; ++b) {
         const int k = 32 * b + lane;
         v[b] = real && k < p ? mr[k] : 0.f;
+        if (diag && k == i) {
+            diag[row] = v[b];
+            v[b] = 0.f;
+        }
         mx = fmaxf(mx, fabsf(v[b]));
     }
 #pragma unroll
@@ -580,13 +599,13 @@ CUtensorMap wide_map(void* base, int64_t nblocks, int F)
 }
 
 using WideKernel = void (*)(CUtensorMap, WideArgs);
-// Sums of several accumulators keep their rounding errors past p = 192 (where the sums
-// that this form replaces did).
+// Up to p = WD_FINE_P this form replaces FP32 multiply-adds (k_admm_resident).
+constexpr int WD_FINE_P = 192;
 WideKernel wide_kernel(int nq, int p)
 {
-    if (nq == 1) return k_admm_wide<1, false>;
-    if (nq == 2) return p <= 192 ? k_admm_wide<2, false> : k_admm_wide<2, true>;
-    return nq == 3 ? k_admm_wide<3, true> : k_admm_wide<4, true>;
+    if (nq == 1) return k_admm_wide<1, false, true>;
+    if (nq == 2) return p <= WD_FINE_P ? k_admm_wide<2, false, true> : k_admm_wide<2, true, false>;
+    return nq == 3 ? k_admm_wide<3, true, false> : k_admm_wide<4, true, false>;
 }
 
 struct WideShape {
@@ -619,7 +638,7 @@ bool wide_shape(int p, int F, WideShape& s)
 bool admm_solve_wide(const AdmmProblem<float>& P, cudaStream_t s)
 {
     const int64_t nchains = P.warm ? P.r : P.r * P.q;
-    if (P.p > 32 * WD_KB_MAX || P.z0 || P.u_out || nchains > (1 << 30) || !gram_tc_available()) return false;
+    if (P.p <= WD_MIN_P || P.p > 32 * WD_KB_MAX || P.z0 || P.u_out || nchains > (1 << 30) || !gram_tc_available()) return false;
     // Fewest CTAs per chain tile while the tiles fill the device; with fewer tiles, more
     // CTAs each (their epilogues and products shrink with F)
     const int p = (int)P.p;
@@ -632,6 +651,7 @@ bool admm_solve_wide(const AdmmProblem<float>& P, cudaStream_t s)
     }
     if (!best.F) return false;
     const int ppad = best.cs * best.F;
+    const bool fine = p <= WD_FINE_P;
     const WideKernel kern = wide_kernel(best.nq, p);
     allow_max_dynamic_smem((const void*)kern);
     cudaLaunchConfig_t cfg = {};
@@ -650,15 +670,16 @@ bool admm_solve_wide(const AdmmProblem<float>& P, cudaStream_t s)
     UOI_CUDA(cudaOccupancyMaxActiveClusters(&resident, kern, &cfg));
     if (resident < 1) return false;
     const int per = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(nchains, WD_CHAINS), resident / P.G));
-    DevBuf mp(sizeof(__half) * 2 * (size_t)P.G * ppad * ppad, s), rinv(sizeof(float) * (size_t)P.G * ppad, s);
+    DevBuf mp(sizeof(__half) * 2 * (size_t)P.G * ppad * ppad, s), rinv(sizeof(float) * (size_t)P.G * ppad * 2, s);
     DevBuf cn(sizeof(float) * (size_t)P.G * P.r, s);
     DevBuf vb((size_t)P.G * per * 2 * best.kb * 2 * WD_BLOCK, s);
     UOI_CUDA(cudaMemsetAsync(vb.ptr, 0, vb.bytes, s));
     DevBuf nrm(sizeof(float) * (size_t)P.G * per * 2 * 2 * best.cs * 5 * WD_CHAINS, s);
     DevBuf next(sizeof(int32_t) * (size_t)(P.G + 1), s);
     UOI_CUDA(cudaMemsetAsync(next.ptr, 0, next.bytes, s));
+    float* diag = rinv.as<float>() + (size_t)P.G * ppad;
     k_wide_split_m<<<(unsigned)ceil_div((int64_t)P.G * ppad * 32, 256), 256, 0, s>>>(
-        P.M, P.G, p, best.cs, best.F, best.kb, rinv.as<float>(), mp.as<__half>());
+        P.M, P.G, p, best.cs, best.F, best.kb, rinv.as<float>(), fine ? diag : nullptr, mp.as<__half>());
     UOI_CHECK_LAUNCH();
     k_wide_c_norms<<<(unsigned)ceil_div((int64_t)P.G * P.r * 32, 256), 256, 0, s>>>(P.c, (int64_t)P.G * P.r, P.p,
                                                                                     cn.as<float>());
@@ -669,7 +690,7 @@ bool admm_solve_wide(const AdmmProblem<float>& P, cudaStream_t s)
     a.cs = best.cs; a.F = best.F; a.kb = best.kb; a.nslots = best.nslots; a.per = per;
     a.tmem_cols = best.tmem_cols;
     a.rho = (float)P.rho; a.abs_tol = (float)P.abs_tol; a.rel_tol = (float)P.rel_tol; a.sqrtp = (float)sqrt((double)p);
-    a.c = P.c; a.cn = cn.as<float>(); a.row_inv = rinv.as<float>(); a.lambdas = P.lambdas;
+    a.c = P.c; a.cn = cn.as<float>(); a.row_inv = rinv.as<float>(); a.diag = diag; a.lambdas = P.lambdas;
     a.v = vb.as<__half>(); a.norms = nrm.as<float>(); a.chain_next = next.as<int32_t>();
     a.beta = P.beta; a.iters = P.iters; a.conv = P.conv; a.family = P.family; a.near_count = P.near_count;
     a.err = next.as<int32_t>() + P.G;
