@@ -351,6 +351,11 @@ int uoi_selftest_index_check(int64_t index, int64_t extent, void* stream);
  * a full device (UOI_ERR_OOM where the call has no smaller way).  0 ends this. */
 int uoi_selftest_alloc_limit(uint64_t bytes);
 
+/* Test support (the paper has no counterpart): with on != 0, FP64 ADMM solves of
+ * the calling host thread take the schedule with one launch per iteration, which
+ * serves p of about 5000 and more, whatever their size; 0 ends this. */
+int uoi_selftest_admm_streaming(int32_t on);
+
 /* Text of a status code (static storage). */
 const char* uoi_status_string(int status);
 

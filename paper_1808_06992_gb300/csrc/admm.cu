@@ -1414,36 +1414,21 @@ bool try_resident<float>(const AdmmDev<float>& d, int32_t* chain_next, cudaStrea
 
 }  // namespace
 
-template <typename T>
-void admm_solve(const AdmmProblem<T>& P, cudaStream_t s)
+thread_local bool g_admm_streaming = false;
+
+namespace {
+
+// One launch per iteration and one to check it (FP64 past the chain schedule's shared memory, p of
+// about 5000 and more).
+void solve_streaming(const AdmmProblem<double>& P, const AdmmDev<double>& d, int32_t nchains, cudaStream_t s)
 {
-    if (P.G <= 0 || P.p <= 0 || P.r <= 0 || P.q <= 0) return;
-    AdmmDev<T> d = to_dev(P);
-    const int32_t nchains = P.warm ? (int32_t)P.r : (int32_t)(P.r * P.q);
-    if constexpr (sizeof(T) == 4)
-        if (nchains > 4 && admm_solve_wide(P, s)) return;
-    {
-        // chain counters and (FP64) row-sum bounds, zero, then the exponents of a streamed M
-        DevBuf next(sizeof(int32_t) * (size_t)P.G * (2 + (sizeof(T) == 8 ? (size_t)P.p : 0)), s);
-        UOI_CUDA(cudaMemsetAsync(next.ptr, 0, sizeof(int32_t) * 2 * (size_t)P.G, s));
-        if (try_resident<T>(d, next.as<int32_t>(), s)) return;
-    }
-    if constexpr (sizeof(T) == 4) {
-        if (admm_tc_available()) {               // FP32 state: x-update on the tensor cores
-            const AdmmProblem<float>& Pf = reinterpret_cast<const AdmmProblem<float>&>(P);
-            if (admm_batch_try_join(Pf, s)) return;   // solved with the rest of a batch
-            admm_solve_tc(Pf, s);
-            return;
-        }
-    }
-    // streaming schedule
     const int64_t slots = (int64_t)P.G * nchains;
     const int p = (int)P.p;
     const bool gemv = nchains <= 4;
     const int RT = gemv ? (int)ceil_div(p, GV_ROWS) : (int)ceil_div(p, SG_TM);
-    DevBuf zb(sizeof(T) * slots * p, s), ub(sizeof(T) * slots * p, s);
-    DevBuf v0(sizeof(T) * slots * p, s), v1(sizeof(T) * slots * p, s);
-    DevBuf nb(sizeof(T) * slots * RT * 5, s);
+    DevBuf zb(sizeof(double) * slots * p, s), ub(sizeof(double) * slots * p, s);
+    DevBuf v0(sizeof(double) * slots * p, s), v1(sizeof(double) * slots * p, s);
+    DevBuf nb(sizeof(double) * slots * RT * 5, s);
     DevBuf sj(sizeof(int32_t) * slots, s), sje(sizeof(int32_t) * slots, s), sit(sizeof(int32_t) * slots, s);
     DevBuf a0(sizeof(int32_t) * slots, s), a1(sizeof(int32_t) * slots, s);
     DevBuf c0(sizeof(int32_t) * P.G, s), c1(sizeof(int32_t) * P.G, s);
@@ -1458,12 +1443,12 @@ void admm_solve(const AdmmProblem<T>& P, cudaStream_t s)
     S.cnt[0] = c0.as<int32_t>(); S.cnt[1] = c1.as<int32_t>();
     S.total[0] = tot.as<int32_t>(); S.total[1] = tot.as<int32_t>() + 1;
     S.nchains = nchains;
-    k_stream_init<T><<<(unsigned)std::min<int64_t>(ceil_div(slots, 256), 4096), 256, 0, s>>>(d, S);
+    k_stream_init<double><<<(unsigned)std::min<int64_t>(ceil_div(slots, 256), 4096), 256, 0, s>>>(d, S);
     UOI_CHECK_LAUNCH();
     count_launch();
     if (P.z0 && !P.warm) {
-        k_stream_init_state<T><<<(unsigned)std::min<int64_t>(ceil_div(slots * p, 256), 8192), 256, 0, s>>>(
-            d, slots * p, zb.as<T>(), ub.as<T>(), v0.as<T>());
+        k_stream_init_state<double><<<(unsigned)std::min<int64_t>(ceil_div(slots * p, 256), 8192), 256, 0, s>>>(
+            d, slots * p, zb.as<double>(), ub.as<double>(), v0.as<double>());
         UOI_CHECK_LAUNCH();
         count_launch();
     }
@@ -1471,40 +1456,62 @@ void admm_solve(const AdmmProblem<T>& P, cudaStream_t s)
     int32_t* host_total = pinned_scratch_i32();
     const int64_t bound = (int64_t)(P.warm ? P.q : 1) * P.max_iter + 2;
     const int check_every = 8;
-    T* V[2] = { v0.as<T>(), v1.as<T>() };
+    double* V[2] = { v0.as<double>(), v1.as<double>() };
     int cur = 0;
     bool done = false;
-    try {
-        for (int64_t it = 0; it < bound && !done; ++it) {
-            if (gemv) {
-                dim3 grid((unsigned)RT, (unsigned)P.G);
-                k_stream_gemv<T, 4><<<grid, 256, 0, s>>>(d, S, cur, V[cur], V[cur ^ 1], zb.as<T>(),
-                                                          ub.as<T>(), nb.as<T>(), RT);
-            } else {
-                dim3 grid((unsigned)RT, (unsigned)ceil_div(nchains, SG_TN), (unsigned)P.G);
-                ktimer_begin(TK_XUPDATE, s);
-                k_stream_gemm<T><<<grid, 256, 0, s>>>(d, S, cur, V[cur], V[cur ^ 1], zb.as<T>(),
-                                                      ub.as<T>(), nb.as<T>(), RT);
-                ktimer_end(TK_XUPDATE, s, 0.0, 0.0);
-            }
-            UOI_CHECK_LAUNCH();
-            dim3 gc((unsigned)ceil_div(nchains, 8), (unsigned)P.G);
-            k_stream_check<T><<<gc, 256, 0, s>>>(d, S, cur, zb.as<T>(), ub.as<T>(), V[cur ^ 1],
-                                                  nb.as<T>(), RT);
-            UOI_CHECK_LAUNCH();
-            count_launch(2);
-            cur ^= 1;
-            if ((it + 1) % check_every == 0 || it + 1 == bound) {
-                UOI_CUDA(cudaMemcpyAsync(host_total, S.total[cur], sizeof(int32_t),
-                                         cudaMemcpyDeviceToHost, s));
-                UOI_CUDA(cudaStreamSynchronize(s));
-                done = *host_total == 0;
-            }
+    for (int64_t it = 0; it < bound && !done; ++it) {
+        if (gemv) {
+            dim3 grid((unsigned)RT, (unsigned)P.G);
+            k_stream_gemv<double, 4><<<grid, 256, 0, s>>>(d, S, cur, V[cur], V[cur ^ 1], zb.as<double>(),
+                                                      ub.as<double>(), nb.as<double>(), RT);
+        } else {
+            dim3 grid((unsigned)RT, (unsigned)ceil_div(nchains, SG_TN), (unsigned)P.G);
+            ktimer_begin(TK_XUPDATE, s);
+            k_stream_gemm<double><<<grid, 256, 0, s>>>(d, S, cur, V[cur], V[cur ^ 1], zb.as<double>(),
+                                                  ub.as<double>(), nb.as<double>(), RT);
+            ktimer_end(TK_XUPDATE, s, 0.0, 0.0);
         }
-    } catch (...) {
-        throw;
+        UOI_CHECK_LAUNCH();
+        dim3 gc((unsigned)ceil_div(nchains, 8), (unsigned)P.G);
+        k_stream_check<double><<<gc, 256, 0, s>>>(d, S, cur, zb.as<double>(), ub.as<double>(), V[cur ^ 1],
+                                              nb.as<double>(), RT);
+        UOI_CHECK_LAUNCH();
+        count_launch(2);
+        cur ^= 1;
+        if ((it + 1) % check_every == 0 || it + 1 == bound) {
+            UOI_CUDA(cudaMemcpyAsync(host_total, S.total[cur], sizeof(int32_t),
+                                     cudaMemcpyDeviceToHost, s));
+            UOI_CUDA(cudaStreamSynchronize(s));
+            done = *host_total == 0;
+        }
     }
     if (!done) throw Error(UOI_ERR_TIMEOUT, "ADMM streaming loop exceeded its iteration bound");
+}
+
+}  // namespace
+
+template <typename T>
+void admm_solve(const AdmmProblem<T>& P, cudaStream_t s)
+{
+    if (P.G <= 0 || P.p <= 0 || P.r <= 0 || P.q <= 0) return;
+    AdmmDev<T> d = to_dev(P);
+    const int32_t nchains = P.warm ? (int32_t)P.r : (int32_t)(P.r * P.q);
+    if constexpr (sizeof(T) == 4)
+        if (nchains > 4 && admm_solve_wide(P, s)) return;
+    if (sizeof(T) == 4 || !g_admm_streaming) {
+        // chain counters and (FP64) row-sum bounds, zero, then the exponents of a streamed M
+        DevBuf next(sizeof(int32_t) * (size_t)P.G * (2 + (sizeof(T) == 8 ? (size_t)P.p : 0)), s);
+        UOI_CUDA(cudaMemsetAsync(next.ptr, 0, sizeof(int32_t) * 2 * (size_t)P.G, s));
+        if (try_resident<T>(d, next.as<int32_t>(), s)) return;
+    }
+    if constexpr (sizeof(T) == 4) {
+        // FP32 state: x-update on the tensor cores
+        if (!admm_tc_available()) throw Error(UOI_ERR_UNSUPPORTED, "the mixed form's ADMM needs sm_103a tensor cores");
+        if (admm_batch_try_join(P, s)) return;   // solved with the rest of a batch
+        admm_solve_tc(P, s);
+    } else {
+        solve_streaming(P, d, nchains, s);
+    }
 }
 
 template void admm_solve<double>(const AdmmProblem<double>&, cudaStream_t);

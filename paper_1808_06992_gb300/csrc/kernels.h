@@ -233,6 +233,8 @@ struct AdmmProblem {
 constexpr double kNearThreshold = 1e-6;
 template <typename T>
 void admm_solve(const AdmmProblem<T>& P, cudaStream_t s);
+// For tests, per host thread: FP64 solves take the streaming schedule whatever their size.
+extern thread_local bool g_admm_streaming;
 // Streaming schedule with the tensor-core x-update (FP32 state, p > resident limit).
 bool admm_tc_available();
 void admm_solve_tc(const AdmmProblem<float>& P, cudaStream_t s);

@@ -11,7 +11,9 @@
 // with arrive = 1 the thread arrives first, so the wait must succeed at once.
 //
 // uoi_selftest_alloc_limit makes device allocations of the calling thread above a size fail
-// as they do on a full device, so that what a call does then can be seen without filling one.
+// as they do on a full device, so that what a call does then can be seen without filling one;
+// uoi_selftest_admm_streaming has its FP64 solves take the schedule that is otherwise reached
+// from p of about 5000 on.
 #include <cuda_runtime.h>
 
 #include "kernels.h"
@@ -56,6 +58,12 @@ namespace uoi { extern thread_local uint64_t g_alloc_limit; }
 extern "C" int uoi_selftest_alloc_limit(uint64_t bytes)
 {
     g_alloc_limit = bytes;
+    return UOI_OK;
+}
+
+extern "C" int uoi_selftest_admm_streaming(int32_t on)
+{
+    g_admm_streaming = on != 0;
     return UOI_OK;
 }
 

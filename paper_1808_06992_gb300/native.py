@@ -139,6 +139,7 @@ def _configure(L):
         L.uoi_selftest_wait.argtypes = [C.c_uint64, i32, C.POINTER(d), vp]
         L.uoi_selftest_index_check.argtypes = [i64, i64, vp]
         L.uoi_selftest_alloc_limit.argtypes = [C.c_uint64]
+        L.uoi_selftest_admm_streaming.argtypes = [i32]
         L.uoi_status_string.argtypes = [C.c_int]
         L.uoi_status_string.restype = C.c_char_p
         L.uoi_get_last_error_detail.argtypes = [C.c_char_p, C.c_size_t]
@@ -150,7 +151,7 @@ EXPORTED = ("uoi_params_default", "uoi_lasso_fit", "uoi_lasso_fit_batch", "uoi_v
             "lasso_admm_batch", "lasso_admm_batch_noalloc", "uoi_weighted_moments",
             "uoi_ws_param_count", "uoi_ws_create", "uoi_ws_load", "uoi_ws_save", "uoi_ws_free",
             "uoi_ws_set_params", "uoi_ws_get_params", "uoi_ws_forward", "uoi_ws_loss_grad",
-            "uoi_ws_train", "uoi_ws_dataset", "uoi_selftest_wait", "uoi_selftest_index_check", "uoi_selftest_alloc_limit", "uoi_status_string", "uoi_get_last_error_detail",
+            "uoi_ws_train", "uoi_ws_dataset", "uoi_selftest_wait", "uoi_selftest_index_check", "uoi_selftest_alloc_limit", "uoi_selftest_admm_streaming", "uoi_status_string", "uoi_get_last_error_detail",
             "uoi_shutdown")
 
 
@@ -510,6 +511,11 @@ def selftest_index_check(index, extent, stream=None):
 def selftest_alloc_limit(nbytes):
     """Device allocations of this thread above nbytes fail (see uoi_selftest_alloc_limit); 0: none do."""
     return _check(lib().uoi_selftest_alloc_limit(int(nbytes)))
+
+
+def selftest_admm_streaming(on):
+    """This thread's FP64 solves take the large-p schedule (see uoi_selftest_admm_streaming)."""
+    return _check(lib().uoi_selftest_admm_streaming(1 if on else 0))
 
 
 def shutdown():
