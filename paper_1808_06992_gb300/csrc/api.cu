@@ -1273,6 +1273,7 @@ void uoi_shutdown(void)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return;
     cudaDeviceSynchronize();
+    uoi::release_side_streams(dev);
     cudaMemPool_t pool;
     if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
 }

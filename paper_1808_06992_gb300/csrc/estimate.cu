@@ -15,6 +15,7 @@
 // x_0 = 0, whose iterates stay in the range of G and converge to the
 // minimum-norm least-squares solution; they are flagged.
 #include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "fixed_dot.cuh"
@@ -1372,24 +1373,59 @@ __global__ void __launch_bounds__(UNION_WORDS) k_union_cols(const uint64_t* fam,
 
 // A second stream per host thread and device, for work that runs beside the thread's main
 // stream (the smaller classes of the loss pass, half of the batch of the tensor-core
-// inverse, sums of the warm-start gradient); made on first use, given back when the thread ends.
+// inverse, sums of the warm-start gradient).  A thread takes one on first use and hands it on
+// when it ends (idle: every user waits for it), so there are as many as threads were at work at
+// once; uoi_shutdown destroys those no thread holds.  Destroying them with each batch's workers
+// cost 2 to 4 % of a batch of 24.
+namespace {
+struct SidePool {
+    std::mutex mu;
+    std::vector<std::vector<cudaStream_t>> idle;             // by device
+};
+SidePool& side_pool()
+{
+    static SidePool* pool = new SidePool;                    // outlives the threads that hand streams back
+    return *pool;
+}
+struct SideStreams {
+    std::vector<cudaStream_t> of;                            // by device
+    ~SideStreams()
+    {
+        SidePool& p = side_pool();
+        std::lock_guard<std::mutex> lock(p.mu);
+        if (p.idle.size() < of.size()) p.idle.resize(of.size());
+        for (size_t d = 0; d < of.size(); ++d)
+            if (of[d]) p.idle[d].push_back(of[d]);
+    }
+};
+}  // namespace
+
 cudaStream_t side_stream()
 {
-    struct Streams {
-        std::vector<cudaStream_t> of;                        // by device
-        ~Streams()
-        {
-            for (cudaStream_t q : of)
-                if (q) cudaStreamDestroy(q);
-        }
-    };
-    thread_local Streams streams;
+    thread_local SideStreams mine;
     int dev = 0;
     UOI_CUDA(cudaGetDevice(&dev));
-    if ((size_t)dev >= streams.of.size()) streams.of.resize((size_t)dev + 1, nullptr);
-    cudaStream_t& q = streams.of[(size_t)dev];
+    if ((size_t)dev >= mine.of.size()) mine.of.resize((size_t)dev + 1, nullptr);
+    cudaStream_t& q = mine.of[(size_t)dev];
+    if (!q) {
+        SidePool& p = side_pool();
+        std::lock_guard<std::mutex> lock(p.mu);
+        if ((size_t)dev < p.idle.size() && !p.idle[(size_t)dev].empty()) {
+            q = p.idle[(size_t)dev].back();
+            p.idle[(size_t)dev].pop_back();
+        }
+    }
     if (!q) UOI_CUDA(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
     return q;
+}
+
+void release_side_streams(int dev)
+{
+    SidePool& p = side_pool();
+    std::lock_guard<std::mutex> lock(p.mu);
+    if ((size_t)dev >= p.idle.size()) return;
+    for (cudaStream_t q : p.idle[(size_t)dev]) cudaStreamDestroy(q);
+    p.idle[(size_t)dev].clear();
 }
 
 int32_t union_columns(const uint64_t* family, int64_t count, int64_t p, int32_t* cols,

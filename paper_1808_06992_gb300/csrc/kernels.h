@@ -183,6 +183,7 @@ void spd_inverse_tc(const float* A, int64_t p, int32_t G, float* M, DevStatus* s
                     int32_t* bad = nullptr);   // bad[k] = 1 where a pivot was not positive (zero before)
 // The calling host thread's second stream on the current device (estimate.cu).
 cudaStream_t side_stream();
+void release_side_streams(int dev);     // those that ended threads have handed back
 // M_k = (G_k/n_k + rho I)^{-1} in FP64 accuracy by Newton's iteration from the FP32 inverse
 // (inverse_f64.cu); A: B x p x p scratch.  Per system, 1 if it is done and 0 (nothing usable in
 // M_k) where the size is not its own or the iteration does not settle: the caller then takes the

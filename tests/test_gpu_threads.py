@@ -31,5 +31,7 @@ def test_gradients_and_fits_from_short_lived_threads():
         t.start()
         t.join()
     assert len(got) == 12
+    native.lib().uoi_shutdown()                          # the ended threads' stream goes; calls go on
+    call()
     for (loss, grad), beta in got:
         assert loss == want[0] and np.array_equal(grad, want[1]) and torch.equal(beta, fit)
