@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(256, 1) k_admm_resident(AdmmDev<T> P, int32_t*
 // at 64 clocks, two block barriers, the exchange); past L2 the stream of M.
 // Measured (one call; one warp per chain or two launches per iteration, then this schedule
 // with FP64 products, then as it is): 200 x 50, 20 chains, 598 iterations each: 12.7, 2.3,
-// 1.65 ms; p = 400, 20 chains: 38, 6.9, 3.8 ms; p = 1000 (M 160 MB): 124, 52, 14 ms
+// 1.6 ms; p = 400, 20 chains: 38, 6.9, 3.8 ms; p = 1000 (M 160 MB): 124, 52, 13.5 ms
 // (26 ms with 8 and 3 blocks per pass instead of 6 and 5: a pass of few blocks has few
 // loads in flight);
 // p = 150, 128 chains: 110, 5.1, 3.0 ms.

@@ -26,10 +26,10 @@
 // ends is replaced by the group's next one; its first product is masked (V = 0).
 // Every wait is bounded (one second) and reports UOI_ERR_TIMEOUT.
 //
-// What bounds it: the length of one iteration, 9.6k clocks at p = 192 (2 CTAs of 96
+// What bounds it: the length of one iteration, 10.5k clocks at p = 192 (2 CTAs of 96
 // features): V's first block 1.0k after cbar, six blocks of products 2.3k, the update
-// 3.4k (about 27 instructions per element on 8 warps), the fences around cbar 1.7k; at
-// p = 384 12.0k, at 500 14.2k, where the products (72 clocks each) lead.  One launch per
+// 4k (about 29 instructions per element on 8 warps), the fences around cbar 1.7k; at
+// p = 384 12.5k, at 500 14.6k, where the products (72 clocks each) lead.  One launch per
 // step spent 88k clocks per iteration at p = 384, half of them between launches.
 // Measured, ADMM stage of a fit (before: the CUDA-core kernel with M in shared memory for
 // p <= 192, else k_xupdate_tc once per iteration): VAR p = 192, 30 x 32 46.4 -> 18.7 ms;

@@ -15,8 +15,8 @@
 // Why: this part's FP64 pipe takes 19 clocks per warp multiply-add, and factor, triangular
 // inverse and product need p^3 / 2 of them per system; here FP64 work is p^2 per step.
 // Measured, 20 systems, factor stage against Cholesky, triangular inverse and product in FP64:
-// p = 1000 33.3 -> 9.2 ms (residuals 4, FP32 products 2.8, FP32 inverse 1.5), 600 10.9 -> 3.3,
-// 400 4.9 -> 1.65, 150 1.26 -> 0.45, 65 0.40 -> 0.30; below 64 columns the
+// p = 1000 33.3 -> 9.0 ms (residuals 4, FP32 products 2.8, FP32 inverse 1.5), 600 10.9 -> 3.15,
+// 400 4.9 -> 1.6, 150 1.26 -> 0.43, 65 0.40 -> 0.30; below 64 columns the
 // factor's 0.35 ms are not beaten.  |M b| against 80-bit arithmetic: the factor's error or
 // less (tests/test_gpu_inverse_newton.py).
 #include <algorithm>

@@ -239,12 +239,12 @@ extern thread_local bool g_admm_streaming;
 // Streaming schedule with the tensor-core x-update (FP32 state, p > resident limit).
 bool admm_tc_available();
 void admm_solve_tc(const AdmmProblem<float>& P, cudaStream_t s);
-// The whole solve in one launch for many chains and p <= 512 (admm_wide.cu); false
+// The whole solve in one launch for many chains and 64 < p <= 512 (admm_wide.cu); false
 // (nothing launched) where it does not apply.
 bool admm_solve_wide(const AdmmProblem<float>& P, cudaStream_t s);
 // Grouped solve of a batch of problems.  Each batch worker thread enters the batch
 // before a fit and leaves it after; the fit's first tensor-core ADMM solve
-// (admm_solve<float> past the resident schedule) joins the batch instead of
+// (admm_solve<float> past the one-launch schedules) joins the batch instead of
 // running alone: its state is prepared on the worker's stream, a solver thread
 // iterates it together with the other members (grouped launches replayed as CUDA
 // graphs, tiles chosen by timing) and releases the worker once its columns have
